@@ -809,6 +809,7 @@ void cd_tree_free(cd_tree t)
 {
     if (!t) return;
     cudaDeviceSynchronize();
+    scratch_trim();
     free_workspace(t);
     free_side_streams(t);
     free_host_io(t);

@@ -299,6 +299,12 @@ bool stats_timing();
 // buffer it may reference has been freed or reallocated.
 cudaError_t lib_free(void *p);
 int64_t free_generation();
+// stats.cu: stream-ordered scratch of one call (cudaMallocFromPoolAsync on a
+// library-owned pool of the current device that keeps at most 64 MiB between
+// calls; scratch_trim gives that back, called by cd_tree_free)
+cudaError_t scratch_alloc(void **p, size_t bytes, cudaStream_t s);
+void scratch_free(void *p, cudaStream_t s);
+void scratch_trim();
 // launch counters and flops by kind (CD_K_COUNT entries): a copy, and adding
 // sign x counts (a graph replay adds what its capture recorded)
 void stats_snapshot(int64_t *count, double *flops);

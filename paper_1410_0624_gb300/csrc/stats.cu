@@ -69,6 +69,51 @@ cudaError_t lib_free(void *p)
 
 int64_t free_generation() { return g_free_gen.load(); }
 
+static std::mutex g_scratch_mu;
+static cudaMemPool_t g_scratch[64];
+
+cudaError_t scratch_alloc(void **p, size_t bytes, cudaStream_t s)
+{
+    *p = nullptr;
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+    cudaMemPool_t pool;
+    {
+        std::lock_guard<std::mutex> lk(g_scratch_mu);
+        if (!g_scratch[dev]) {
+            cudaMemPoolProps props = {};
+            props.allocType = cudaMemAllocationTypePinned;
+            props.location.type = cudaMemLocationTypeDevice;
+            props.location.id = dev;
+            uint64_t keep = (uint64_t)64 << 20;
+            e = cudaMemPoolCreate(&g_scratch[dev], &props);
+            if (e == cudaSuccess) e = cudaMemPoolSetAttribute(g_scratch[dev], cudaMemPoolAttrReleaseThreshold, &keep);
+            if (e != cudaSuccess) {
+                cudaGetLastError();
+                if (g_scratch[dev]) cudaMemPoolDestroy(g_scratch[dev]);
+                g_scratch[dev] = nullptr;
+                return e;
+            }
+        }
+        pool = g_scratch[dev];
+    }
+    e = cudaMallocFromPoolAsync(p, bytes, pool, s);
+    if (e != cudaSuccess) cudaGetLastError();
+    return e;
+}
+
+void scratch_free(void *p, cudaStream_t s) { cudaFreeAsync(p, s); }
+
+void scratch_trim()
+{
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return;
+    std::lock_guard<std::mutex> lk(g_scratch_mu);
+    if (g_scratch[dev]) cudaMemPoolTrimTo(g_scratch[dev], 0);
+}
+
 void stats_snapshot(int64_t *count, double *flops)
 {
     std::lock_guard<std::mutex> lk(g_mu);

@@ -1,0 +1,49 @@
+"""Kernel variants chosen by a rule on sizes, each at the edges of its range
+against the general path or the oracle."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_1410_0624_gb300 import colden, synth
+
+BOX = 10 * synth.PC_CM
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib():
+    colden.load(build_if_missing=True)
+
+
+def _rho(L, seed, sigma=1.5):
+    return synth.lognormal_iid(1 << L, 10.0, sigma, seed=seed)
+
+
+@pytest.mark.parametrize("L,n,dset", [(3, 400_000, ("axes", 0, 0)), (5, 70_001, ("mxn", 7, 5)),
+                                      (6, 33_000, ("healpix", 2, 0)), (7, 32_768, ("mxn", 3, 4))])
+def test_raymarch_in_spatial_order_is_row_by_row_the_same(L, n, dset):
+    # a list long enough to be marched in spatial order (repeated leaves and
+    # entries out of range among it) against short pieces of it, bit for bit
+    tree = colden.build_tree_uniform(torch.from_numpy(_rho(L, 7)).cuda(), BOX)
+    geom = colden.precompute_geometry(*dset)
+    rng = np.random.default_rng(n)
+    m = rng.integers(0, tree.n_leaf, n)
+    m[:: 9973] = -1
+    m[5:: 9973] = tree.n_leaf
+    lv = torch.from_numpy(m).cuda()
+    out = torch.full((n, geom.n_dir), -1.0, device="cuda")
+    colden.raymarch(tree, geom, out, leaves=lv)
+    ref = torch.full((n, geom.n_dir), -1.0, device="cuda")
+    for i in range(0, n, 8000):
+        piece = torch.empty((min(8000, n - i), geom.n_dir), device="cuda")
+        colden.raymarch(tree, geom, piece, leaves=lv[i:i + 8000].contiguous())
+        ref[i:i + 8000] = piece
+    assert torch.equal(out, ref)
+    bad = torch.from_numpy((m < 0) | (m >= tree.n_leaf)).cuda()
+    assert bool((out[bad] == 0).all()) and bool((out[~bad] > 0).all())
+    rows = np.flatnonzero((m >= 0) & (m < tree.n_leaf))[:: max(1, n // 200)]
+    ijk = oracle.morton_ijk(L)[m[rows]]
+    want = oracle.Tree.uniform(_rho(L, 7), BOX).raymarch(geom.dirs, np.full(len(rows), L), ijk)
+    got = out[torch.from_numpy(rows).cuda()].double().cpu().numpy()
+    assert np.max(np.abs(got - want) / want) < 2e-5   # the ray-marcher's tolerance
