@@ -492,6 +492,17 @@ cd_status check_net(cd_net net)
     return CD_OK;
 }
 
+cd_status check_batch(cd_net net, int64_t B, const float *x, const float *y)
+{
+    const cd_status st = check_net(net);
+    if (st != CD_OK) return st;
+    if (B < 1 || B > kChunkRows * 4 || !x || !y) {
+        set_error("batch size %lld outside 1 .. %lld or NULL data", (long long)B, (long long)kChunkRows * 4);
+        return CD_EINVAL;
+    }
+    return CD_OK;
+}
+
 }  // namespace
 
 // Computes (or reuses) every shell's sum kept apart: C[k] for k = 3 .. L-2 and
@@ -597,7 +608,7 @@ cd_status column_density_learned(cd_tree t, cd_geom g, const cd_opts &o, float *
     for (int64_t c0 = 0; c0 < t->n_leaf; c0 += chunk) {
         const int64_t cn = std::min(chunk, t->n_leaf - c0);
         if ((st = launch_features(t, g, cn, c0, nullptr, lv.x, lv.n_tree, s)) != CD_OK) return st;
-        if ((st = mlp_forward(net, cn, lv.x, nullptr, lv.delta, s)) != CD_OK) return st;
+        if ((st = mlp_forward(net, cn, lv.x, lv.delta, s)) != CD_OK) return st;
         LaunchScope ls(CD_K_FEATURES, s);
         learned_combine<<<grid_for(cn * 32, kThreads), kThreads, 0, s>>>(
             cn, nd, lv.n_tree, lv.delta, net->dlo, net->dhi, (float)o.av_per_nh, (float)o.shield_k, n_h ? n_h + c0 * nd : nullptr,
@@ -691,7 +702,7 @@ cd_status cd_net_create(int n_dir, int hidden, const float *params, cd_net *out)
     cudaGetDevice(&net->dev);
     const size_t P = (size_t)net->lay.total, I = (size_t)net->lay.n_in;
     bool ok = alloc(&net->p, P) == CD_OK && alloc(&net->m, P) == CD_OK && alloc(&net->v, P) == CD_OK &&
-              alloc(&net->grad, P) == CD_OK && alloc(&net->mu, I) == CD_OK && alloc(&net->sinv, I) == CD_OK;
+              alloc(&net->mu, I) == CD_OK && alloc(&net->sinv, I) == CD_OK;
     if (!ok) {
         cd_net_free(net);
         return CD_ENOMEM;
@@ -738,7 +749,7 @@ cd_status cd_net_forward(cd_net net, int64_t n, const float *x, float *delta, vo
     cudaStream_t s = (cudaStream_t)stream;
     for (int64_t c0 = 0; c0 < n; c0 += kChunkRows) {
         const int64_t cn = std::min<int64_t>(kChunkRows, n - c0);
-        if ((st = mlp_forward(net, cn, x + c0 * L.n_in, nullptr, delta + c0 * L.nd, s)) != CD_OK) return st;
+        if ((st = mlp_forward(net, cn, x + c0 * L.n_in, delta + c0 * L.nd, s)) != CD_OK) return st;
     }
     return CD_OK;
 }
@@ -747,27 +758,20 @@ cd_status cd_net_loss_grad(cd_net net, int64_t B, const float *x, const float *y
                            float *grad, void *stream)
 {
     NvtxRange nvtx_range("colden:net_loss_grad");
-    cd_status st = check_net(net);
+    const cd_status st = check_batch(net, B, x, y);
     if (st != CD_OK) return st;
-    if (B < 1 || B > kChunkRows * 4 || !x || !y) {
-        set_error("batch size %lld outside 1 .. %lld or NULL data", (long long)B, (long long)kChunkRows * 4);
-        return CD_EINVAL;
-    }
-    cudaStream_t s = (cudaStream_t)stream;
-    if ((st = mlp_loss_grad(net, B, x, y, rows, loss, s)) != CD_OK) return st;
-    if (grad) CD_CUDA(cudaMemcpyAsync(grad, net->grad, sizeof(float) * net->lay.total, cudaMemcpyDeviceToDevice, s));
-    return CD_OK;
+    return mlp_loss_grad(net, B, x, y, rows, loss, grad, (cudaStream_t)stream);
 }
 
 cd_status cd_net_train_step(cd_net net, int64_t B, const float *x, const float *y, const int64_t *rows,
                             const cd_adam *hp, float *loss, void *stream)
 {
     NvtxRange nvtx_range("colden:net_train_step");
-    cd_status st = cd_net_loss_grad(net, B, x, y, rows, loss, nullptr, stream);
+    const cd_status st = check_batch(net, B, x, y);
     if (st != CD_OK) return st;
     cd_adam h;
     if (hp) h = *hp; else cd_adam_default(&h);
-    return mlp_adam(net, h, (cudaStream_t)stream);
+    return mlp_train_step(net, B, x, y, rows, h, loss, (cudaStream_t)stream);
 }
 
 cd_status cd_net_get_state(cd_net net, float *params, float *mu, float *sinv, float *adam_m, float *adam_v,
@@ -881,7 +885,7 @@ void cd_net_free(cd_net net)
 {
     if (!net) return;
     cudaDeviceSynchronize();
-    for (float *p : {net->p, net->m, net->v, net->grad, net->mu, net->sinv, net->act.U, net->act.Z1, net->act.A1,
+    for (float *p : {net->p, net->m, net->v, net->mu, net->sinv, net->act.U, net->act.Z1, net->act.A1,
                      net->act.Z2, net->act.A2, net->act.D, net->act.G, net->act.part, net->act.red})
         if (p) cd::lib_free(p);
     net_free_tc(net);

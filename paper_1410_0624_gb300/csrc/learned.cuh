@@ -30,16 +30,17 @@ struct NetLayout {
     }
 };
 
-// Activations of one batch: row-major [cap][...].
+// Activations of one batch: row-major [rows][...].
 struct Activations {
-    int64_t cap = 0;
-    float *U = nullptr;     // standardised inputs [cap][n_in]
-    float *Z1 = nullptr, *A1 = nullptr, *Z2 = nullptr, *A2 = nullptr;   // [cap][H]
-    float *D = nullptr;     // delta, then d loss / d delta [cap][nd]
-    float *G = nullptr;     // d loss / d (A or Z) scratch [cap][H]
-    float *part = nullptr;  // split-K partial sums
+    float *U = nullptr;                   // standardised inputs [rows][n_in]
+    float *A1 = nullptr, *A2 = nullptr;   // [rows][H]
+    float *Z1 = nullptr, *Z2 = nullptr;   // training: pre-activations [rows][H] (Z1 becomes d loss / d z1)
+    float *G = nullptr;                   // training: d loss / d z2 [rows][H]
+    float *D = nullptr;                   // training: d loss / d delta [rows][nd]
+    size_t cap[7] = {};                   // floats of U, A1, A2, Z1, Z2, G, D
+    float *part = nullptr;  // partial gradients, one parameter vector per split of the batch
     size_t part_cap = 0;
-    float *red = nullptr;   // partial sums of the loss and the normaliser
+    float *red = nullptr;   // partial sums of the loss
     size_t red_cap = 0;
 };
 
@@ -51,7 +52,6 @@ struct cd_net_s {
     float *mu = nullptr;      // [n_in]
     float *sinv = nullptr;    // [n_in]
     float *m = nullptr, *v = nullptr;   // Adam moments
-    float *grad = nullptr;    // [total]
     int64_t step = 0;
     // trusted range of delta (cd_net_set_delta_range): outside it, or where
     // delta is not finite, the learned form returns the plain column
@@ -67,14 +67,14 @@ struct cd_net_s {
 namespace cd {
 
 // mlp.cu
-cd_status net_reserve(cd_net net, int64_t rows);
-// delta [B][nd] of rows `rows` (NULL: 0..B-1) of x; keeps the activations
-// (for a following backward) when keep != 0
-cd_status mlp_forward(cd_net net, int64_t B, const float *x, const int64_t *rows, float *delta, cudaStream_t s);
-// loss and gradient into net->grad; loss_out may be NULL
-cd_status mlp_loss_grad(cd_net net, int64_t B, const float *x, const float *y, const int64_t *rows,
-                        float *loss_out, cudaStream_t s);
-cd_status mlp_adam(cd_net net, const cd_adam &hp, cudaStream_t s);
+// delta [B][nd] of rows 0 .. B-1 of x
+cd_status mlp_forward(cd_net net, int64_t B, const float *x, float *delta, cudaStream_t s);
+// loss and gradient of the batch (rows NULL: rows 0 .. B-1); either output may be NULL
+cd_status mlp_loss_grad(cd_net net, int64_t B, const float *x, const float *y, const int64_t *rows, float *loss_out,
+                        float *grad, cudaStream_t s);
+// the same, followed by one Adam step
+cd_status mlp_train_step(cd_net net, int64_t B, const float *x, const float *y, const int64_t *rows, const cd_adam &hp,
+                         float *loss_out, cudaStream_t s);
 cd_status mlp_fit_normaliser(cd_net net, int64_t n, const float *x, cudaStream_t s);
 
 // mlp_tc.cu: the fused BF16 tensor-core inference

@@ -5,6 +5,7 @@ import pytest
 import torch
 
 import oracle
+from oracle import learned as ol
 from paper_1410_0624_gb300 import colden, synth
 
 BOX = 10 * synth.PC_CM
@@ -47,3 +48,34 @@ def test_raymarch_in_spatial_order_is_row_by_row_the_same(L, n, dset):
     want = oracle.Tree.uniform(_rho(L, 7), BOX).raymarch(geom.dirs, np.full(len(rows), L), ijk)
     got = out[torch.from_numpy(rows).cuda()].double().cpu().numpy()
     assert np.max(np.abs(got - want) / want) < 2e-5   # the ray-marcher's tolerance
+
+
+@pytest.mark.parametrize("nd,H,B", [(5, 16, 33), (3, 97, 130), (12, 64, 4931), (48, 128, 9729), (7, 50, 38913),
+                                    (13, 61, 38912), (12, 100, 39001)])
+def test_network_at_the_edges_of_its_gemm_tiles(nd, H, B):
+    # batches of the small, medium and large tiles (48, 64 and 128 columns wide),
+    # full and ragged, with gathered rows; tolerances as for any other batch
+    rng = np.random.default_rng(B)
+    p = synth.mlp_init(nd, H, 2)
+    net = colden.Net(nd, H, p)
+    x = synth.mlp_inputs(B + 7, 8 * nd + 1, seed=B)
+    y = (0.3 * rng.standard_normal((B + 7, nd))).astype(np.float32)
+    rows = rng.integers(0, B + 7, B)
+    mu, sinv = ol.normaliser(x.astype(np.float64))
+    st = net.state()
+    st["mu"], st["sinv"] = mu.astype(np.float32), sinv.astype(np.float32)
+    net.load_state(st)
+    args = (ol.unpack(p.astype(np.float64), nd, H), st["mu"].astype(np.float64), st["sinv"].astype(np.float64),
+            x[rows].astype(np.float64))
+    dx, dy, dr = torch.from_numpy(x).cuda(), torch.from_numpy(y).cuda(), torch.from_numpy(rows).cuda()
+    delta = torch.full((B, nd), 9.0, device="cuda")
+    net.forward(dx[dr].contiguous(), delta)
+    assert np.max(np.abs(delta.cpu().numpy() - ol.forward(*args)[0])) < 1e-4
+    loss, alone = torch.zeros(1, device="cuda"), torch.zeros(1, device="cuda")
+    grad = torch.full((net.n_params,), 9.0, device="cuda")
+    net.loss_grad(dx, dy, loss, grad, rows=dr)
+    net.loss_grad(dx, dy, alone, rows=dr)
+    want, g_or = ol.loss_grad(*args, y[rows].astype(np.float64))
+    g_or = ol.pack(g_or)
+    assert loss.item() == pytest.approx(want, rel=1e-5) and torch.equal(loss, alone)
+    assert np.max(np.abs(grad.cpu().numpy() - g_or)) < 1e-4 * np.max(np.abs(g_or))
