@@ -905,18 +905,19 @@ cd_status column_density_amr(cd_tree t, cd_geom g, const cd_opts &opts, float *n
     // far-shell prefixes of the refined cells
     for (int k = 3; k <= L - 2 && !insitu; ++k) {
         if (!t->n_ref[k]) continue;
-        if (tc && k >= 4 && t->tc_ref[k].ntiles) {
+        if ((tc || ext_fp32_serves_list(k, 4, g)) && k >= 4 && t->tc_ref[k].ntiles) {
             ExtLaunch e = {};
             e.k = k;
             e.nd = nd;
             e.tmask = 4;
+            e.rho[3] = t->rho_lvl[k - 2];
             e.dx[3] = dx(k - 2);
             e.prefix_in = (k - 1 >= 3) ? t->ws.S[k - 1] : nullptr;
             e.out = t->ws.S[k];
             // a fully refined level (below the base level) keeps every cell in Morton
             // order, so it takes the whole-level tiles of a uniform tree
             e.list = t->n_ref[k] == ((int64_t)1 << (3 * k)) ? nullptr : &t->tc_ref[k];
-            cd_status st = launch_ext_tc(e, t->rho_brick, g, s);
+            const cd_status st = tc ? launch_ext_tc(e, t->rho_brick, g, s) : launch_ext_fp32(e, g, s);
             if (st != CD_OK) return st;
             CD_CUDA(cudaEventRecord(t->ev_S[k], s));
             have_S[k] = true;
@@ -955,15 +956,18 @@ cd_status column_density_amr(cd_tree t, cd_geom g, const cd_opts &opts, float *n
             have_E[k] = true;
             continue;
         }
-        if (tc && k >= 4 && t->tc_oct[k].ntiles) {
+        if ((tc || ext_fp32_serves_list(k, 7, g)) && k >= 4 && t->tc_oct[k].ntiles) {
             ExtLaunch e = {};
             e.k = k;
             e.nd = nd;
             e.tmask = 7;
-            for (int q = 1; q <= 3; ++q) e.dx[q] = dx(k - q + 1);
+            for (int q = 1; q <= 3; ++q) {
+                e.rho[q] = t->rho_lvl[k - q + 1];
+                e.dx[q] = dx(k - q + 1);
+            }
             e.out = t->ws.E + t->oct_begin[k] * nd;
             e.list = &t->tc_oct[k];
-            cd_status st = launch_ext_tc(e, t->rho_brick, g, s_oct);
+            const cd_status st = tc ? launch_ext_tc(e, t->rho_brick, g, s_oct) : launch_ext_fp32(e, g, s_oct);
             if (st != CD_OK) return st;
             CD_CUDA(cudaEventRecord(t->ev_E[k], s_oct));
             have_E[k] = true;

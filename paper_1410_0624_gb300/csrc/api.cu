@@ -477,6 +477,7 @@ cd_status cd_precompute_geometry(int scheme, int p0, int p1, const double *dirs,
     }
     cd_status st = build_geometry_tables(g, s);
     if (st != CD_OK) return fail(st);
+    if ((st = build_row_lists(g, s)) != CD_OK) return fail(st);
     if ((st = build_tc_tables(g, s)) != CD_OK) return fail(st);
     // the tables are complete on return, so evaluations on any stream (not
     // only those ordered after `stream`) may read them
@@ -844,6 +845,10 @@ void cd_geom_free(cd_geom g)
     for (int t = 0; t < 4; ++t) {
         if (g->tab[t]) cd::lib_free(g->tab[t]);
         if (g->cmax[t]) cd::lib_free(g->cmax[t]);
+    }
+    for (cd_geom_s::RowList &L : g->rows) {
+        if (L.quad) cd::lib_free(L.quad);
+        if (L.start) cd::lib_free(L.start);
     }
     if (g->kloc) cd::lib_free(g->kloc);
     if (g->wb) cd::lib_free(g->wb);

@@ -1,5 +1,7 @@
-// FP32 CUDA-core form of the shell contraction (Eq. N_discret, one level of
-// receiving cells per launch).  For every cell c at level k and direction d:
+// FP32 CUDA-core forms of the shell contraction (Eq. N_discret, one level of
+// receiving cells per launch): the row form below serves receiving levels >= 4
+// and lists, the block form the few cells of coarser levels and runs of tables
+// the row form has no list for.  For every cell c at level k and direction d:
 //   out[c][d] = prefix_in[parent(c)][d]
 //             + sum_{t in tmask} dx_{k-t+1} sum_s rho_{k-t+1}(stencil_t(c), s) K_t[cfg_t(c)][d][s]
 // with the 6^3 stencil of table t anchored at the ancestor A_{k-t} of c and
@@ -17,6 +19,7 @@
 // contiguous, and each (cfg) row is walked to the largest non-zero count of
 // its directions (padding entries have weight 0).
 #include "common.cuh"
+#include "umma.cuh"
 
 namespace cd {
 namespace {
@@ -94,10 +97,388 @@ __global__ void __launch_bounds__(kExtThreads) shell_sum_fp32(ExtArgs P)
     }
 }
 
+
+// ---- row form (receiving levels >= 4) -------------------------------------------
+//
+// The kernel above reads a table entry (8 bytes, mostly from L2) and a density
+// from shared memory per lane, whose 32 directions hit random banks; its rows
+// are padded to the longest direction (18 entries where 10 are not zero).  Here
+// a warp computes four directions of 32 receiving cells of one configuration: a
+// lane has one direction and four cells, so that one entry (a broadcast read
+// for the eight lanes of a direction) serves four densities that lie next to
+// one another (16-byte reads without bank conflicts), and four directions walk
+// only as many entries as the longest of them has.
+//
+// One CTA takes 32 parents P of one class (the six Morton bits that, with the
+// child, select the weight rows): every cell of a level has the 64 classes of a
+// uniform tree, a list (AMR) groups its receivers' parents by class.  The
+// stencils of the three tables around every P are staged once as X[s][parent]
+// (648 densities per P, for 8 children x n_dir sums of about ten entries); 16
+// warps take the 8 children and halves of the directions.  A warp's entries are
+// one stream that comes through a small ring of asynchronous copies.  A 4 x 4
+// exchange between the lanes of a cell group turns the sums into rows of four
+// directions.
+//
+// What bounds it: shared memory, one wavefront per 32 (cell, direction) and
+// entry (L1 data pipe 93 % busy).  Octs of 256^3, 48 directions: 0.424 ms
+// against 1.400 with the kernel above; 40 cone-averaged directions at 128^3
+// (39 entries): 0.117 against 0.917; far shells of 64^3 cells 0.049 against
+// 0.130.  Steps on the way: one direction and lane-wise rows 0.49 ms (140
+// instructions an output row, entries read by every warp), the entries from L1
+// instead of the ring 0.68 (their latency).
+constexpr int kRowThreads = 512, kRowPitch = 36, kRowCells = CD_STENCIL, kRingQuads = 4;
+
+struct RowArgs {
+    int k, nd;
+    int t0, nt;                  // tables t0 .. t0 + nt - 1 are staged
+    const float *rho[4];         // dense level arrays by table
+    float scale;                 // dx of the weights' unit
+    const RowQuad *quad;
+    const int *start;
+    int width, cfg_mask;         // quad chunks per four directions at most; the configuration bits of the largest table
+    const float *prefix;         // S_{k-1} or NULL
+    float *out;
+    int64_t nG, nblk;            // uniform: 8^(k-3) rows per class in blocks of 32
+    const int4 *tiles;           // list: {class, first row, rows, half} in pairs, 128 rows at most
+    const uint64_t *row_key;     // list: parent Morton keys
+    const int32_t *row_out;      // list: [row][8] output row of child o, -1 if not a receiver
+    const int32_t *prefix_row;   // list: prefix row of each output row
+    int64_t n_out, n_prefix;     // rows (bounds checks)
+};
+
+template <bool kList>
+__global__ void __launch_bounds__(kRowThreads, 2) shell_rows_fp32(const __grid_constant__ RowArgs A)
+{
+    extern __shared__ __align__(128) float smem[];
+    float *X = smem;                                                  // [nt 216 + 1][36], the last row zero
+    __shared__ int s_p[3][32];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int nd = A.nd, nq = (nd + 3) >> 2;
+    RowQuad *ring = reinterpret_cast<RowQuad *>(smem + ((A.nt * kRowCells + 1) * kRowPitch + 31) / 32 * 32) +
+                    warp * 2 * kRingQuads;
+    int cls, nrows;
+    int64_t first;
+    if (kList) {
+        const int4 t = A.tiles[2 * (blockIdx.x >> 2)];
+        cls = t.x;
+        const int sub = 32 * (int)(blockIdx.x & 3);
+        first = t.y + sub;
+        nrows = min(32, t.z - sub);
+        if (nrows <= 0) return;
+    } else {
+        cls = (int)(blockIdx.x / A.nblk);                             // a class's blocks run together
+        first = (int64_t)(blockIdx.x % A.nblk) * 32;
+        nrows = (int)(A.nG - first < 32 ? A.nG - first : 32);
+    }
+    const int o = warp & 7, c9 = (cls << 3) | o, cfg = c9 & A.cfg_mask;
+    // this warp's quads of directions [qa, qb) and their stream of quad chunks
+    // (a ring block past the lists is allocated)
+    const int half = (nq + 1) / 2, qa = (warp >> 3) * half, qb = min(nq, qa + half);
+    const int *start = A.start + (size_t)cfg * (nq + 1);
+    const int first_quad = qa < qb ? start[qa] : 0, n = qa < qb ? start[qb] - first_quad : 0;
+    const char *stream = reinterpret_cast<const char *>(A.quad + (size_t)cfg * nq * A.width + first_quad);
+    static_assert(kRingQuads * sizeof(RowQuad) == 32 * 16, "a ring block is one copy per lane");
+    const auto issue = [&](int blk) {
+        if (blk * kRingQuads < n)
+            cp_async16(reinterpret_cast<char *>(ring + (blk & 1) * kRingQuads) + 16 * lane,
+                       stream + (size_t)blk * kRingQuads * sizeof(RowQuad) + 16 * lane, 16u);
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    issue(0);
+    issue(1);
+    if (warp == 0) {
+        const bool live = lane < nrows;
+        const uint64_t P = !live ? 0 : kList ? A.row_key[first + lane] : (uint64_t)(first + lane) << 6 | (uint64_t)cls;
+        s_p[0][lane] = live ? (int)compact3(P) : -1;
+        s_p[1][lane] = (int)compact3(P >> 1);
+        s_p[2][lane] = (int)compact3(P >> 2);
+    }
+    for (int i = tid; i < kRowPitch; i += kRowThreads) X[A.nt * kRowCells * kRowPitch + i] = 0.f;
+    // this lane's output and prefix rows once its sums are exchanged: parent 4 (lane & 7) + (lane >> 3)
+    const int g = lane >> 3, r_out = 4 * (lane & 7) + g;
+    int64_t orow = -1, prow = -1;
+    if (r_out < nrows) {
+        orow = kList ? (int64_t)A.row_out[8 * (first + r_out) + o] : (first + r_out) * 512 + c9;
+        if (orow >= 0 && !in_bounds(orow, A.n_out, kCheckFp32Out)) orow = -1;
+        if (orow >= 0 && A.prefix) prow = kList ? (int64_t)A.prefix_row[orow] : (first + r_out) * 64 + cls;
+        if (prow >= 0 && !in_bounds(prow, A.n_prefix, kCheckFp32Prefix)) prow = -1;
+    }
+    float *out = A.out + (orow < 0 ? 0 : orow) * nd;
+    const float *pre = prow < 0 ? nullptr : A.prefix + prow * nd;
+    __syncthreads();
+
+    // stage the stencils: a warp takes (y, z) rows of one table's stencils, three
+    // reads of a pair of cells for the 32 parents; its lanes take the three pairs
+    // of four parents that are neighbours in x on a uniform tree (one line of
+    // densities) before the next four
+    const int groups = 16 / A.nt, q = warp % A.nt, sub = warp / A.nt;
+    if (sub < groups) {
+        const int t = A.t0 + q, side = 1 << (A.k - t + 1);
+        const float *rho = A.rho[t];
+        int base[3], dst[3];
+        uint32_t in_y[3], in_z[3];
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+            const int u = lane + 32 * j, a = 2 * (u % 3), v = u / 3, gr = v >> 2;
+            const int r = (v & 1) | ((v & 2) << 2) | ((gr & 3) << 1) | ((gr >> 2) << 4);
+            const int px = s_p[0][r];
+            const int x = 2 * ((px >> (t - 1)) - 1) + a, y = 2 * ((s_p[1][r] >> (t - 1)) - 1),
+                      z = 2 * ((s_p[2][r] >> (t - 1)) - 1);
+            base[j] = (z * side + y) * side + x;
+            dst[j] = (q * kRowCells + a) * kRowPitch + r;
+            in_y[j] = in_z[j] = 0;
+#pragma unroll
+            for (int i = 0; i < 6; ++i) {
+                in_y[j] |= (uint32_t)(y + i >= 0 && y + i < side) << i;
+                in_z[j] |= (uint32_t)(z + i >= 0 && z + i < side) << i;
+            }
+            if (px < 0 || x < 0 || x >= side) in_y[j] = 0;
+        }
+        for (int bc0 = sub; bc0 < 36; bc0 += 4 * groups) {
+            float2 f[4][3];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const int bc = bc0 + i * groups, b = bc % 6, c = bc / 6, step = (c * side + b) * side;
+#pragma unroll
+                for (int j = 0; j < 3; ++j) {
+                    f[i][j] = make_float2(0.f, 0.f);
+                    if (bc < 36 && ((in_y[j] >> b) & (in_z[j] >> c) & 1u) &&
+                        in_bounds((long long)base[j] + step + 1, (long long)side * side * side, kCheckListLevel))
+                        f[i][j] = *reinterpret_cast<const float2 *>(rho + (base[j] + step));
+                }
+            }
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const int bc = bc0 + i * groups;
+                if (bc >= 36) break;
+#pragma unroll
+                for (int j = 0; j < 3; ++j) {
+                    float *p = X + 6 * bc * kRowPitch + dst[j];
+                    p[0] = f[i][j].x;
+                    p[kRowPitch] = f[i][j].y;
+                }
+            }
+        }
+    }
+    __syncthreads();
+
+    const char *Xl = reinterpret_cast<const char *>(X + 4 * (lane & 7));
+    float acc[4] = {0.f, 0.f, 0.f, 0.f};                              // direction 4 quad + g of parents 4 (lane & 7) ..
+    int d = 4 * qa;
+    const auto add = [&](int off, float w) {
+        const float4 x = *reinterpret_cast<const float4 *>(Xl + off);
+        acc[0] = fmaf(x.x, w, acc[0]);
+        acc[1] = fmaf(x.y, w, acc[1]);
+        acc[2] = fmaf(x.z, w, acc[2]);
+        acc[3] = fmaf(x.w, w, acc[3]);
+    };
+    for (int blk = 0; blk * kRingQuads < n; ++blk) {
+        asm volatile("cp.async.wait_group 1;" ::: "memory");
+        __syncwarp();
+        const RowChunk *rb = ring[(blk & 1) * kRingQuads].d + g;
+        const int cnt = min(kRingQuads, n - blk * kRingQuads);
+#pragma unroll 1
+        for (int j = 0; j < cnt; ++j, rb += 4) {
+            const RowChunk v = *rb;
+            const int ow = v.off.w & ~1;                              // bit 0: the quad's last chunk
+            if (in_bounds(max(max(v.off.x, v.off.y), max(v.off.z, ow)), (A.nt * kRowCells + 1) * kRowPitch * 4,
+                          kCheckFp32Region)) {
+                add(v.off.x, v.w.x);
+                add(v.off.y, v.w.y);
+                add(v.off.z, v.w.z);
+                add(ow, v.w.w);
+            }
+            if (!(v.off.w & 1)) continue;
+            // exchange: lane g of a group of four parents gets its parent's four directions
+            const bool g0 = g & 1, g1 = g & 2;
+            float s0 = __shfl_xor_sync(0xffffffffu, g0 ? acc[0] : acc[1], 8);
+            float s1 = __shfl_xor_sync(0xffffffffu, g0 ? acc[2] : acc[3], 8);
+            if (g0) { acc[0] = s0; acc[2] = s1; } else { acc[1] = s0; acc[3] = s1; }
+            s0 = __shfl_xor_sync(0xffffffffu, g1 ? acc[0] : acc[2], 16);
+            s1 = __shfl_xor_sync(0xffffffffu, g1 ? acc[1] : acc[3], 16);
+            if (g1) { acc[0] = s0; acc[1] = s1; } else { acc[2] = s0; acc[3] = s1; }
+            if (orow >= 0) {
+                if ((nd & 3) == 0) {
+                    float4 p = make_float4(0.f, 0.f, 0.f, 0.f);
+                    if (pre) p = *reinterpret_cast<const float4 *>(pre + d);
+                    *reinterpret_cast<float4 *>(out + d) =
+                        make_float4(fmaf(A.scale, acc[0], p.x), fmaf(A.scale, acc[1], p.y), fmaf(A.scale, acc[2], p.z),
+                                    fmaf(A.scale, acc[3], p.w));
+                } else {
+#pragma unroll
+                    for (int i = 0; i < 4; ++i)
+                        if (d + i < nd) out[d + i] = fmaf(A.scale, acc[i], pre ? pre[d + i] : 0.f);
+                }
+            }
+            acc[0] = acc[1] = acc[2] = acc[3] = 0.f;
+            d += 4;
+        }
+        __syncwarp();
+        issue(blk + 2);
+    }
+}
+
+// One warp per configuration of list i, a lane per quad of directions: the
+// quads' chunks one after another (at least one each), start[cfg][quad] the
+// first of each.  A quad has as many as its longest direction; entries not used
+// have weight 0 and point at the zero row, and bit 0 of the last offset marks
+// the quad's last chunk.
+__global__ void __launch_bounds__(128) row_lists(int i, int nd, int ncfg, const int2 *t1, const int2 *t2,
+                                                 const int2 *t3, int maxe, int width, RowQuad *__restrict__ quad,
+                                                 int *__restrict__ start)
+{
+    const int cfg = (int)(blockIdx.x * 4 + (threadIdx.x >> 5)), lane = threadIdx.x & 31;
+    if (cfg >= ncfg) return;
+    const int nq = (nd + 3) / 4;
+    const int ta = i < 3 ? i + 1 : 1, tb = i < 3 ? i + 1 : 3;
+    const int zero = (tb - ta + 1) * kRowCells * kRowPitch * 4;
+    const auto entry = [&](int t, int q, int d) {   // entries of a row come first, then zeros
+        const int2 *tab = t == 1 ? t1 : t == 2 ? t2 : t3;
+        return tab[((size_t)(cfg & ((1 << (3 * t)) - 1)) * maxe + q) * nd + d];
+    };
+    int done = 0;
+    for (int q0 = 0; q0 < nq; q0 += 32) {
+        const int qd = q0 + lane;
+        int chunks = qd < nq ? 1 : 0;
+        for (int d = 4 * qd; d < min(nd, 4 * qd + 4); ++d) {
+            int count = 0;
+            for (int t = ta; t <= tb; ++t)
+                for (int q = 0; q < maxe && __int_as_float(entry(t, q, d).y) != 0.f; ++q) ++count;
+            chunks = max(chunks, (count + 3) / 4);
+        }
+        int inc = chunks;
+        for (int s = 1; s < 32; s <<= 1) {
+            const int v = __shfl_up_sync(0xffffffffu, inc, s);
+            if (lane >= s) inc += v;
+        }
+        const int first = done + inc - chunks;
+        done += __shfl_sync(0xffffffffu, inc, 31);
+        if (qd < nq) {
+            start[(size_t)cfg * (nq + 1) + qd] = first;
+            for (int j = 0; j < 4; ++j) {
+                RowQuad *to = quad + (size_t)cfg * nq * width + first;
+                const int d = 4 * qd + j;
+                int t = ta, q = 0;
+                for (int c = 0; c < chunks; ++c) {
+                    float w[4];
+                    int off[4];
+                    for (int e = 0; e < 4; ++e) {
+                        w[e] = 0.f;
+                        off[e] = zero;
+                        while (d < nd && t <= tb) {
+                            const int2 v = q < maxe ? entry(t, q, d) : make_int2(0, 0);
+                            if (__int_as_float(v.y) == 0.f) {
+                                ++t;
+                                q = 0;
+                                continue;
+                            }
+                            const int R = region_side(t);
+                            const int s = v.x % R + 6 * ((v.x / R) % R) + 36 * (v.x / (R * R));
+                            w[e] = __int_as_float(v.y) * (i < 3 ? 1.f : (float)(1 << (t - 1)));
+                            off[e] = ((t - ta) * kRowCells + s) * kRowPitch * 4;
+                            ++q;
+                            break;
+                        }
+                    }
+                    if (c == chunks - 1) off[3] |= 1;
+                    to[c].d[j] = {make_float4(w[0], w[1], w[2], w[3]), make_int4(off[0], off[1], off[2], off[3])};
+                }
+            }
+        }
+        __syncwarp();
+    }
+    if (lane == 0) start[(size_t)cfg * (nq + 1) + nq] = done;
+}
+
+size_t row_smem(int nt)
+{
+    return sizeof(float) * (((size_t)(nt * kRowCells + 1) * kRowPitch + 31) / 32 * 32) +
+           16 * 2 * kRingQuads * sizeof(RowQuad);
+}
+
+// the list of a table mask, or -1
+int row_list(int tmask) { return tmask == 1 ? 0 : tmask == 2 ? 1 : tmask == 4 ? 2 : tmask == 7 ? 3 : -1; }
+
+cd_status launch_rows(const ExtLaunch &a, cd_geom g, cudaStream_t s)
+{
+    const int li = row_list(a.tmask);
+    const cd_geom_s::RowList &L = g->rows[li];
+    RowArgs A = {};
+    A.k = a.k;
+    A.nd = a.nd;
+    A.t0 = li < 3 ? li + 1 : 1;
+    A.nt = li < 3 ? 1 : 3;
+    for (int t = 1; t <= 3; ++t) A.rho[t] = a.rho[t];
+    A.scale = a.dx[A.t0];
+    A.quad = L.quad;
+    A.start = L.start;
+    A.width = L.width;
+    A.cfg_mask = (li < 3 ? 8 << (3 * li) : 512) - 1;
+    A.prefix = a.prefix_in;
+    A.out = a.out;
+    int64_t grid;
+    if (a.list) {
+        A.tiles = a.list->tiles;
+        A.row_key = a.list->key;
+        A.row_out = a.list->out;
+        A.prefix_row = a.list->recv_parent;
+        A.n_out = a.list->n_recv;
+        A.n_prefix = (int64_t)1 << (3 * (a.k - 1));
+        grid = a.list->ntiles / 2 * 4;
+    } else {
+        A.nG = (int64_t)1 << (3 * (a.k - 3));
+        A.nblk = (A.nG + 31) / 32;
+        A.n_out = (int64_t)1 << (3 * a.k);
+        A.n_prefix = (int64_t)1 << (3 * (a.k - 1));
+        grid = 64 * A.nblk;
+    }
+    if (grid == 0) return CD_OK;
+    const size_t smem = row_smem(A.nt);
+    const auto kern = a.list ? shell_rows_fp32<true> : shell_rows_fp32<false>;
+    CD_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)row_smem(3)));
+    LaunchScope ls(CD_K_SHELL, s);
+    kern<<<(unsigned)grid, kRowThreads, smem, s>>>(A);
+    CD_CHECK_LAUNCH();
+    return CD_OK;
+}
+
 }  // namespace
+
+bool ext_fp32_serves_list(int k, int tmask, cd_geom g)
+{
+    const int li = row_list(tmask);
+    return k >= 4 && li >= 0 && g->rows[li].quad != nullptr;
+}
+
+cd_status build_row_lists(cd_geom g, cudaStream_t s)
+{
+    // rows of a list are as wide as the largest counts allow; direction sets
+    // whose lists would take more than 256 MB stay with the tables alone
+    constexpr size_t kMaxBytes = (size_t)256 << 20;
+    for (int i = 0; i < 4; ++i) {
+        cd_geom_s::RowList &L = g->rows[i];
+        const int ncfg = i < 3 ? 8 << (3 * i) : 512;
+        L.width = ((i < 3 ? 1 : 3) * g->maxe + 3) / 4;
+        const int nq = (g->n_dir + 3) / 4;
+        const size_t quads = (size_t)ncfg * nq * L.width + kRingQuads;   // the kernel reads whole blocks
+        if (quads * sizeof(RowQuad) > kMaxBytes) continue;
+        if (cudaMalloc(&L.quad, quads * sizeof(RowQuad)) != cudaSuccess ||
+            cudaMalloc(&L.start, sizeof(int) * ncfg * (nq + 1)) != cudaSuccess) {
+            cudaGetLastError();
+            set_error("cannot allocate the shell row lists (%zu bytes)", quads * sizeof(RowQuad));
+            return CD_ENOMEM;
+        }
+        LaunchScope ls(CD_K_OTHER, s);
+        row_lists<<<(unsigned)((ncfg + 3) / 4), 128, 0, s>>>(i, g->n_dir, ncfg, g->tab[1], g->tab[2], g->tab[3], g->maxe,
+                                                            L.width, L.quad, L.start);
+        CD_CHECK_LAUNCH();
+    }
+    return CD_OK;
+}
 
 cd_status launch_ext_fp32(const ExtLaunch &a, cd_geom g, cudaStream_t s)
 {
+    if (ext_fp32_serves_list(a.k, a.tmask, g)) return launch_rows(a, g, s);
     ExtArgs P;
     P.a = a;
     // largest span <= min(3, k) that still gives >= 304 CTAs (2 per SM)

@@ -142,6 +142,17 @@ struct LevelSums {
     int64_t rows = 0;
 };
 
+// Four entries of a sparse shell row: weights and the byte offsets of the
+// staged stencil rows they multiply (colden_fp32.cu); a quad chunk has four for
+// each of four directions.
+struct RowChunk {
+    float4 w;
+    int4 off;
+};
+struct RowQuad {
+    RowChunk d[4];
+};
+
 // A sparse set of receiving cells of one level (AMR meshes), arranged for the
 // tensor-core shell contraction: the receivers' parents grouped by class
 // (the low six Morton bits), and the tiles over those rows.
@@ -251,6 +262,16 @@ struct cd_geom_s {
     int maxe = 0;
     int2 *tab[4] = {};
     int *cmax[4] = {};
+    // the same weights in quad chunks for the row kernel (colden_fp32.cu): list
+    // i = 0 .. 2 holds table i + 1, list 3 all three with table t's weights times
+    // 2^(t-1).  A configuration's chunks start at cfg * n_quad * width, its quads
+    // of four directions one after another from start[cfg][0 .. n_quad].  NULL
+    // where a list would take too much memory
+    struct RowList {
+        int width = 0;                  // chunks of a quad at most
+        cd::RowQuad *quad = nullptr;
+        int *start = nullptr;
+    } rows[4];
     float *kloc = nullptr;              // [8 t][8 s][nd], units of dx
     // BF16 B operands for the tensor-core contraction (see colden_tc.cu)
     __nv_bfloat16 *wb = nullptr;
@@ -376,10 +397,14 @@ struct ExtLaunch {
     float dx[4];              // dx of that shell level, cm
     const float *prefix_in;   // S_{k-1} (Morton) or NULL
     float *out;               // Morton [8^k][nd], or [n_recv][nd] with a list
-    const TcList *list;       // tensor-core form only: receivers of an AMR level (NULL: every cell of level k)
+    const TcList *list;       // receivers of an AMR level (NULL: every cell of level k)
     int tiles_per_cta;        // tensor-core form: 0 = persistent CTAs (two per SM); n = one CTA per n tiles
 };
 cd_status launch_ext_fp32(const ExtLaunch &a, cd_geom g, cudaStream_t s);
+// whether launch_ext_fp32 serves a list of receivers of level k with these tables
+bool ext_fp32_serves_list(int k, int tmask, cd_geom g);
+// the chunk lists of the tables (after build_geometry_tables)
+cd_status build_row_lists(cd_geom g, cudaStream_t s);
 
 struct LeafLaunch {
     int64_t n_oct;

@@ -79,3 +79,43 @@ def test_network_at_the_edges_of_its_gemm_tiles(nd, H, B):
     g_or = ol.pack(g_or)
     assert loss.item() == pytest.approx(want, rel=1e-5) and torch.equal(loss, alone)
     assert np.max(np.abs(grad.cpu().numpy() - g_or)) < 1e-4 * np.max(np.abs(g_or))
+
+
+@pytest.mark.parametrize("L,dset,mode", [(5, ("custom", 0, 0, [[0.3, -0.5, 0.8]]), 0), (5, ("mxn", 3, 1), 0),
+                                         (6, ("mxn", 5, 3), 0), (6, ("mxn", 14, 9), 0), (7, ("axes", 0, 0), 0),
+                                         (7, ("mxn", 5, 8), 2), (8, ("mxn", 2, 2), 0)])
+def test_fp32_shell_rows_match_oracle(L, dset, mode):
+    # direction counts that fill a quad of directions or leave part of it, levels
+    # with fewer and more parents per class than a CTA takes; FP32 tolerance
+    rho = _rho(L, 50 + L)
+    tree = colden.build_tree_uniform(torch.from_numpy(rho).cuda(), BOX)
+    geom = colden.precompute_geometry(*dset, mode=mode)
+    nh = torch.empty((tree.n_leaf, geom.n_dir), device="cuda")
+    colden.column_density(tree, geom, n_h=nh)
+    corner = np.array([0, tree.n_leaf - 1, tree.n_leaf // 2, tree.n_leaf // 8 + 1])
+    rows = np.unique(np.concatenate([corner, np.random.default_rng(L).integers(0, tree.n_leaf, 250)]))
+    ijk = oracle.morton_ijk(L)[rows] if L < 8 else tree.leaves()[1][rows]
+    T = oracle.Tree.uniform(rho, BOX)
+    lv = np.full(len(rows), L)
+    want = T.column_density_cone(geom.dirs, lv, ijk) if mode else T.column_density(geom.dirs, lv, ijk)
+    got = nh[torch.from_numpy(rows).cuda()].double().cpu().numpy()
+    assert np.max(np.abs(got - want) / want) <= 1e-5
+
+
+@pytest.mark.parametrize("dset", [("mxn", 5, 3), ("axes", 0, 0), ("healpix", 2, 0)])
+def test_fp32_shell_rows_on_lists_match_uniform(dset):
+    # a mesh refined in one corner: its finest leaves far inside the refined part
+    # and its base leaves against the oracle's adaptive tree
+    fine = _rho(7, 3, 1.0)
+    fine[:40, :44, :48] *= 50.0
+    lv = synth.amr_leaves(fine, 5, [100.0, 200.0])
+    tree = colden.build_tree_amr(5, 7, BOX, lv["level"], lv["ijk"], lv["rho"])
+    geom = colden.precompute_geometry(*dset)
+    nh = torch.empty((tree.n_leaf, geom.n_dir), device="cuda")
+    colden.column_density(tree, geom, n_h=nh)
+    level, ijk = tree.leaves()
+    rng = np.random.default_rng(1)
+    rows = np.concatenate([rng.choice(np.flatnonzero(level == l), 120) for l in np.unique(level)])
+    want = oracle.Tree.amr(5, 7, BOX, lv["level"], lv["ijk"], lv["rho"]).column_density(geom.dirs, level[rows], ijk[rows])
+    got = nh[torch.from_numpy(rows).cuda()].double().cpu().numpy()
+    assert np.max(np.abs(got - want) / want) <= 1e-5
