@@ -537,6 +537,222 @@ __global__ void __launch_bounds__(512, 1) leaf_tc(LeafTcArgs P0, LeafBatch Bt)
     }
 }
 
+// ---- few directions: octs as rows ------------------------------------------------
+//
+// Up to 32 directions the tile above is mostly latency: 128 leaves of 12
+// directions are 1 536 sums behind three barriers and a product.  Here a row of
+// the product is an oct: D[oct][t nd + d] = sum_s rho[oct][s] (dx_L Kloc[t][s][d])
+// has M = 128 octs, N = 8 nd columns (at most 256) and K = 16 (its 8 siblings and
+// 8 zeros; the same BF16 operands as above), so that one product and one round
+// of barriers serve 1 024 leaves.  A thread has one oct: its external column
+// E + Sp stays in registers for the 8 children, and their screening factors are
+// 32 contiguous bytes.
+// N_H and A_V rows leave through a per-warp transpose, 128 bytes of a row at a
+// time.
+// What bounds it: the exponentials (16 a clock and SM), with rows the HBM
+// stores.  256^3 leaves, 12 directions: 0.068 ms for the screening factor alone,
+// 0.189 with N_H, 0.327 with A_V too (4.9 TB/s), against 0.314, 0.339 and 0.691 in
+// tiles of 128 leaves; 32 directions: 0.210, 0.456, 0.845 against 0.389, 0.759,
+// 3.08.  (Rows stored straight from the threads, 16 bytes each: 0.49 for N_H
+// at 12 directions.)
+struct LeafOctArgs {
+    LeafLaunch a;
+    int64_t ntiles;              // of 128 octs
+    float c2;                    // -shield_k av_per_nh log2(e)
+    uint32_t pipe_polls;
+};
+
+template <int ND>
+struct LeafOctShape {
+    static constexpr int N = 8 * ND;
+    static constexpr int kCols = N <= 64 ? 64 : N <= 128 ? 128 : 256;   // TMEM columns of a group
+    static constexpr int kGroups = 512 / kCols > 4 ? 4 : 512 / kCols;
+    static constexpr uint32_t kB = N * 32, kA = 4096;                    // operand bytes (K = 16)
+    static constexpr uint32_t kE = 128 * ND * 4, kP = 16 * ND * 4, kStage = kE + kP + 4096;
+    static constexpr uint32_t kGroup = kA + 2 * kStage;
+    static constexpr uint32_t kT = 128 * 36 * 4;                         // a group's row transposes
+    static constexpr size_t smem(int G, bool rows) { return kB + (size_t)G * (kGroup + (rows ? kT : 0)); }
+};
+
+// kRows: N_H or A_V rows are wanted (16-byte aligned)
+template <int ND, bool kRows>
+__global__ void __launch_bounds__(128 * LeafOctShape<ND>::kGroups, 1) leaf_oct_tc(const __grid_constant__ LeafOctArgs P)
+{
+    using S = LeafOctShape<ND>;
+    extern __shared__ __align__(1024) unsigned char smem[];
+    __shared__ uint64_t bar[3 * S::kGroups];      // [g] products, [G + 2 g + stage] input stages
+    __shared__ uint32_t tslot;
+    __shared__ int sflag[S::kGroups];
+    const int tid = threadIdx.x, warp = tid >> 5, g = warp >> 2, quarter = warp & 3, i = tid & 127;
+    const int G = blockDim.x >> 7;
+    unsigned char *sA = smem + S::kB + (size_t)g * S::kGroup;
+    unsigned char *stage0 = sA + S::kA;
+    const int64_t n_oct = P.a.n_oct;
+    const auto octs = [&](int64_t tile) { return (uint32_t)(n_oct - tile * 128 < 128 ? n_oct - tile * 128 : 128); };
+    const auto prefetch = [&](int64_t tile, int s) {
+        const int64_t o0 = tile * 128;
+        const uint32_t nb = octs(tile);
+        uint64_t *b = &bar[S::kGroups + 2 * g + s];
+        unsigned char *st = stage0 + s * S::kStage;
+        if (!(in_bounds(o0, n_oct, kCheckLeafTcIn) && in_bounds(o0 + nb - 1, n_oct, kCheckLeafTcIn) &&
+              (!P.a.Sp || in_bounds((o0 + nb - 1) >> 3, n_oct / 8, kCheckLeafTcIn)))) {
+            mbar_expect_tx(b, 0);
+            return;
+        }
+        const uint32_t bp = P.a.Sp ? (nb + 7) / 8 * ND * 4 : 0u;
+        mbar_expect_tx(b, nb * (ND * 4 + 32) + bp);
+        bulk_g2s(st, P.a.E + o0 * ND, nb * ND * 4, b);
+        if (P.a.Sp) bulk_g2s(st + S::kE, P.a.Sp + (o0 >> 3) * ND, bp, b);
+        bulk_g2s(st + S::kE + S::kP, P.a.rho_leaf + o0 * 8, nb * 32, b);
+    };
+
+    if (tid == 0) {
+        for (int b = 0; b < 3 * S::kGroups; ++b) mbar_init(&bar[b], 1);
+        fence_mbar_init();
+        for (int q = 0; q < S::kGroups; ++q) sflag[q] = 0;
+    }
+    for (int n = tid; n < S::N; n += blockDim.x) {
+        const float *k = P.a.kloc + (n / ND) * 8 * ND + n % ND;
+        float v[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) v[q] = P.a.dx_leaf * k[q * ND];
+        *reinterpret_cast<uint4 *>(smem + op_off(n, 0, 16)) = make_uint4(
+            pack_bf16x2(v[0], v[1]), pack_bf16x2(v[2], v[3]), pack_bf16x2(v[4], v[5]), pack_bf16x2(v[6], v[7]));
+        *reinterpret_cast<uint4 *>(smem + op_off(n, 8, 16)) = make_uint4(0, 0, 0, 0);
+    }
+    *reinterpret_cast<uint4 *>(sA + op_off(i, 8, 16)) = make_uint4(0, 0, 0, 0);
+    fence_proxy_async_smem();
+    if (warp == 0) tmem_alloc(&tslot, S::kCols * S::kGroups);
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tD = tslot + (uint32_t)(g * S::kCols), taddr = tD + ((uint32_t)(quarter * 32) << 16);
+    const int64_t first = (int64_t)blockIdx.x * G + g, stride = (int64_t)gridDim.x * G;
+    uint32_t phase = 0, sphase[2] = {0, 0};
+    bool pending[2] = {false, false}, fault = false;
+    if (i == 0 && first < P.ntiles) {
+        prefetch(first, 0);
+        pending[0] = true;
+    }
+    int s = 0;
+    for (int64_t tile = first; tile < P.ntiles; tile += stride, s ^= 1) {
+        if (i == 0) {
+            if (tile + stride < P.ntiles) {
+                prefetch(tile + stride, s ^ 1);
+                pending[s ^ 1] = true;
+            }
+            if (mbar_wait_bounded(&bar[S::kGroups + 2 * g + s], sphase[s], P.pipe_polls)) {
+                pending[s] = false;
+                sphase[s] ^= 1;
+            } else {
+                sflag[g] = 1;
+            }
+        }
+        named_barrier(1 + g, 128);
+        if (sflag[g]) {
+            fault = true;
+            break;
+        }
+        const unsigned char *st = stage0 + s * S::kStage;
+        const float *rho = reinterpret_cast<const float *>(st + S::kE + S::kP) + 8 * i;
+        const float4 r0 = *reinterpret_cast<const float4 *>(rho), r1 = *reinterpret_cast<const float4 *>(rho + 4);
+        *reinterpret_cast<uint4 *>(sA + op_off(i, 0, 16)) = make_uint4(
+            pack_bf16x2(r0.x, r0.y), pack_bf16x2(r0.z, r0.w), pack_bf16x2(r1.x, r1.y), pack_bf16x2(r1.z, r1.w));
+        float e[ND];
+#pragma unroll
+        for (int d = 0; d < ND; d += 4) {
+            float4 v = *reinterpret_cast<const float4 *>(reinterpret_cast<const float *>(st) + i * ND + d);
+            if (P.a.Sp) {
+                const float4 p = *reinterpret_cast<const float4 *>(reinterpret_cast<const float *>(st + S::kE) + (i >> 3) * ND + d);
+                v.x += p.x;
+                v.y += p.y;
+                v.z += p.z;
+                v.w += p.w;
+            }
+            e[d] = v.x;
+            e[d + 1] = v.y;
+            e[d + 2] = v.z;
+            e[d + 3] = v.w;
+        }
+        fence_proxy_async_smem();
+        tc_fence_before();
+        named_barrier(1 + g, 128);
+        if (i == 0) {
+            tc_fence_after();
+            umma_bf16(tD, umma_smem_desc(smem_u32(sA), 128, 256), umma_smem_desc(smem_u32(smem), 128, 256),
+                      umma_idesc_bf16(128, S::N), 0u);
+            umma_commit(&bar[g]);
+            if (!mbar_wait_bounded(&bar[g], phase, P.pipe_polls)) sflag[g] = 1;
+        }
+        phase ^= 1;
+        named_barrier(1 + g, 128);
+        if (sflag[g]) {
+            fault = true;
+            break;
+        }
+        tc_fence_after();
+        const int64_t oct = tile * 128 + i;
+        const bool ok = oct < n_oct && in_bounds(oct, n_oct, kCheckLeafTcOut);
+        // rows: 32 columns of the warp's 32 octs at a time turn into 128-byte
+        // pieces of the octs' rows through a padded square of shared memory
+        float *T = reinterpret_cast<float *>(smem + S::kB + (size_t)G * S::kGroup) + (warp * 32) * 36;
+        const int lane = tid & 31;
+        const int64_t row0 = tile * 128 + quarter * 32 + (lane >> 3);
+        float acc[8];
+#pragma unroll
+        for (int t = 0; t < 8; ++t) acc[t] = 0.f;
+#pragma unroll
+        for (int c = 0; c < S::N; c += 32) {
+            uint32_t v[32];
+            __syncwarp();
+            tmem_ld32(taddr + (uint32_t)c, v);
+            tmem_ld_wait();
+#pragma unroll
+            for (int j = 0; j < 32; j += 4) {
+                const int t = (c + j) / ND, d = (c + j) % ND;
+                const float4 N = make_float4(__uint_as_float(v[j]) + e[d], __uint_as_float(v[j + 1]) + e[d + 1],
+                                             __uint_as_float(v[j + 2]) + e[d + 2], __uint_as_float(v[j + 3]) + e[d + 3]);
+                acc[t] += (fast_exp2(P.c2 * N.x) + fast_exp2(P.c2 * N.y)) + (fast_exp2(P.c2 * N.z) + fast_exp2(P.c2 * N.w));
+                if (kRows) *reinterpret_cast<float4 *>(T + lane * 36 + j) = N;
+            }
+            if (kRows) {
+                __syncwarp();
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    const int64_t o = row0 + 4 * j;
+                    if (o >= n_oct || !in_bounds(o, n_oct, kCheckLeafTcOut)) break;
+                    const float4 N = *reinterpret_cast<const float4 *>(T + ((lane >> 3) + 4 * j) * 36 + 4 * (lane & 7));
+                    const int64_t at = o * S::N + c + 4 * (lane & 7);
+                    const float k = P.a.av_per_nh;
+                    if (P.a.n_h) *reinterpret_cast<float4 *>(P.a.n_h + at) = N;
+                    if (P.a.a_v) *reinterpret_cast<float4 *>(P.a.a_v + at) = make_float4(N.x * k, N.y * k, N.z * k, N.w * k);
+                }
+            }
+        }
+        if (P.a.shield && ok) {
+            float4 *sh = reinterpret_cast<float4 *>(P.a.shield + oct * 8);
+            const float n = (float)ND;
+            sh[0] = make_float4(acc[0] / n, acc[1] / n, acc[2] / n, acc[3] / n);
+            sh[1] = make_float4(acc[4] / n, acc[5] / n, acc[6] / n, acc[7] / n);
+        }
+        tc_fence_before();
+    }
+    if (i == 0) {
+        if (fault) {
+            atomicExch(&g_leaftc_fault, 1);
+            mbar_wait_bounded(&bar[g], phase ^ 1, kMaxPolls);   // let an issued product finish
+        }
+        for (int b = 0; b < 2; ++b)
+            if (pending[b]) mbar_wait_bounded(&bar[S::kGroups + 2 * g + b], sphase[b], kMaxPolls);
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 0) {
+        tc_fence_after();
+        tmem_dealloc(tslot, S::kCols * S::kGroups);
+    }
+}
+
 int sms()
 {
     int dev = 0, n = 0;
@@ -546,6 +762,31 @@ int sms()
 }
 
 bool aligned16(const void *p) { return ((uintptr_t)p & 15) == 0; }
+
+template <int ND>
+cd_status launch_leaf_oct(const LeafOctArgs &P, cudaStream_t s)
+{
+    using S = LeafOctShape<ND>;
+    // as many groups a CTA as leave every SM one (a small tree's tiles go to more SMs)
+    int G = S::kGroups;
+    while (G > 1 && (P.ntiles + G - 1) / G < sms()) --G;
+    const auto kern = P.a.n_h || P.a.a_v ? leaf_oct_tc<ND, true> : leaf_oct_tc<ND, false>;
+    const bool rows = P.a.n_h || P.a.a_v;
+    const size_t smem = S::smem(G, rows);
+    CD_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::smem(S::kGroups, rows)));
+    const int64_t grid = std::min<int64_t>((P.ntiles + G - 1) / G, sms());
+    LaunchScope ls(CD_K_LEAF, s, 2.0 * (double)P.ntiles * 128.0 * 16 * S::N);
+    kern<<<(unsigned)grid, 128 * G, smem, s>>>(P);
+    CD_CHECK_LAUNCH();
+    return CD_OK;
+}
+
+// poll limit of the pipeline waits (cd_debug_wait_polls)
+uint32_t pipe_polls()
+{
+    const int64_t cap = g_pipe_polls.load();
+    return cap < 0 ? kMaxPolls : (uint32_t)std::min<int64_t>(cap, kMaxPolls);
+}
 
 }  // namespace
 
@@ -561,6 +802,26 @@ cd_status launch_leaf_tc(const LeafLaunch &a, cudaStream_t s)
     if (!list && (n_leaf < 128 || n_leaf % 128 != 0)) return CD_EUNSUPPORTED;
     if (list && ((a.Sp && !a.oparent) || !aligned16(a.oleaf) || (a.n_h && !aligned16(a.n_h)))) return CD_EUNSUPPORTED;
     if (n_leaf == 0) return CD_OK;
+    // 8 n_dir columns fit one product up to 32 directions; from 128 leaves to 256^3
+    // the oct form is the faster one there (8.0 against 8.2 us at 16^3, 12.0 against
+    // 14.5 at 64^3, 12 directions), beyond them tiles of 128 leaves
+    if (!list && nd <= 32 && aligned16(a.n_h) && aligned16(a.a_v) && aligned16(a.shield)) {
+        LeafOctArgs Q;
+        Q.a = a;
+        Q.ntiles = (a.n_oct + 127) / 128;
+        Q.c2 = (float)(-(double)a.shield_k * (double)a.av_per_nh * 1.4426950408889634);
+        Q.pipe_polls = pipe_polls();
+        switch (nd) {
+        case 4: return launch_leaf_oct<4>(Q, s);
+        case 8: return launch_leaf_oct<8>(Q, s);
+        case 12: return launch_leaf_oct<12>(Q, s);
+        case 16: return launch_leaf_oct<16>(Q, s);
+        case 20: return launch_leaf_oct<20>(Q, s);
+        case 24: return launch_leaf_oct<24>(Q, s);
+        case 28: return launch_leaf_oct<28>(Q, s);
+        default: return launch_leaf_oct<32>(Q, s);
+        }
+    }
     LeafTcArgs P;
     P.a = a;
     P.list = list;
@@ -570,10 +831,7 @@ cd_status launch_leaf_tc(const LeafLaunch &a, cudaStream_t s)
     P.c2 = (float)(-(double)a.shield_k * (double)a.av_per_nh * 1.4426950408889634);
     P.out_bulk = a.n_h && aligned16(a.n_h);
     P.form = leaf_form(a, P.out_bulk, list);
-    {
-        const int64_t cap = g_pipe_polls.load();
-        P.pipe_polls = cap < 0 ? kMaxPolls : (uint32_t)std::min<int64_t>(cap, kMaxPolls);
-    }
+    P.pipe_polls = pipe_polls();
     P.span_max = g_span_max.load();
     int dev = 0, smax = 0;
     cudaGetDevice(&dev);
@@ -633,10 +891,7 @@ cd_status launch_leaf_tc_batch(const void *jobs, const int2 *tile_ref, int64_t t
     P.form = form;
     P.list = (form & kFormList) != 0;
     P.out_bulk = (form & kFormBulk) != 0;
-    {
-        const int64_t cap = g_pipe_polls.load();
-        P.pipe_polls = cap < 0 ? kMaxPolls : (uint32_t)std::min<int64_t>(cap, kMaxPolls);
-    }
+    P.pipe_polls = pipe_polls();
     int dev = 0, smax = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&smax, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);

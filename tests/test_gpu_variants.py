@@ -119,3 +119,31 @@ def test_fp32_shell_rows_on_lists_match_uniform(dset):
     want = oracle.Tree.amr(5, 7, BOX, lv["level"], lv["ijk"], lv["rho"]).column_density(geom.dirs, level[rows], ijk[rows])
     got = nh[torch.from_numpy(rows).cuda()].double().cpu().numpy()
     assert np.max(np.abs(got - want) / want) <= 1e-5
+
+
+@pytest.mark.parametrize("dset", [("mxn", 1, 4), ("mxn", 2, 4), ("healpix", 1, 0), ("mxn", 4, 4), ("mxn", 5, 4),
+                                  ("mxn", 4, 6), ("mxn", 4, 7), ("mxn", 8, 4)])
+@pytest.mark.parametrize("L", [3, 4, 6])
+def test_bf16_leaves_of_few_directions(L, dset):
+    # every direction count of the oct form, a tree smaller than its tile and
+    # larger ones, each set of outputs; BF16 tolerances
+    rho = _rho(L, 9)
+    tree = colden.build_tree_uniform(torch.from_numpy(rho).cuda(), BOX)
+    geom = colden.precompute_geometry(*dset)
+    nd = geom.n_dir
+    new = lambda *s: torch.full(s, -1.0, device="cuda")  # noqa: E731
+    nh, av, sh = new(tree.n_leaf, nd), new(tree.n_leaf, nd), new(tree.n_leaf)
+    colden.column_density(tree, geom, n_h=nh, a_v=av, shield=sh, precision=colden.BF16)
+    nh2, av2, sh2 = new(tree.n_leaf, nd), new(tree.n_leaf, nd), new(tree.n_leaf)
+    colden.column_density(tree, geom, n_h=nh2, precision=colden.BF16)
+    colden.column_density(tree, geom, a_v=av2, precision=colden.BF16)
+    colden.column_density(tree, geom, shield=sh2, precision=colden.BF16)
+    colden.device_status()
+    assert torch.equal(nh, nh2) and torch.equal(av, av2) and torch.equal(sh, sh2)
+    rows = np.unique(np.random.default_rng(L).integers(0, tree.n_leaf, 300))
+    want = oracle.Tree.uniform(rho, BOX).column_density(geom.dirs, np.full(len(rows), L), oracle.morton_ijk(L)[rows])
+    at = torch.from_numpy(rows).cuda()
+    got = nh[at].double().cpu().numpy()
+    assert np.max(np.abs(got - want) / want) <= 1e-2
+    assert np.max(np.abs(av[at].double().cpu().numpy() - oracle.a_v(got)) / oracle.a_v(got)) < 1e-6
+    assert np.max(np.abs(sh[at].double().cpu().numpy() - oracle.shield(want))) <= 5e-3
