@@ -138,8 +138,8 @@ struct LevelSums {
     int64_t geom_uid = 0, rho_version = -1;   // what the sums were computed for
     float *C[CD_MAXL + 1] = {};   // shell of level k-2 seen from level-k cells, no prefix, [8^k][ndir]
     float *Et[4] = {};            // oct level, table t alone (shell of level L-t), [n_oct][ndir]
-    float *x = nullptr, *n_tree = nullptr, *delta = nullptr;   // chunk buffers of the FP32 learned path
-    int64_t rows = 0;
+    float *chunk = nullptr;       // chunk buffers of the FP32 learned path
+    int64_t chunk_floats = 0;
 };
 
 // Four entries of a sparse shell row: weights and the byte offsets of the

@@ -86,6 +86,69 @@ __global__ void __launch_bounds__(kThreads) learned_features(FeatArgs A)
     }
 }
 
+// Inputs of the FP32 learned columns for a run of octs: the external slots once
+// per oct, slot 0 and the density per leaf, standardised (mlp.cu,
+// mlp_forward_octs), and the plain columns.  One thread per (oct, direction).
+struct OctFeatArgs {
+    int64_t first, n;               // octs
+    int L, nd;
+    float dx_leaf;
+    const float *rho_leaf;
+    const float *kloc;
+    const float *Et[4];
+    const float *C[CD_MAXL + 1];
+    const float *mu, *sinv;         // [8 nd + 1]
+    float *ue, *ul, *n_tree;        // [n][7 nd], [8 n][nd + 1], [8 n][nd]
+};
+
+__device__ __forceinline__ float standardised_log(float v, float floor, float mu, float sinv)
+{
+    return fminf(fmaxf((logf(fmaxf(v, floor)) - mu) * sinv, -kUMax), kUMax);
+}
+
+__global__ void __launch_bounds__(kThreads) oct_features(const __grid_constant__ OctFeatArgs A)
+{
+    const int nd = A.nd;
+    const int64_t total = A.n * nd;
+    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total;
+         e += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t i = e / nd, oct = A.first + i;
+        const int d = (int)(e - i * nd);
+        float c[kSlots];
+#pragma unroll
+        for (int sl = 0; sl < kSlots; ++sl) c[sl] = 0.f;
+#pragma unroll
+        for (int dl = 1; dl < CD_MAXL; ++dl) {      // dl constant after unrolling
+            if (dl > A.L - 1) break;
+            const float v = dl <= 3 ? A.Et[dl][oct * nd + d] : A.C[A.L - dl + 2][(oct >> (3 * (dl - 3))) * nd + d];
+            c[dl < kSlots ? dl : kSlots - 1] += v;
+        }
+        float ext = 0.f;
+        float *ue = A.ue + i * (kSlots - 1) * nd + d;
+#pragma unroll
+        for (int sl = 1; sl < kSlots; ++sl) {
+            ext += c[sl];
+            ue[(sl - 1) * nd] = standardised_log(c[sl], kCFloor, A.mu[sl * nd + d], A.sinv[sl * nd + d]);
+        }
+        float rho[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) rho[q] = A.rho_leaf[oct * 8 + q];
+        const float mu = A.mu[d], sinv = A.sinv[d];
+#pragma unroll
+        for (int t = 0; t < 8; ++t) {
+            float loc = 0.f;
+#pragma unroll
+            for (int q = 0; q < 8; ++q) loc = fmaf(rho[q], A.kloc[(t * 8 + q) * nd + d], loc);
+            const float c0 = A.dx_leaf * loc;
+            const int64_t row = 8 * i + t;
+            A.n_tree[row * nd + d] = c0 + ext;
+            A.ul[row * (nd + 1) + d] = standardised_log(c0, kCFloor, mu, sinv);
+            if (d == 0)
+                A.ul[row * (nd + 1) + nd] = standardised_log(rho[t], kNFloor, A.mu[kSlots * nd], A.sinv[kSlots * nd]);
+        }
+    }
+}
+
 struct MarchArgs {
     int64_t n, n_leaf;
     const int64_t *leaves;    // [n] leaf of each row, or NULL: row r is leaf r
@@ -564,11 +627,9 @@ void free_level_sums(cd_tree t)
         if (lv.Et[i]) cd::lib_free(lv.Et[i]);
         lv.Et[i] = nullptr;
     }
-    for (float **p : {&lv.x, &lv.n_tree, &lv.delta}) {
-        if (*p) cd::lib_free(*p);
-        *p = nullptr;
-    }
-    lv.rows = 0;
+    if (lv.chunk) cd::lib_free(lv.chunk);
+    lv.chunk = nullptr;
+    lv.chunk_floats = 0;
     lv.ndir = 0;
     lv.geom_uid = 0;
     lv.rho_version = -1;
@@ -593,26 +654,46 @@ cd_status column_density_learned(cd_tree t, cd_geom g, const cd_opts &o, float *
     }
     if ((st = ensure_level_sums(t, g, CD_FP32, s)) != CD_OK) return st;
     LevelSums &lv = t->lv;
-    const int64_t chunk = std::min<int64_t>(kChunkRows, t->n_leaf);
-    if (lv.rows < chunk) {
-        for (float **p : {&lv.x, &lv.n_tree, &lv.delta}) {
-            if (*p) cd::lib_free(*p);
-            *p = nullptr;
-        }
-        lv.rows = 0;
-        if (alloc(&lv.x, (size_t)chunk * net->lay.n_in) != CD_OK || alloc(&lv.n_tree, (size_t)chunk * nd) != CD_OK ||
-            alloc(&lv.delta, (size_t)chunk * nd) != CD_OK)
-            return CD_ENOMEM;
-        lv.rows = chunk;
+    // chunks of whole octs
+    const int64_t chunk = std::min<int64_t>(kChunkRows / 8, t->n_oct), H = net->lay.H;
+    const auto pad = [](int64_t n) { return (n + 63) & ~(int64_t)63; };   // 256-byte sub-buffers
+    const int64_t n_ue = pad(chunk * (kSlots - 1) * nd), n_ul = pad(8 * chunk * (nd + 1)), n_t = pad(8 * chunk * nd),
+                  n_h_ = pad(chunk * H), n_wl = pad(H * (nd + 1)), need = n_ue + n_ul + 2 * n_t + n_h_ + n_wl;
+    if (lv.chunk_floats < need) {
+        if (lv.chunk) cd::lib_free(lv.chunk);
+        lv.chunk = nullptr;
+        lv.chunk_floats = 0;
+        if (alloc(&lv.chunk, (size_t)need) != CD_OK) return CD_ENOMEM;
+        lv.chunk_floats = need;
     }
-    for (int64_t c0 = 0; c0 < t->n_leaf; c0 += chunk) {
-        const int64_t cn = std::min(chunk, t->n_leaf - c0);
-        if ((st = launch_features(t, g, cn, c0, nullptr, lv.x, lv.n_tree, s)) != CD_OK) return st;
-        if ((st = mlp_forward(net, cn, lv.x, lv.delta, s)) != CD_OK) return st;
+    OctFeatArgs A = {};
+    A.L = t->L;
+    A.nd = nd;
+    A.dx_leaf = dx_of(t, t->L);
+    A.rho_leaf = t->rho_leaf;
+    A.kloc = g->kloc;
+    for (int i = 0; i < 4; ++i) A.Et[i] = lv.Et[i];
+    for (int k = 0; k <= CD_MAXL; ++k) A.C[k] = lv.C[k];
+    A.mu = net->mu;
+    A.sinv = net->sinv;
+    A.ue = lv.chunk;
+    A.ul = A.ue + n_ue;
+    A.n_tree = A.ul + n_ul;
+    float *delta = A.n_tree + n_t, *h = delta + n_t, *wl = h + n_h_;
+    for (int64_t c0 = 0; c0 < t->n_oct; c0 += chunk) {
+        A.first = c0;
+        A.n = std::min(chunk, t->n_oct - c0);
+        {
+            LaunchScope ls(CD_K_FEATURES, s);
+            oct_features<<<grid_for(A.n * nd, kThreads), kThreads, 0, s>>>(A);
+            CD_CHECK_LAUNCH();
+        }
+        if ((st = mlp_forward_octs(net, A.n, A.ue, A.ul, h, wl, delta, s)) != CD_OK) return st;
         LaunchScope ls(CD_K_FEATURES, s);
-        learned_combine<<<grid_for(cn * 32, kThreads), kThreads, 0, s>>>(
-            cn, nd, lv.n_tree, lv.delta, net->dlo, net->dhi, (float)o.av_per_nh, (float)o.shield_k, n_h ? n_h + c0 * nd : nullptr,
-            a_v ? a_v + c0 * nd : nullptr, shield ? shield + c0 : nullptr);
+        const int64_t r0 = 8 * c0, rn = 8 * A.n;
+        learned_combine<<<grid_for(rn * 32, kThreads), kThreads, 0, s>>>(
+            rn, nd, A.n_tree, delta, net->dlo, net->dhi, (float)o.av_per_nh, (float)o.shield_k,
+            n_h ? n_h + r0 * nd : nullptr, a_v ? a_v + r0 * nd : nullptr, shield ? shield + r0 : nullptr);
         CD_CHECK_LAUNCH();
     }
     return CD_OK;

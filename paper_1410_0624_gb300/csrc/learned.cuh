@@ -69,6 +69,11 @@ namespace cd {
 // mlp.cu
 // delta [B][nd] of rows 0 .. B-1 of x
 cd_status mlp_forward(cd_net net, int64_t B, const float *x, float *delta, cudaStream_t s);
+// delta of the 8 leaves of each oct from standardised inputs: ue [octs][7 nd] the
+// external slots, ul [8 octs][nd + 1] slot 0 and the density; scratch h [octs][H]
+// and wl [H][nd + 1]
+cd_status mlp_forward_octs(cd_net net, int64_t octs, const float *ue, const float *ul, float *h, float *wl, float *delta,
+                           cudaStream_t s);
 // loss and gradient of the batch (rows NULL: rows 0 .. B-1); either output may be NULL
 cd_status mlp_loss_grad(cd_net net, int64_t B, const float *x, const float *y, const int64_t *rows, float *loss_out,
                         float *grad, cudaStream_t s);

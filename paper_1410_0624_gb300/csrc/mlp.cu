@@ -25,7 +25,7 @@ constexpr int BK = 16, kGemmStages = 3;
 // B, is p[r ld + k] or p[k ld + r]
 enum { OP_N = 0, OP_T = 1 };
 
-enum { EPI_STORE = 0, EPI_BIAS = 1, EPI_BIAS_GELU = 2, EPI_GELU_BWD = 3, EPI_RESIDUAL = 4 };
+enum { EPI_STORE = 0, EPI_BIAS = 1, EPI_BIAS_GELU = 2, EPI_GELU_BWD = 3, EPI_RESIDUAL = 4, EPI_OCT_GELU = 5 };
 
 struct Gemm {
     int M, N, K;
@@ -35,7 +35,7 @@ struct Gemm {
     int64_t ldb;
     float *C;
     int64_t ldc;
-    const float *bias;     // EPI_BIAS, EPI_BIAS_GELU, EPI_RESIDUAL: [N]
+    const float *bias;     // EPI_BIAS, EPI_BIAS_GELU, EPI_RESIDUAL: [N]; EPI_OCT_GELU: [M / 8][ldc], row m / 8
     float *Z;              // EPI_BIAS_GELU: pre-activation out (ldc), may be NULL
     const float *Zin;      // EPI_GELU_BWD: pre-activation (ldc); may alias C
     const float *Y;        // EPI_RESIDUAL: targets [.][N]; C = scale (C - Y[rows])
@@ -192,6 +192,7 @@ __device__ __forceinline__ void gemm_tile(const Gemm &g, int bm, int bn, int z, 
                         zz[q] = v;
                         v = gelu_f(v);
                     }
+                    if (EPI == EPI_OCT_GELU) v = gelu_f(v + g.bias[(int64_t)(m >> 3) * g.ldc + n + q]);
                     if (EPI == EPI_GELU_BWD) v *= gelu_grad_f(g.Zin[o + q]);
                     if (EPI == EPI_RESIDUAL) {
                         const float res = v - g.Y[src * g.N + n + q];
@@ -445,14 +446,17 @@ cd_status grow(T **p, size_t *cap, size_t need)
     return CD_OK;
 }
 
-// activations of `rows` rows; the pre-activations and the backward scratch
-// only for training
-cd_status net_reserve(cd_net net, int64_t rows, bool train)
+// activations of `rows` rows: the two layers' outputs, before them the
+// standardised inputs unless the caller has its own, after them the
+// pre-activations and the backward scratch of training
+enum { kOwnInputs = 1, kTraining = 2 };
+
+cd_status net_reserve(cd_net net, int64_t rows, int what)
 {
     Activations &a = net->act;
     const size_t h = (size_t)net->lay.H, d = (size_t)net->lay.nd, width[7] = {(size_t)net->lay.n_in, h, h, h, h, h, d};
     float **p[7] = {&a.U, &a.A1, &a.A2, &a.Z1, &a.Z2, &a.G, &a.D};
-    for (int i = 0; i < (train ? 7 : 3); ++i) {
+    for (int i = what & kOwnInputs ? 0 : 1; i < (what & kTraining ? 7 : 3); ++i) {
         const cd_status st = grow(p[i], &a.cap[i], rows * width[i]);
         if (st != CD_OK) return st;
     }
@@ -464,7 +468,7 @@ cd_status net_reserve(cd_net net, int64_t rows, bool train)
 cd_status hidden_layers(cd_net net, int64_t B, const float *x, const int64_t *rows, bool train, cudaStream_t s)
 {
     const NetLayout &L = net->lay;
-    cd_status st = net_reserve(net, B, train);
+    cd_status st = net_reserve(net, B, train ? kOwnInputs | kTraining : kOwnInputs);
     if (st != CD_OK) return st;
     Activations &a = net->act;
     const float *P = net->p;
@@ -502,6 +506,49 @@ cd_status mlp_forward(cd_net net, int64_t B, const float *x, float *delta, cudaS
     g.M = (int)B;
     g.N = L.nd; g.K = L.H; g.A = net->act.A2; g.lda = L.H; g.B = net->p + L.W3; g.ldb = L.H;
     g.C = delta; g.ldc = L.nd; g.bias = net->p + L.b3;
+    return run_gemm<OP_N, OP_N, EPI_BIAS>(g, s);
+}
+
+// Wl[h][0 .. nd] = columns 0 .. nd-1 and 8 nd of W1 (slot 0 and the density)
+static __global__ void local_weights(int H, int nd, const float *__restrict__ W1, float *__restrict__ Wl)
+{
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < H * (nd + 1); i += gridDim.x * blockDim.x) {
+        const int h = i / (nd + 1), j = i - h * (nd + 1);
+        Wl[i] = W1[(int64_t)h * (kSlots * nd + 1) + (j < nd ? j : kSlots * nd)];
+    }
+}
+
+// Layer 1 by octs: the seven external slots are the same for an oct's 8 leaves,
+// so their part of z1 (and b1) is one product over the octs and a leaf adds its
+// own nd + 1 inputs: 91 instead of 385 multiply-adds a leaf and unit at 48
+// directions.
+cd_status mlp_forward_octs(cd_net net, int64_t octs, const float *ue, const float *ul, float *h, float *wl, float *delta,
+                           cudaStream_t s)
+{
+    const NetLayout &L = net->lay;
+    cd_status st = net_reserve(net, 8 * octs, 0);
+    if (st != CD_OK) return st;
+    Activations &a = net->act;
+    const float *P = net->p;
+    {
+        LaunchScope ls(CD_K_NET, s);
+        local_weights<<<grid_for((int64_t)L.H * (L.nd + 1), 256), 256, 0, s>>>(L.H, L.nd, P + L.W1, wl);
+        CD_CHECK_LAUNCH();
+    }
+    Gemm g = {};
+    g.M = (int)octs;
+    g.N = L.H; g.K = (kSlots - 1) * L.nd; g.A = ue; g.lda = g.K; g.B = P + L.W1 + L.nd; g.ldb = L.n_in;
+    g.C = h; g.ldc = L.H; g.bias = P + L.b1;
+    if ((st = run_gemm<OP_N, OP_N, EPI_BIAS>(g, s)) != CD_OK) return st;
+    g.M = (int)(8 * octs);
+    g.K = L.nd + 1; g.A = ul; g.lda = g.K; g.B = wl; g.ldb = g.K;
+    g.C = a.A1; g.bias = h;
+    if ((st = run_gemm<OP_N, OP_N, EPI_OCT_GELU>(g, s)) != CD_OK) return st;
+    g.K = L.H; g.A = a.A1; g.lda = L.H; g.B = P + L.W2; g.ldb = L.H;
+    g.C = a.A2; g.bias = P + L.b2;
+    if ((st = run_gemm<OP_N, OP_N, EPI_BIAS_GELU>(g, s)) != CD_OK) return st;
+    g.N = L.nd; g.A = a.A2; g.B = P + L.W3;
+    g.C = delta; g.ldc = L.nd; g.bias = P + L.b3;
     return run_gemm<OP_N, OP_N, EPI_BIAS>(g, s);
 }
 

@@ -147,3 +147,27 @@ def test_bf16_leaves_of_few_directions(L, dset):
     assert np.max(np.abs(got - want) / want) <= 1e-2
     assert np.max(np.abs(av[at].double().cpu().numpy() - oracle.a_v(got)) / oracle.a_v(got)) < 1e-6
     assert np.max(np.abs(sh[at].double().cpu().numpy() - oracle.shield(want))) <= 5e-3
+
+
+@pytest.mark.parametrize("L,dset,H", [(1, ("healpix", 1, 0), 16), (2, ("axes", 0, 0), 33), (4, ("mxn", 5, 3), 64),
+                                      (5, ("healpix", 2, 0), 128), (6, ("mxn", 7, 12), 40)])
+def test_fp32_learned_columns_by_octs(L, dset, H):
+    # the learned columns (layer 1 by octs) against features and network row by
+    # row; the two differ by the order of FP32 sums: 1e-5 on a correction of
+    # order one, 2e-5 relative on the column
+    rho = _rho(L, 21)
+    tree = colden.build_tree_uniform(torch.from_numpy(rho).cuda(), BOX)
+    geom = colden.precompute_geometry(*dset)
+    nd = geom.n_dir
+    net = colden.Net(nd, H, synth.mlp_init(nd, H, 5, out_scale=0.3))
+    x = torch.empty((tree.n_leaf, 8 * nd + 1), device="cuda")
+    nt, delta = torch.empty((tree.n_leaf, nd), device="cuda"), torch.empty((tree.n_leaf, nd), device="cuda")
+    colden.learned_features(tree, geom, x, nt)
+    net.fit_normaliser(x)
+    net.forward(x, delta)
+    nh, av, sh = torch.empty_like(nt), torch.empty_like(nt), torch.empty(tree.n_leaf, device="cuda")
+    colden.column_density(tree, geom, n_h=nh, a_v=av, shield=sh, net=net)
+    want = nt.double() * torch.exp(delta.double())
+    assert float(((nh.double() - want).abs() / want).max()) < 2e-5
+    assert float(((av.double() - want / 1.87e21).abs() / (want / 1.87e21)).max()) < 2e-5
+    assert float((sh.double() - torch.exp(-2.5 * want / 1.87e21).mean(1)).abs().max()) < 1e-5
