@@ -127,6 +127,7 @@ __global__ void __launch_bounds__(kExtThreads) shell_sum_fp32(ExtArgs P)
 // instructions an output row, entries read by every warp), the entries from L1
 // instead of the ring 0.68 (their latency).
 constexpr int kRowThreads = 512, kRowPitch = 36, kRowCells = CD_STENCIL, kRingQuads = 4;
+constexpr int kRowMinEntries = 48;   // directions x longest row
 
 struct RowArgs {
     int k, nd;
@@ -265,13 +266,7 @@ __global__ void __launch_bounds__(kRowThreads, 2) shell_rows_fp32(const __grid_c
     const char *Xl = reinterpret_cast<const char *>(X + 4 * (lane & 7));
     float acc[4] = {0.f, 0.f, 0.f, 0.f};                              // direction 4 quad + g of parents 4 (lane & 7) ..
     int d = 4 * qa;
-    const auto add = [&](int off, float w) {
-        const float4 x = *reinterpret_cast<const float4 *>(Xl + off);
-        acc[0] = fmaf(x.x, w, acc[0]);
-        acc[1] = fmaf(x.y, w, acc[1]);
-        acc[2] = fmaf(x.z, w, acc[2]);
-        acc[3] = fmaf(x.w, w, acc[3]);
-    };
+    const auto cells = [&](int off) { return *reinterpret_cast<const float4 *>(Xl + off); };
     for (int blk = 0; blk * kRingQuads < n; ++blk) {
         asm volatile("cp.async.wait_group 1;" ::: "memory");
         __syncwarp();
@@ -283,10 +278,12 @@ __global__ void __launch_bounds__(kRowThreads, 2) shell_rows_fp32(const __grid_c
             const int ow = v.off.w & ~1;                              // bit 0: the quad's last chunk
             if (in_bounds(max(max(v.off.x, v.off.y), max(v.off.z, ow)), (A.nt * kRowCells + 1) * kRowPitch * 4,
                           kCheckFp32Region)) {
-                add(v.off.x, v.w.x);
-                add(v.off.y, v.w.y);
-                add(v.off.z, v.w.z);
-                add(ow, v.w.w);
+                // four entries at a time: rows of a cone have forty
+                const float4 x0 = cells(v.off.x), x1 = cells(v.off.y), x2 = cells(v.off.z), x3 = cells(ow);
+                acc[0] += fmaf(x3.x, v.w.w, fmaf(x2.x, v.w.z, fmaf(x1.x, v.w.y, x0.x * v.w.x)));
+                acc[1] += fmaf(x3.y, v.w.w, fmaf(x2.y, v.w.z, fmaf(x1.y, v.w.y, x0.y * v.w.x)));
+                acc[2] += fmaf(x3.z, v.w.w, fmaf(x2.z, v.w.z, fmaf(x1.z, v.w.y, x0.z * v.w.x)));
+                acc[3] += fmaf(x3.w, v.w.w, fmaf(x2.w, v.w.z, fmaf(x1.w, v.w.y, x0.w * v.w.x)));
             }
             if (!(v.off.w & 1)) continue;
             // exchange: lane g of a group of four parents gets its parent's four directions
@@ -446,8 +443,11 @@ cd_status launch_rows(const ExtLaunch &a, cd_geom g, cudaStream_t s)
 
 bool ext_fp32_serves_list(int k, int tmask, cd_geom g)
 {
+    // with hardly anything to sum (the six axis rays have three entries at most)
+    // staging a parent's stencils costs more than the block form's gathers
+    // (64^3: 24.6 against 23.1 us; 12 HEALPix directions 24.4 against 28.7)
     const int li = row_list(tmask);
-    return k >= 4 && li >= 0 && g->rows[li].quad != nullptr;
+    return k >= 4 && li >= 0 && g->rows[li].quad != nullptr && g->n_dir * g->maxe >= kRowMinEntries;
 }
 
 cd_status build_row_lists(cd_geom g, cudaStream_t s)
@@ -479,6 +479,10 @@ cd_status build_row_lists(cd_geom g, cudaStream_t s)
 cd_status launch_ext_fp32(const ExtLaunch &a, cd_geom g, cudaStream_t s)
 {
     if (ext_fp32_serves_list(a.k, a.tmask, g)) return launch_rows(a, g, s);
+    if (a.list) {
+        set_error("the FP32 block form serves whole levels only");
+        return CD_EUNSUPPORTED;
+    }
     ExtArgs P;
     P.a = a;
     // largest span <= min(3, k) that still gives >= 304 CTAs (2 per SM)

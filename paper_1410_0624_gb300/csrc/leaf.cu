@@ -16,8 +16,9 @@
 //     stores, so HBM sees full-line writes;
 //   - the direction sum of the screening factor goes through a shared-memory
 //     partial array (no atomics).
-// A generic one-thread-per-leaf kernel covers direction counts that are not a
-// multiple of four and unaligned output pointers.
+// Direction counts that are not a multiple of four and unaligned output pointers
+// go to a kernel of one warp per child of 32 octs, or with very few or very many
+// of them to a generic one-thread-per-leaf kernel.
 #include <algorithm>
 #include <mutex>
 
@@ -277,6 +278,96 @@ __global__ void __launch_bounds__(256) leaf_generic(LeafLaunch P, float c_exp, f
     }
 }
 
+// Direction counts that are not a multiple of four, and unaligned outputs: a
+// CTA takes 32 octs, a warp one of their children and a lane one oct, which
+// walks the directions.  The local weights are then the same for a warp (two
+// 16-byte broadcasts for eight FMAs), the oct's densities stay in registers, the
+// external columns E + Sp come from shared memory (odd pitch: no bank
+// conflicts), and 32 directions of the 32 octs at a time turn into coalesced row
+// pieces through a padded square.
+// What bounds it: shared memory, about eight wavefronts per 32 outputs.  An FP32
+// evaluation of 256^3 at 35 directions took 6.20 ms with a thread a leaf (32 rows
+// a store) and takes 1.83, at 81 directions 14.6 and 4.7, of 64^3 at 9
+// directions 32 and 25 us.
+constexpr int kOctWarps = 8;   // one per child
+
+__host__ __device__ constexpr int oct_pitch(int nd) { return nd | 1; }
+
+size_t leaf_oct_smem(int nd, bool rows)
+{
+    return sizeof(float) * (64 * (size_t)nd + (size_t)32 * oct_pitch(nd) + (rows ? kOctWarps * 32 * 33 : 0));
+}
+
+template <bool kRows>
+__global__ void __launch_bounds__(32 * kOctWarps) leaf_oct_fp32(LeafLaunch P, float c_exp, float inv_nd)
+{
+    extern __shared__ __align__(16) float sm[];
+    const int nd = P.nd, pitch = oct_pitch(nd);
+    const int t = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    float *sK = sm;                                                        // [8 t][nd][8 s], times dx
+    float *sE = sK + 64 * nd;                                              // [32 octs][pitch]
+    float *T = sE + 32 * pitch + t * 32 * 33;                              // [32 octs][33]
+    for (int i = threadIdx.x; i < 64 * nd; i += blockDim.x) {
+        const int d = i % nd, ts = i / nd;                                 // kloc[t][s][d]
+        sK[((ts >> 3) * nd + d) * 8 + (ts & 7)] = P.dx_leaf * P.kloc[i];
+    }
+    const int64_t tiles = (P.n_oct + 31) / 32;
+    for (int64_t tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
+        const int64_t o0 = tile * 32, oct = o0 + lane;
+        const int nb = (int)(P.n_oct - o0 < 32 ? P.n_oct - o0 : 32);
+        if (!in_bounds(o0 + nb - 1, P.n_oct, kCheckLeafIn)) break;
+        const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
+        const float4 r0 = lane < nb ? *reinterpret_cast<const float4 *>(P.rho_leaf + oct * 8) : z;
+        const float4 r1 = lane < nb ? *reinterpret_cast<const float4 *>(P.rho_leaf + oct * 8 + 4) : z;
+        for (int i = threadIdx.x; i < nb * nd; i += blockDim.x) {
+            const int o = i / nd, d = i - o * nd;
+            float e = P.E ? P.E[o0 * nd + i] : 0.f;
+            if (P.Sp) e += P.Sp[((o0 + o) >> 3) * nd + d];
+            sE[o * pitch + d] = e;
+        }
+        __syncthreads();
+        const float *E = sE + lane * pitch, *K = sK + t * nd * 8;
+        float acc = 0.f;
+        for (int d0 = 0; d0 < nd; d0 += 32) {
+            const int w = min(32, nd - d0);
+#pragma unroll 4
+            for (int j = 0; j < w; ++j) {
+                const float4 k0 = *reinterpret_cast<const float4 *>(K + (d0 + j) * 8),
+                             k1 = *reinterpret_cast<const float4 *>(K + (d0 + j) * 8 + 4);
+                float v = E[d0 + j];
+                v = fmaf(r0.x, k0.x, v);
+                v = fmaf(r0.y, k0.y, v);
+                v = fmaf(r0.z, k0.z, v);
+                v = fmaf(r0.w, k0.w, v);
+                v = fmaf(r1.x, k1.x, v);
+                v = fmaf(r1.y, k1.y, v);
+                v = fmaf(r1.z, k1.z, v);
+                v = fmaf(r1.w, k1.w, v);
+                if (kRows) T[lane * 33 + j] = v;
+                acc += __expf(c_exp * v);
+            }
+            if (!kRows) continue;
+            __syncwarp();
+            if (lane < w) {
+                const int64_t at = (o0 * 8 + t) * nd + d0 + lane;
+                if (P.n_h) {
+                    float *out = P.n_h + at;
+#pragma unroll 8
+                    for (int o = 0; o < nb; ++o) out[(int64_t)o * 8 * nd] = T[o * 33 + lane];
+                }
+                if (P.a_v) {
+                    float *out = P.a_v + at;
+#pragma unroll 8
+                    for (int o = 0; o < nb; ++o) out[(int64_t)o * 8 * nd] = T[o * 33 + lane] * P.av_per_nh;
+                }
+            }
+            __syncwarp();
+        }
+        if (P.shield && lane < nb) P.shield[oct * 8 + t] = acc * inv_nd;
+        __syncthreads();   // every warp is done with the external columns
+    }
+}
+
 struct DevInfo {
     int sms = 0;
 };
@@ -330,6 +421,22 @@ cd_status launch_leaf(const LeafLaunch &a, cudaStream_t s)
         const int64_t grid = std::min<int64_t>(P.nbatch, (int64_t)per_sm * sm_count());
         LaunchScope ls(CD_K_LEAF, s);
         kern<<<(unsigned)grid, threads, smem, s>>>(P);
+        CD_CHECK_LAUNCH();
+        return CD_OK;
+    }
+    const bool rows = a.n_h || a.a_v;
+    // hardly any directions leave a warp too little to do per tile: up to 4 at any
+    // size (256^3 at 3 directions 0.39 against 0.26 ms), up to 8 on trees below 32^3
+    // (16^3 at 6: 12.3 against 10.4 us)
+    if (nd >= (a.n_oct >= 4096 ? 5 : 9) && leaf_oct_smem(nd, rows) <= 200 * 1024 && aligned16(a.rho_leaf)) {
+        const auto kern = rows ? leaf_oct_fp32<true> : leaf_oct_fp32<false>;
+        const size_t smem = leaf_oct_smem(nd, rows);
+        CD_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        int per_sm = 0;
+        CD_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 32 * kOctWarps, smem));
+        const int64_t grid = std::min<int64_t>((a.n_oct + 31) / 32, (int64_t)sm_count() * std::max(1, per_sm));
+        LaunchScope ls(CD_K_LEAF, s);
+        kern<<<(unsigned)std::max<int64_t>(grid, 1), 32 * kOctWarps, smem, s>>>(a, c_exp, inv_nd);
         CD_CHECK_LAUNCH();
         return CD_OK;
     }

@@ -171,3 +171,31 @@ def test_fp32_learned_columns_by_octs(L, dset, H):
     assert float(((nh.double() - want).abs() / want).max()) < 2e-5
     assert float(((av.double() - want / 1.87e21).abs() / (want / 1.87e21)).max()) < 2e-5
     assert float((sh.double() - torch.exp(-2.5 * want / 1.87e21).mean(1)).abs().max()) < 1e-5
+
+
+@pytest.mark.parametrize("L,dset,shift", [(1, ("mxn", 5, 7), 0), (2, ("mxn", 3, 3), 0), (4, ("mxn", 11, 3), 0),
+                                          (5, ("axes", 0, 0), 0), (5, ("mxn", 5, 1), 0), (5, ("mxn", 13, 5), 0),
+                                          (4, ("healpix", 2, 0), 1), (6, ("mxn", 3, 4), 2), (3, ("mxn", 127, 1), 0),
+                                          (2, ("mxn", 97, 5), 0), (5, ("mxn", 2, 2), 3)])
+def test_fp32_leaves_of_any_direction_count_and_alignment(L, dset, shift):
+    # counts that are no multiple of four, outputs off the 16-byte boundary, and
+    # both sides of the rule's lines; FP32 tolerances on every leaf
+    rho = _rho(L, 31)
+    tree = colden.build_tree_uniform(torch.from_numpy(rho).cuda(), BOX)
+    geom = colden.precompute_geometry(*dset)
+    nd, n = geom.n_dir, tree.n_leaf
+    buf = torch.full((2 * n * nd + n + 64,), -1.0, device="cuda")
+    nh = buf[shift:shift + n * nd]
+    av = buf[n * nd + 2 * shift:][:n * nd]
+    sh = torch.full((n + 8,), -1.0, device="cuda")[shift:shift + n]
+    colden.column_density(tree, geom, n_h=nh, a_v=av, shield=sh)
+    only = torch.full((n + 8,), -1.0, device="cuda")[shift:shift + n]
+    colden.column_density(tree, geom, shield=only)
+    assert torch.equal(sh, only)
+    rows = np.arange(n) if n <= 4096 else np.unique(np.random.default_rng(L).integers(0, n, 2000))
+    want = oracle.Tree.uniform(rho, BOX).column_density(geom.dirs, np.full(len(rows), L), oracle.morton_ijk(L)[rows])
+    at = torch.from_numpy(rows).cuda()
+    got = nh.reshape(n, nd)[at].double().cpu().numpy()
+    assert np.max(np.abs(got - want) / want) <= 1e-5
+    assert np.max(np.abs(av.reshape(n, nd)[at].double().cpu().numpy() - oracle.a_v(got)) / oracle.a_v(got)) < 1e-6
+    assert np.max(np.abs(sh[at].double().cpu().numpy() - oracle.shield(want))) <= 1e-5
