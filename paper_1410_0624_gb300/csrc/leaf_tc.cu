@@ -62,7 +62,8 @@ struct LeafTcArgs {
 
 // what a leaf row reads and writes: the parent prefix, staged rows (bulk
 // stores) or direct n_h rows, A_V, the screening factor, list tiles
-constexpr int kFormSp = 1, kFormBulk = 2, kFormNh = 4, kFormAv = 8, kFormShield = 16, kFormList = 32;
+constexpr int kFormSp = 1, kFormBulk = 2, kFormNh = 4, kFormAv = 8, kFormShield = 16, kFormList = 32,
+              kFormAvRows = 64;   // A_V alone: its rows are the staged ones, n_h points at a_v
 
 __host__ __device__ inline int leaf_form(const LeafLaunch &a, bool out_bulk, bool list)
 {
@@ -186,12 +187,12 @@ __device__ __forceinline__ T ldg_copy(const T *p)
 }
 
 // One leaf row of a tile: N_H[d] = loc[d] (x dx when kScale) + E[d] (+ Sp[d]),
-// written to the staging row (kOut 1) or straight to n_h (kOut 2, rows with
-// ok only), optionally A_V = N_H av_per_nh; returns sum_d 2^(c2 N_H[d]).  All
-// 32 lanes of a warp take the same instance (the form is a launch constant).
-template <bool kSp, int kOut, bool kAv, bool kScale>
+// written to the staging row (kOut & 1; as A_V with kOut & 4) and / or straight
+// to n_h (kOut & 2, rows with ok only); returns sum_d 2^(c2 N_H[d]).  All 32 lanes of a warp take the
+// same instance (the form is a launch constant).
+template <bool kSp, int kOut, bool kScale>
 __device__ __forceinline__ float leaf_rows(uint32_t taddr, int nd, const float *Ei, const float *Pi, float *orow,
-                                           float *nh, float *av, bool ok, float c2, float avk, float dxs)
+                                           float *nh, bool ok, float c2, float dxs, float avk)
 {
     float acc = 0.f;
 #pragma unroll 1
@@ -219,18 +220,15 @@ __device__ __forceinline__ float leaf_rows(uint32_t taddr, int nd, const float *
                                 __uint_as_float(v[j4 + 2]) + e.z, __uint_as_float(v[j4 + 3]) + e.w);
             }
             acc += (fast_exp2(c2 * N.x) + fast_exp2(c2 * N.y)) + (fast_exp2(c2 * N.z) + fast_exp2(c2 * N.w));
-            if (kOut == 1) *reinterpret_cast<float4 *>(orow + c + j4) = N;
-            if (kOut == 2 && ok) {
+            if (kOut & 4)
+                *reinterpret_cast<float4 *>(orow + c + j4) = make_float4(N.x * avk, N.y * avk, N.z * avk, N.w * avk);
+            else if (kOut & 1)
+                *reinterpret_cast<float4 *>(orow + c + j4) = N;
+            if ((kOut & 2) && ok) {
                 nh[c + j4] = N.x;
                 nh[c + j4 + 1] = N.y;
                 nh[c + j4 + 2] = N.z;
                 nh[c + j4 + 3] = N.w;
-            }
-            if (kAv && ok) {
-                av[c + j4] = N.x * avk;
-                av[c + j4 + 1] = N.y * avk;
-                av[c + j4 + 2] = N.z * avk;
-                av[c + j4 + 3] = N.w * avk;
             }
         }
     }
@@ -430,6 +428,7 @@ __global__ void __launch_bounds__(512, 1) leaf_tc(LeafTcArgs P0, LeafBatch Bt)
         const int32_t *sL = reinterpret_cast<const int32_t *>(st + S.st_l);
         const int nb = tile_octs(P, tile, lst);
         const float dxs = kMode == 2 ? P.a.dx_leaf : 1.f;   // batched: Kloc in units of dx
+        int av_row = -1;                                     // this thread's output row
         {
             // output row of this leaf: Morton position, or the list's row (-1: none)
             const int64_t m = lst ? ((i >> 3) < nb ? (int64_t)sL[i] : -1) : tile * 128 + i;
@@ -447,29 +446,29 @@ __global__ void __launch_bounds__(512, 1) leaf_tc(LeafTcArgs P0, LeafBatch Bt)
             float *orow = sO + (size_t)i * nd;
             const float c2 = P.c2, avk = P.a.av_per_nh;
             // the output form is a launch constant (kernel parameter): pick the
-            // loop once, outside the per-direction work
+            // loop once, outside the per-direction work.  A_V rows are staged too
+            // and leave after the tile's last barrier
             const int fm = P0.form;
-            float *av = (fm & kFormAv) ? P.a.a_v + mr * nd : nullptr;
             float *nh = (fm & kFormNh) ? P.a.n_h + mr * nd : nullptr;
             float *shp = (fm & kFormShield) ? P.a.shield + mr : nullptr;
-            const int form = fm & (kFormSp | kFormBulk | kFormNh | kFormAv);
+            const int form = (fm & kFormSp ? 1 : 0) |
+                             (fm & kFormAvRows ? 8 : (fm & (kFormBulk | kFormAv) ? 2 : 0) | (fm & kFormNh ? 4 : 0));
             const uint32_t taddr = tD + lane_off;
             float acc;
             __syncwarp();
             switch (form) {
-            case 0: acc = leaf_rows<false, 0, false, kMode == 2>(taddr, nd, Ei, Pi, orow, nh, av, ok, c2, avk, dxs); break;
-            case 1: acc = leaf_rows<true, 0, false, kMode == 2>(taddr, nd, Ei, Pi, orow, nh, av, ok, c2, avk, dxs); break;
-            case 2: acc = leaf_rows<false, 1, false, kMode == 2>(taddr, nd, Ei, Pi, orow, nh, av, ok, c2, avk, dxs); break;
-            case 3: acc = leaf_rows<true, 1, false, kMode == 2>(taddr, nd, Ei, Pi, orow, nh, av, ok, c2, avk, dxs); break;
-            case 4: acc = leaf_rows<false, 2, false, kMode == 2>(taddr, nd, Ei, Pi, orow, nh, av, ok, c2, avk, dxs); break;
-            case 5: acc = leaf_rows<true, 2, false, kMode == 2>(taddr, nd, Ei, Pi, orow, nh, av, ok, c2, avk, dxs); break;
-            case 8: acc = leaf_rows<false, 0, true, kMode == 2>(taddr, nd, Ei, Pi, orow, nh, av, ok, c2, avk, dxs); break;
-            case 9: acc = leaf_rows<true, 0, true, kMode == 2>(taddr, nd, Ei, Pi, orow, nh, av, ok, c2, avk, dxs); break;
-            case 10: acc = leaf_rows<false, 1, true, kMode == 2>(taddr, nd, Ei, Pi, orow, nh, av, ok, c2, avk, dxs); break;
-            case 11: acc = leaf_rows<true, 1, true, kMode == 2>(taddr, nd, Ei, Pi, orow, nh, av, ok, c2, avk, dxs); break;
-            case 12: acc = leaf_rows<false, 2, true, kMode == 2>(taddr, nd, Ei, Pi, orow, nh, av, ok, c2, avk, dxs); break;
-            default: acc = leaf_rows<true, 2, true, kMode == 2>(taddr, nd, Ei, Pi, orow, nh, av, ok, c2, avk, dxs); break;
+            case 0: acc = leaf_rows<false, 0, kMode == 2>(taddr, nd, Ei, Pi, orow, nh, ok, c2, dxs, avk); break;
+            case 1: acc = leaf_rows<true, 0, kMode == 2>(taddr, nd, Ei, Pi, orow, nh, ok, c2, dxs, avk); break;
+            case 2: acc = leaf_rows<false, 1, kMode == 2>(taddr, nd, Ei, Pi, orow, nh, ok, c2, dxs, avk); break;
+            case 3: acc = leaf_rows<true, 1, kMode == 2>(taddr, nd, Ei, Pi, orow, nh, ok, c2, dxs, avk); break;
+            case 4: acc = leaf_rows<false, 2, kMode == 2>(taddr, nd, Ei, Pi, orow, nh, ok, c2, dxs, avk); break;
+            case 5: acc = leaf_rows<true, 2, kMode == 2>(taddr, nd, Ei, Pi, orow, nh, ok, c2, dxs, avk); break;
+            case 6: acc = leaf_rows<false, 3, kMode == 2>(taddr, nd, Ei, Pi, orow, nh, ok, c2, dxs, avk); break;
+            case 7: acc = leaf_rows<true, 3, kMode == 2>(taddr, nd, Ei, Pi, orow, nh, ok, c2, dxs, avk); break;
+            case 8: acc = leaf_rows<false, 5, kMode == 2>(taddr, nd, Ei, Pi, orow, nh, ok, c2, dxs, avk); break;
+            default: acc = leaf_rows<true, 5, kMode == 2>(taddr, nd, Ei, Pi, orow, nh, ok, c2, dxs, avk); break;
             }
+            av_row = ok ? (int)m : -1;
             if ((fm & kFormShield) && ok) *shp = acc / (float)nd;
         }
         // list tiles: do the tile's leaf rows form one run (row of leaf i = row of leaf 0 + i)?
@@ -492,6 +491,28 @@ __global__ void __launch_bounds__(512, 1) leaf_tc(LeafTcArgs P0, LeafBatch Bt)
         fence_proxy_async_smem();
         tc_fence_before();
         named_barrier(bid, 128);
+        if (P0.form & kFormAv) {
+            // A_V from the staged rows, each warp its own 32, 16 bytes a lane: whole
+            // lines of consecutive rows (scalar where a_v is off the boundary)
+            const float k = P.a.av_per_nh;
+            const int nq = nd >> 2;
+            const bool vec = ((uintptr_t)P.a.a_v & 15) == 0;
+            const float *rows = sO + (size_t)quarter * 32 * nd;
+            for (int e = i & 31; e < 32 * nq; e += 32) {
+                const int r = e / nq, row = __shfl_sync(0xffffffffu, av_row, r);
+                if (row < 0) continue;
+                const float4 N = *reinterpret_cast<const float4 *>(rows + 4 * e);
+                float *av = P.a.a_v + (int64_t)row * nd + 4 * (e - r * nq);
+                if (vec) {
+                    *reinterpret_cast<float4 *>(av) = make_float4(N.x * k, N.y * k, N.z * k, N.w * k);
+                } else {
+                    av[0] = N.x * k;
+                    av[1] = N.y * k;
+                    av[2] = N.z * k;
+                    av[3] = N.w * k;
+                }
+            }
+        }
         if (P0.out_bulk && !lst && i == 0 && in_bounds(tile * 128 + 127, 8 * P.a.n_oct, kCheckLeafTcOut)) {
             bulk_s2g(P.a.n_h + tile * 128 * nd, sO, (uint32_t)(128 * nd * 4));
             bulk_commit();
@@ -537,14 +558,15 @@ __global__ void __launch_bounds__(512, 1) leaf_tc(LeafTcArgs P0, LeafBatch Bt)
     }
 }
 
-// ---- few directions: octs as rows ------------------------------------------------
+// ---- few directions, or the screening factor alone: octs as rows -----------------
 //
 // Up to 32 directions the tile above is mostly latency: 128 leaves of 12
 // directions are 1 536 sums behind three barriers and a product.  Here a row of
 // the product is an oct: D[oct][t nd + d] = sum_s rho[oct][s] (dx_L Kloc[t][s][d])
-// has M = 128 octs, N = 8 nd columns (at most 256) and K = 16 (its 8 siblings and
-// 8 zeros; the same BF16 operands as above), so that one product and one round
-// of barriers serve 1 024 leaves.  A thread has one oct: its external column
+// has M = 128 octs, N = 8 nd columns (at most 256; beyond 32 directions two
+// products of four children) and K = 16 (its 8 siblings and 8 zeros; the same
+// BF16 operands as above), so that one product and one round of barriers serve
+// 1 024 leaves.  A thread has one oct: its external column
 // E + Sp stays in registers for the 8 children, and their screening factors are
 // 32 contiguous bytes.
 // N_H and A_V rows leave through a per-warp transpose, 128 bytes of a row at a
@@ -565,7 +587,10 @@ struct LeafOctArgs {
 template <int ND>
 struct LeafOctShape {
     static constexpr int N = 8 * ND;
-    static constexpr int kCols = N <= 64 ? 64 : N <= 128 ? 128 : 256;   // TMEM columns of a group
+    static constexpr int kParts = N > 256 ? 2 : 1;                       // products a tile: all children, or four
+    static constexpr int kN = N / kParts;
+    static_assert(kN % 32 == 0, "a product is drained 32 columns at a time");
+    static constexpr int kCols = kN <= 64 ? 64 : kN <= 128 ? 128 : 256;  // TMEM columns of a group
     static constexpr int kGroups = 512 / kCols > 4 ? 4 : 512 / kCols;
     static constexpr uint32_t kB = N * 32, kA = 4096;                    // operand bytes (K = 16)
     static constexpr uint32_t kE = 128 * ND * 4, kP = 16 * ND * 4, kStage = kE + kP + 4096;
@@ -677,20 +702,6 @@ __global__ void __launch_bounds__(128 * LeafOctShape<ND>::kGroups, 1) leaf_oct_t
         fence_proxy_async_smem();
         tc_fence_before();
         named_barrier(1 + g, 128);
-        if (i == 0) {
-            tc_fence_after();
-            umma_bf16(tD, umma_smem_desc(smem_u32(sA), 128, 256), umma_smem_desc(smem_u32(smem), 128, 256),
-                      umma_idesc_bf16(128, S::N), 0u);
-            umma_commit(&bar[g]);
-            if (!mbar_wait_bounded(&bar[g], phase, P.pipe_polls)) sflag[g] = 1;
-        }
-        phase ^= 1;
-        named_barrier(1 + g, 128);
-        if (sflag[g]) {
-            fault = true;
-            break;
-        }
-        tc_fence_after();
         const int64_t oct = tile * 128 + i;
         const bool ok = oct < n_oct && in_bounds(oct, n_oct, kCheckLeafTcOut);
         // rows: 32 columns of the warp's 32 octs at a time turn into 128-byte
@@ -703,9 +714,31 @@ __global__ void __launch_bounds__(128 * LeafOctShape<ND>::kGroups, 1) leaf_oct_t
         for (int t = 0; t < 8; ++t) acc[t] = 0.f;
 #pragma unroll
         for (int c = 0; c < S::N; c += 32) {
+            if (c % S::kN == 0) {
+                // the product of the next children (the accumulator is drained: the tile's
+                // operands, or the part before, are behind this barrier)
+                if (c) {
+                    tc_fence_before();
+                    named_barrier(1 + g, 128);
+                }
+                if (i == 0) {
+                    tc_fence_after();
+                    umma_bf16(tD, umma_smem_desc(smem_u32(sA), 128, 256), umma_smem_desc(smem_u32(smem) + c * 32, 128, 256),
+                              umma_idesc_bf16(128, S::kN), 0u);
+                    umma_commit(&bar[g]);
+                    if (!mbar_wait_bounded(&bar[g], phase, P.pipe_polls)) sflag[g] = 1;
+                }
+                phase ^= 1;
+                named_barrier(1 + g, 128);
+                if (sflag[g]) {
+                    fault = true;
+                    break;
+                }
+                tc_fence_after();
+            }
             uint32_t v[32];
             __syncwarp();
-            tmem_ld32(taddr + (uint32_t)c, v);
+            tmem_ld32(taddr + (uint32_t)(c % S::kN), v);
             tmem_ld_wait();
 #pragma unroll
             for (int j = 0; j < 32; j += 4) {
@@ -729,6 +762,7 @@ __global__ void __launch_bounds__(128 * LeafOctShape<ND>::kGroups, 1) leaf_oct_t
                 }
             }
         }
+        if (fault) break;
         if (P.a.shield && ok) {
             float4 *sh = reinterpret_cast<float4 *>(P.a.shield + oct * 8);
             const float n = (float)ND;
@@ -770,8 +804,10 @@ cd_status launch_leaf_oct(const LeafOctArgs &P, cudaStream_t s)
     // as many groups a CTA as leave every SM one (a small tree's tiles go to more SMs)
     int G = S::kGroups;
     while (G > 1 && (P.ntiles + G - 1) / G < sms()) --G;
-    const auto kern = P.a.n_h || P.a.a_v ? leaf_oct_tc<ND, true> : leaf_oct_tc<ND, false>;
     const bool rows = P.a.n_h || P.a.a_v;
+    auto kern = leaf_oct_tc<ND, false>;
+    if constexpr (S::kParts == 1)
+        if (rows) kern = leaf_oct_tc<ND, true>;
     const size_t smem = S::smem(G, rows);
     CD_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::smem(S::kGroups, rows)));
     const int64_t grid = std::min<int64_t>((P.ntiles + G - 1) / G, sms());
@@ -804,23 +840,22 @@ cd_status launch_leaf_tc(const LeafLaunch &a, cudaStream_t s)
     if (n_leaf == 0) return CD_OK;
     // 8 n_dir columns fit one product up to 32 directions; from 128 leaves to 256^3
     // the oct form is the faster one there (8.0 against 8.2 us at 16^3, 12.0 against
-    // 14.5 at 64^3, 12 directions), beyond them tiles of 128 leaves
-    if (!list && nd <= 32 && aligned16(a.n_h) && aligned16(a.a_v) && aligned16(a.shield)) {
+    // 14.5 at 64^3, 12 directions).  Beyond them it takes two products (of a
+    // multiple of 32 columns each) and only calls that want the screening factor
+    // alone (256^3, 48 directions: 0.249 against 0.456 ms); N_H rows are bound by
+    // their stores, which tiles of 128 leaves send as bulk copies
+    if (!list && (nd <= 32 || (nd % 8 == 0 && !a.n_h && !a.a_v)) && aligned16(a.n_h) && aligned16(a.a_v) && aligned16(a.shield)) {
         LeafOctArgs Q;
         Q.a = a;
         Q.ntiles = (a.n_oct + 127) / 128;
         Q.c2 = (float)(-(double)a.shield_k * (double)a.av_per_nh * 1.4426950408889634);
         Q.pipe_polls = pipe_polls();
-        switch (nd) {
-        case 4: return launch_leaf_oct<4>(Q, s);
-        case 8: return launch_leaf_oct<8>(Q, s);
-        case 12: return launch_leaf_oct<12>(Q, s);
-        case 16: return launch_leaf_oct<16>(Q, s);
-        case 20: return launch_leaf_oct<20>(Q, s);
-        case 24: return launch_leaf_oct<24>(Q, s);
-        case 28: return launch_leaf_oct<28>(Q, s);
-        default: return launch_leaf_oct<32>(Q, s);
-        }
+        using Launch = cd_status (*)(const LeafOctArgs &, cudaStream_t);
+        static constexpr Launch kLaunch[16] = {
+            launch_leaf_oct<4>, launch_leaf_oct<8>, launch_leaf_oct<12>, launch_leaf_oct<16>, launch_leaf_oct<20>,
+            launch_leaf_oct<24>, launch_leaf_oct<28>, launch_leaf_oct<32>, nullptr, launch_leaf_oct<40>,
+            nullptr, launch_leaf_oct<48>, nullptr, launch_leaf_oct<56>, nullptr, launch_leaf_oct<64>};
+        return kLaunch[nd / 4 - 1](Q, s);
     }
     LeafTcArgs P;
     P.a = a;
@@ -829,8 +864,16 @@ cd_status launch_leaf_tc(const LeafLaunch &a, cudaStream_t s)
     P.n_leaf = n_leaf;
     P.ntiles = (a.n_oct + 15) / 16;
     P.c2 = (float)(-(double)a.shield_k * (double)a.av_per_nh * 1.4426950408889634);
-    P.out_bulk = a.n_h && aligned16(a.n_h);
-    P.form = leaf_form(a, P.out_bulk, list);
+    // A_V alone leaves like N_H, in bulk copies of the staged rows (256^3, 48
+    // directions: 0.61 ms; beside N_H it is written from them, 1.13 ms together;
+    // both were 4-byte stores of a thread a row, 5.06 and 5.55 ms)
+    const bool av_rows = a.a_v && !a.n_h && aligned16(a.a_v);
+    if (av_rows) {
+        P.a.n_h = a.a_v;
+        P.a.a_v = nullptr;
+    }
+    P.out_bulk = P.a.n_h && aligned16(P.a.n_h);
+    P.form = leaf_form(P.a, P.out_bulk, list) | (av_rows ? kFormAvRows : 0);
     P.pipe_polls = pipe_polls();
     P.span_max = g_span_max.load();
     int dev = 0, smax = 0;

@@ -122,7 +122,9 @@ def test_fp32_shell_rows_on_lists_match_uniform(dset):
 
 
 @pytest.mark.parametrize("dset", [("mxn", 1, 4), ("mxn", 2, 4), ("healpix", 1, 0), ("mxn", 4, 4), ("mxn", 5, 4),
-                                  ("mxn", 4, 6), ("mxn", 4, 7), ("mxn", 8, 4)])
+                                  ("mxn", 4, 6), ("mxn", 4, 7), ("mxn", 8, 4), ("mxn", 9, 4), ("mxn", 5, 8),
+                                  ("mxn", 11, 4), ("healpix", 2, 0), ("mxn", 13, 4), ("mxn", 7, 8), ("mxn", 15, 4),
+                                  ("mxn", 8, 8)])
 @pytest.mark.parametrize("L", [3, 4, 6])
 def test_bf16_leaves_of_few_directions(L, dset):
     # every direction count of the oct form, a tree smaller than its tile and
@@ -139,14 +141,17 @@ def test_bf16_leaves_of_few_directions(L, dset):
     colden.column_density(tree, geom, a_v=av2, precision=colden.BF16)
     colden.column_density(tree, geom, shield=sh2, precision=colden.BF16)
     colden.device_status()
-    assert torch.equal(nh, nh2) and torch.equal(av, av2) and torch.equal(sh, sh2)
+    # (beyond 32 directions the screening factor alone has a kernel of its own: the
+    # same columns, summed in another order)
+    assert torch.equal(nh, nh2) and torch.equal(av, av2)
+    assert torch.equal(sh, sh2) if nd <= 32 else float((sh - sh2).abs().max()) < 1e-6
     rows = np.unique(np.random.default_rng(L).integers(0, tree.n_leaf, 300))
     want = oracle.Tree.uniform(rho, BOX).column_density(geom.dirs, np.full(len(rows), L), oracle.morton_ijk(L)[rows])
     at = torch.from_numpy(rows).cuda()
     got = nh[at].double().cpu().numpy()
     assert np.max(np.abs(got - want) / want) <= 1e-2
     assert np.max(np.abs(av[at].double().cpu().numpy() - oracle.a_v(got)) / oracle.a_v(got)) < 1e-6
-    assert np.max(np.abs(sh[at].double().cpu().numpy() - oracle.shield(want))) <= 5e-3
+    assert np.max(np.abs(sh2[at].double().cpu().numpy() - oracle.shield(want))) <= 5e-3
 
 
 @pytest.mark.parametrize("L,dset,H", [(1, ("healpix", 1, 0), 16), (2, ("axes", 0, 0), 33), (4, ("mxn", 5, 3), 64),
@@ -199,3 +204,31 @@ def test_fp32_leaves_of_any_direction_count_and_alignment(L, dset, shift):
     assert np.max(np.abs(got - want) / want) <= 1e-5
     assert np.max(np.abs(av.reshape(n, nd)[at].double().cpu().numpy() - oracle.a_v(got)) / oracle.a_v(got)) < 1e-6
     assert np.max(np.abs(sh[at].double().cpu().numpy() - oracle.shield(want))) <= 1e-5
+
+
+@pytest.mark.parametrize("dset", [("mxn", 5, 8), ("healpix", 2, 0), ("mxn", 8, 8)])
+@pytest.mark.parametrize("shift", [0, 1])
+def test_bf16_extinction_rows(dset, shift):
+    # A_V alone, beside N_H and off the 16-byte boundary, on a uniform tree and on
+    # lists whose rows scatter: N_H times the constant, to one rounding (lists
+    # send N_H off the boundary through the FP32 leaf kernel, whose local term is
+    # not rounded: there A_V alone, from the tensor cores, has another N_H)
+    geom = colden.precompute_geometry(*dset)
+    nd = geom.n_dir
+    fine = _rho(6, 4, 1.0)
+    fine[10:30, 5:40, 20:50] *= 30.0
+    lv = synth.amr_leaves(fine, 5, [60.0])
+    for tree in (colden.build_tree_uniform(torch.from_numpy(fine).cuda(), BOX),
+                 colden.build_tree_amr(5, 6, BOX, lv["level"], lv["ijk"], lv["rho"])):
+        n = tree.n_leaf * nd
+        new = lambda: torch.full((n + 4,), -1.0, device="cuda")[shift:shift + n]  # noqa: E731
+        nh, av, alone, sh = new(), new(), new(), torch.empty(tree.n_leaf, device="cuda")
+        colden.column_density(tree, geom, n_h=nh, a_v=av, shield=sh, precision=colden.BF16)
+        colden.column_density(tree, geom, a_v=alone, precision=colden.BF16)
+        colden.device_status()
+        want = nh.double() * colden.opts_default().av_per_nh
+        assert float(nh.min()) > 0
+        for got in (av, alone) if tree.n_oct * 8 == tree.n_leaf or not shift else (av,):
+            assert float(((got.double() - want).abs() / want).max()) < 2e-7
+        sh_want = torch.exp(-2.5 * want.reshape(-1, nd)).mean(1)
+        assert float((sh.double() - sh_want).abs().max()) < 1e-5
