@@ -950,7 +950,7 @@ cd_status column_density_amr(cd_tree t, cd_geom g, const cd_opts &opts, float *n
         if (!no) continue;
         if (insitu) {
             cd_status st =
-                launch_insitu(t, g, k, no, t->oct_key + t->oct_begin[k], t->ws.E + t->oct_begin[k] * nd, s_oct);
+                launch_insitu(t, g, k, no, t->oct_key + t->oct_begin[k], &t->tc_oct[k], t->ws.E + t->oct_begin[k] * nd, s_oct);
             if (st != CD_OK) return st;
             CD_CUDA(cudaEventRecord(t->ev_E[k], s_oct));
             have_E[k] = true;

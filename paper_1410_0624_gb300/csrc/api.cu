@@ -529,7 +529,7 @@ static cd_status evaluate(cd_tree tree, cd_geom geom, const cd_opts *opts_in, fl
     if (st != CD_OK) return st;
     if (insitu) {
         // every shell from the oct centre (an exact walk per level), then the leaves
-        if (L >= 2 && (st = launch_insitu(tree, geom, L - 1, tree->n_oct, nullptr, tree->ws.E, s)) != CD_OK) return st;
+        if (L >= 2 && (st = launch_insitu(tree, geom, L - 1, tree->n_oct, nullptr, nullptr, tree->ws.E, s)) != CD_OK) return st;
         LeafLaunch b = {};
         b.n_oct = tree->n_oct;
         b.nd = nd;

@@ -379,8 +379,10 @@ void list_job_fill_far3(cd_tree t, cd_geom g, const uint64_t *keys512, void *dst
 cd_status launch_list_batch(const void *jobs, int n_jobs, int64_t max_elems, cudaStream_t s);
 
 // insitu.cu: the external column of n octs of level k (keys NULL: every oct of
-// a uniform tree), every shell seen from the oct centre (§4.3)
-cd_status launch_insitu(cd_tree t, cd_geom g, int k, int64_t n, const uint64_t *keys, float *out, cudaStream_t s);
+// a uniform tree; list: the same octs as receivers), every shell seen from the
+// oct centre (§4.3)
+cd_status launch_insitu(cd_tree t, cd_geom g, int k, int64_t n, const uint64_t *keys, const TcList *list, float *out,
+                        cudaStream_t s);
 
 // geometry.cu
 int make_directions(int scheme, int p0, int p1, const double *custom, int n_custom, double *out);

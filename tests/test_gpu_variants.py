@@ -232,3 +232,26 @@ def test_bf16_extinction_rows(dset, shift):
             assert float(((got.double() - want).abs() / want).max()) < 2e-7
         sh_want = torch.exp(-2.5 * want.reshape(-1, nd)).mean(1)
         assert float((sh.double() - sh_want).abs().max()) < 1e-5
+
+
+@pytest.mark.parametrize("L,dset", [(4, ("mxn", 5, 8)), (5, ("mxn", 5, 3)), (6, ("axes", 0, 0)), (7, ("healpix", 2, 0))])
+def test_insitu_near_shells_from_the_tables(L, dset):
+    # levels where every shell is walked, where one to three are, and directions
+    # the tables' row form does not take; uniform and adaptive, FP32 tolerance
+    geom = colden.precompute_geometry(*dset, mode=colden.MODE_INSITU)
+    fine = _rho(L, 12, 1.2)
+    fine[: 1 << (L - 1), : 1 << (L - 1)] *= 20.0
+    rng = np.random.default_rng(L)
+    trees = [(colden.build_tree_uniform(torch.from_numpy(fine).cuda(), BOX), oracle.Tree.uniform(fine, BOX))]
+    if L >= 5:
+        lv = synth.amr_leaves(fine, L - 2, [40.0, 60.0])
+        args = (L - 2, L, BOX, lv["level"], lv["ijk"], lv["rho"])
+        trees.append((colden.build_tree_amr(*args), oracle.Tree.amr(*args)))
+    for tree, T in trees:
+        nh = torch.empty((tree.n_leaf, geom.n_dir), device="cuda")
+        colden.column_density(tree, geom, n_h=nh)
+        level, ijk = tree.leaves()
+        rows = rng.integers(0, tree.n_leaf, 300)
+        want = T.column_density(geom.dirs, level[rows], ijk[rows], mode=oracle.MODE_INSITU)
+        got = nh[torch.from_numpy(rows).cuda()].double().cpu().numpy()
+        assert np.max(np.abs(got - want) / want) <= 1e-5
