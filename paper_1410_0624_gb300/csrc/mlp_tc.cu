@@ -17,9 +17,9 @@
 //                    MMA1 (W1c, + h) -> GELU -> MMA2 (W2, + b2) -> GELU ->
 //                    MMA3 (W3, + b3) = delta log2(e) -> N = N_tree 2^(...),
 //                    A_V and the shield; the tile's N rows leave as one bulk
-//                    copy.  Two independent groups
-//                    of four warps share the weights, so one group's CUDA-core
-//                    work overlaps the other's MMAs.
+//                    copy.  Three independent groups of eight warps share the
+//                    weights, so one group's CUDA-core work overlaps the
+//                    others' MMAs.
 //
 // Additions folded into the MMAs.  Every chain ends with one extra K-step of
 // 16 whose A is a constant one-hot block, A1h[m][k] = (k == m / 8): row m
@@ -34,6 +34,7 @@
 // Waits on the tensor cores are bounded; a timeout sets a device flag
 // (cd_device_status) and the kernel leaves its loop with all threads together.
 #include <algorithm>
+#include <cfloat>
 #include <vector>
 
 #include "learned.cuh"
@@ -113,7 +114,7 @@ struct PackArgs {
     unsigned char *buf;
 };
 
-// W3 and b3 are scaled by log2(e) so that the last chain gives delta log2(e)
+// W2 and W3 carry the half of GELU.  W3 and b3 are scaled by log2(e) so that the last chain gives delta log2(e)
 // and N = N_tree 2^(that).
 __global__ void pack_tc(PackArgs A)
 {
@@ -142,14 +143,14 @@ __global__ void pack_tc(PackArgs A)
         i -= n1e;
         if (i < n2) {
             const int n = (int)(i / kKW), k = (int)(i % kKW);
-            const float v = k < kH ? W2[(int64_t)n * kH + k] : A.p[N.b2 + n];
+            const float v = k < kH ? 0.5f * W2[(int64_t)n * kH + k] : A.p[N.b2 + n];
             reinterpret_cast<__nv_bfloat16 *>(A.buf + T.w2 + op_off(n, k, kKW))[0] = __float2bfloat16_rn(v);
             continue;
         }
         i -= n2;
         if (i < n3) {
             const int n = (int)(i / kKW), k = (int)(i % kKW);
-            const float v = n >= nd ? 0.f : kLog2e * (k < kH ? W3[(int64_t)n * kH + k] : A.p[N.b3 + n]);
+            const float v = n >= nd ? 0.f : kLog2e * (k < kH ? 0.5f * W3[(int64_t)n * kH + k] : A.p[N.b3 + n]);
             reinterpret_cast<__nv_bfloat16 *>(A.buf + T.w3 + op_off(n, k, kKW))[0] = __float2bfloat16_rn(v);
             continue;
         }
@@ -186,19 +187,18 @@ __device__ __forceinline__ uint32_t bf2(float v)   // a BF16 constant in both ha
     return pack_bf16x2(v, v);
 }
 
-// GELU (tanh form) of two BF16 values in packed BF16 arithmetic:
-// g = z/2 (1 + tanh(z (c + c a z^2))).  The result is an operand of the next
-// BF16 product either way.
-__device__ __forceinline__ uint32_t gelu_bf16x2(uint32_t z)
+// Twice the GELU (tanh form) of two BF16 values in packed BF16 arithmetic:
+// 2 g = z (1 + tanh(z (c + c a z^2))).  The result is an operand of the next
+// BF16 product, whose packed weights carry the half (exact in BF16).
+__device__ __forceinline__ uint32_t gelu2_bf16x2(uint32_t z)
 {
-    uint32_t z2, p, inner, t, hz, g;
-    const uint32_t ca = bf2(kGeluC * kGeluA), c = bf2(kGeluC), half = bf2(0.5f);
+    uint32_t z2, p, inner, t, g;
+    const uint32_t ca = bf2(kGeluC * kGeluA), c = bf2(kGeluC);
     asm("mul.rn.bf16x2 %0, %1, %1;" : "=r"(z2) : "r"(z));
     asm("fma.rn.bf16x2 %0, %1, %2, %3;" : "=r"(p) : "r"(z2), "r"(ca), "r"(c));
     asm("mul.rn.bf16x2 %0, %1, %2;" : "=r"(inner) : "r"(p), "r"(z));
     asm("tanh.approx.bf16x2 %0, %1;" : "=r"(t) : "r"(inner));
-    asm("mul.rn.bf16x2 %0, %1, %2;" : "=r"(hz) : "r"(z), "r"(half));
-    asm("fma.rn.bf16x2 %0, %1, %2, %1;" : "=r"(g) : "r"(hz), "r"(t));
+    asm("fma.rn.bf16x2 %0, %1, %2, %1;" : "=r"(g) : "r"(z), "r"(t));
     return g;
 }
 
@@ -213,6 +213,20 @@ __device__ __forceinline__ float fast_log2(float x)
 __device__ __forceinline__ float std_input(float x, float floor_, float a, float b)
 {
     return fminf(fmaxf(fmaf(a, fast_log2(fmaxf(x, floor_)), b), -kUMax), kUMax);
+}
+
+// Two standardised, clipped inputs in BF16.  Rounding keeps order, so clipping
+// after it gives the same values; lo = max(a lg2(floor) + b, -clip) does for the
+// floor and the lower clip (a >= 0; an ignored input has a = b = 0, and its
+// 0 x inf falls back to lo = 0).
+__device__ __forceinline__ uint32_t std_input2(float2 x, float2 a, float2 b, uint32_t lo)
+{
+    const float2 u = __ffma2_rn(a, make_float2(fast_log2(x.x), fast_log2(x.y)), b);
+    uint32_t v = pack_bf16x2(u.x, u.y);
+    const uint32_t hi = pack_bf16x2(kUMax, kUMax);
+    asm("max.bf16x2 %0, %0, %1;" : "+r"(v) : "r"(lo));
+    asm("min.bf16x2 %0, %0, %1;" : "+r"(v) : "r"(hi));
+    return v;
 }
 
 __device__ __forceinline__ float fast_exp2(float x)
@@ -233,9 +247,10 @@ __device__ __forceinline__ void mma_steps(uint32_t tmem_d, uint32_t a0, int Ka, 
                                           bool accumulate_first)
 {
     const uint32_t idesc = umma_idesc_bf16(128, N);
-    for (int ks = 0; ks < steps; ++ks)
-        umma_bf16(tmem_d, umma_smem_desc(a0 + ks * 256, 128, (uint32_t)Ka * 16),
-                  umma_smem_desc(b0 + ks * 256, 128, (uint32_t)Kb * 16), idesc, (ks > 0 || accumulate_first) ? 1u : 0u);
+    // a K-step is 256 bytes: 16 in the descriptor's address field
+    uint64_t da = umma_smem_desc(a0, 128, (uint32_t)Ka * 16), db = umma_smem_desc(b0, 128, (uint32_t)Kb * 16);
+    for (int ks = 0; ks < steps; ++ks, da += 16, db += 16)
+        umma_bf16(tmem_d, da, db, idesc, (ks > 0 || accumulate_first) ? 1u : 0u);
 }
 
 // ---- per-oct part ---------------------------------------------------------------
@@ -493,21 +508,22 @@ struct CellArgs {
     int vec;                         // n_h is 16-byte aligned: a tile's rows leave as one bulk copy
 };
 
-constexpr int kCellThreads = 512;   // two groups of 256: two threads per leaf row, each half the columns
+constexpr int kGroups = 3;                       // tiles in flight per CTA
+constexpr int kGroupThreads = 256;               // two threads per leaf row, each half the columns
+constexpr int kCellThreads = kGroups * kGroupThreads;
+constexpr int kMaxGq = (kMaxNd / 8 + 1) / 2;      // 8-direction groups a thread takes
 
 // Shared memory of learned_cell_tc.  Shared: the weight images, the one-hot
 // block, the local-term operand B_loc [NP x 64] = dx K_loc[t][s][d] at
 // k = 8 t + s, the cell standardisation.  Per group: the operand buffer (the
 // leaf inputs [128 x KC] for MMA1, then the activations [128 x 128] for MMA2
-// and MMA3, then the tile's N rows [128 x nd] FP32 on their way out), the
-// local-term operand A_loc [128 x 64] (row m holds its oct's 8 densities in
-// block t = m % 8, zero elsewhere), and two stages of the tile's inputs that
-// bulk copies bring in one tile ahead (the 16 octs' layer-1 block, which MMA1
-// reads in place, densities of the 128 leaves and external columns of their
-// 16 octs).
+// and MMA3, then the tile's N rows [128 x nd] FP32 on their way out), and two
+// stages of the tile's inputs that bulk copies bring in one tile ahead (the 16
+// octs' layer-1 block, which MMA1 reads in place, densities of the 128 leaves
+// and external columns of their 16 octs).
 struct CellSmem {
-    size_t w1c, w2, w3, onehot, bloc, muc, sic, bar, grp, grp_stride, a, aloc, stage, stage_bytes, st_rho, st_ext,
-        st_h, total;
+    size_t w1c, w2, w3, onehot, bloc, muc, sic, lo, bar, grp, grp_stride, a, stage, stage_bytes, st_rho, st_ext, st_h,
+        total;
 };
 
 __host__ __device__ inline CellSmem cell_smem(const TcLayout &T)
@@ -522,17 +538,17 @@ __host__ __device__ inline CellSmem cell_smem(const TcLayout &T)
     S.bloc = take((size_t)T.NP * 64 * 2);
     S.muc = take((size_t)T.KC * 4);
     S.sic = take((size_t)T.KC * 4);
+    S.lo = take((size_t)T.KC * 2);
     S.bar = take(128);
     S.grp = o;
     S.a = 0;
-    S.aloc = align128((size_t)128 * kH * 2);
     S.st_h = 0;
     S.st_rho = (size_t)kHBlock * 2;
     S.st_ext = S.st_rho + 128 * 4;
     S.stage_bytes = align128(S.st_ext + (size_t)16 * T.nd * 4);
-    S.stage = S.aloc + (size_t)128 * 64 * 2;
+    S.stage = align128((size_t)128 * kH * 2);
     S.grp_stride = S.stage + 2 * S.stage_bytes;
-    S.total = S.grp + 2 * S.grp_stride;
+    S.total = S.grp + kGroups * S.grp_stride;
     return S;
 }
 
@@ -549,6 +565,16 @@ __device__ __forceinline__ void prefetch_tile(const CellArgs &A, const CellSmem 
     bulk_g2s(st + S.st_ext, A.ext + (c0 >> 3) * A.T.nd, b_ext, bar);
 }
 
+// What bounds it: the CUDA cores' work of a tile (GELU of 256 values a leaf,
+// logarithms, exponentials) and the latencies of its four MMA chains, which
+// follow one another; shared memory is at two thirds of its rate (operands of the
+// chains, activations, rows).  Hence three tiles in flight, as many as shared
+// memory holds: every thread polls its chain's mbarrier itself, so that a chain
+// costs one barrier (its operands are ready), and the local term of a tile is
+// issued with the rows of the one before.  A_loc lies in tensor memory, where its
+// zeros cost nothing; activations there too, with two tiles in flight (TMEM has
+// room for no more), take 2.91 ms.  256^3 leaves, 48 directions: 3.25 -> 2.37 ms
+// (0.54 TFLOP of products; two tiles in flight and two barriers a chain before).
 __global__ void __launch_bounds__(kCellThreads, 1) learned_cell_tc(CellArgs A)
 {
     extern __shared__ __align__(1024) unsigned char smem[];
@@ -561,19 +587,22 @@ __global__ void __launch_bounds__(kCellThreads, 1) learned_cell_tc(CellArgs A)
     const bool lead = half == 0 && i == 0;     // issues the group's copies and MMAs
     const float *sMu = reinterpret_cast<const float *>(smem + S.muc);
     const float *sSi = reinterpret_cast<const float *>(smem + S.sic);
-    // [0] weights, [1 + g] group MMAs, [3 + 2 g + stage] group input stages
+    const __nv_bfloat16 *sLo = reinterpret_cast<const __nv_bfloat16 *>(smem + S.lo);
+    // [0] weights, [1 + g] group MMAs, [1 + kGroups + 2 g + stage] group input stages
     uint64_t *bar = reinterpret_cast<uint64_t *>(smem + S.bar);
-    uint32_t *tslot = reinterpret_cast<uint32_t *>(bar + 7);
-    int *sflag = reinterpret_cast<int *>(tslot + 1);                  // [2] per-group fault flags
+    uint64_t *mma_bar = bar + 1 + g, *stage_bar = bar + 1 + kGroups + 2 * g;
+    uint32_t *tslot = reinterpret_cast<uint32_t *>(bar + 1 + 3 * kGroups);
+    // fault flags [group][barrier parity]: set between barriers n - 1 and n, read after n
+    int *sflag = reinterpret_cast<int *>(tslot + 1);
     unsigned char *G = smem + S.grp + g * S.grp_stride;
     unsigned char *sOp = G + S.a;
-    unsigned char *sAloc = G + S.aloc;
-    __shared__ float sAcc[2 * 2 * 128];         // [group][half][row] screening partial sums
+    __shared__ float sAcc[kGroups][2][128];     // [group][half][row] screening partial sums
+    static_assert((1 + 3 * kGroups) * 8 + 4 + 2 * kGroups * 4 <= 128, "barrier block");
 
     if (tid == 0) {
-        for (int b = 0; b < 7; ++b) mbar_init(&bar[b], 1);
+        for (int b = 0; b < 1 + 3 * kGroups; ++b) mbar_init(&bar[b], 1);
         fence_mbar_init();
-        sflag[0] = sflag[1] = 0;
+        for (int b = 0; b < 2 * kGroups; ++b) sflag[b] = 0;
     }
     // B_loc[d][8 t + s] = dx K_loc[t][s][d] (directions past nd are zero)
     for (int e = tid; e < NP * 64; e += kCellThreads) {
@@ -581,14 +610,12 @@ __global__ void __launch_bounds__(kCellThreads, 1) learned_cell_tc(CellArgs A)
         const float v = n < nd ? A.dx_leaf * A.kloc[(k >> 3) * 8 * nd + (k & 7) * nd + n] : 0.f;
         *reinterpret_cast<__nv_bfloat16 *>(smem + S.bloc + op_off(n, k, 64)) = __float2bfloat16_rn(v);
     }
-    // A_loc starts all zero; each tile rewrites only its rows' own blocks
-    for (int e = tid; e < 2 * 128 * 64 / 8; e += kCellThreads) {
-        const int gg = e / (128 * 8), r = e % (128 * 8);
-        reinterpret_cast<uint4 *>(smem + S.grp + gg * S.grp_stride + S.aloc)[r] = make_uint4(0, 0, 0, 0);
-    }
     for (int k = tid; k < KC; k += kCellThreads) {
-        reinterpret_cast<float *>(smem + S.muc)[k] = reinterpret_cast<const float *>(A.tc + T.muc)[k];
-        reinterpret_cast<float *>(smem + S.sic)[k] = reinterpret_cast<const float *>(A.tc + T.sic)[k];
+        const float a = reinterpret_cast<const float *>(A.tc + T.muc)[k], b = reinterpret_cast<const float *>(A.tc + T.sic)[k];
+        reinterpret_cast<float *>(smem + S.muc)[k] = a;
+        reinterpret_cast<float *>(smem + S.sic)[k] = b;
+        reinterpret_cast<__nv_bfloat16 *>(smem + S.lo)[k] =
+            __float2bfloat16_rn(fmaxf(fmaf(a, fast_log2(k == nd ? kNFloor : kCFloor), b), -kUMax));
     }
     for (int e = tid; e < kHBlock; e += kCellThreads) {   // one-hot: row m selects column m / 8
         const int m = e >> 4, k = e & 15;
@@ -608,221 +635,253 @@ __global__ void __launch_bounds__(kCellThreads, 1) learned_cell_tc(CellArgs A)
         bulk_g2s(smem + S.w2, A.tc + T.w2, b2, &bar[0]);
         bulk_g2s(smem + S.w3, A.tc + T.w3, b3, &bar[0]);
     }
-    // per group 256 TMEM columns: D (128: D1, D2, D3 in turn, each read out
-    // before the next chain) and the local term (NP columns, alive through the tile)
-    const uint32_t tD = tbase + (uint32_t)(g * 256), tL = tD + 128;
+    // per group 160 TMEM columns: D (128: D1, D2 in turn, each read out before
+    // the next chain; then D3 in columns 0 .. NP-1), the local term in columns
+    // 64 .. 64 + NP-1 of it (before D1 and again beside D3), and A_loc (32: row m
+    // holds its oct's 8 densities in block t = m % 8, zero elsewhere)
+    const uint32_t tD = tbase + (uint32_t)(g * 160), tL = tD + 64, tA = tD + 128;
     const uint32_t lane_off = (uint32_t)(quarter * 32) << 16;
     const uint32_t a_op = smem_u32(sOp), a_1h = smem_u32(smem + S.onehot);
-    const int bid = 1 + g;                                               // named barrier of the group
-    const int64_t first = 2 * (int64_t)blockIdx.x + g, stride = 2 * (int64_t)gridDim.x;
-    bool weights_ready = false;
-    uint32_t phase = 0, sphase[2] = {0, 0};
-    bool pending[2] = {false, false};          // leader: a prefetch into the stage has not been waited for
+    const int first = blockIdx.x + gridDim.x * g, stride = gridDim.x * kGroups, ntiles = (int)A.ntiles;
+    uint32_t phase = 0, sphase = 0;            // sphase: a bit per stage
+    uint32_t nbar = 0;                         // group barriers passed
+    uint32_t pending = 0;                      // leader, a bit per stage: its prefetch has not been waited for
     bool fault = false;
-    if (lead && first < A.ntiles) {
-        prefetch_tile(A, S, first, G + S.stage, &bar[3 + 2 * g]);
-        pending[0] = true;
-    }
-
-    const bool bulk_out = A.n_h && A.vec;
-    // leader of the group: issue, commit and wait (bounded); everyone learns
-    // the outcome after the group barrier.  layer 0 = the local term.
-    auto issue_and_wait = [&](int layer, uint32_t h_block) {
-        if (lead) {
-            // the previous tile's N rows must have left the operand buffer
-            // before anyone writes it again (right after the local term)
-            if (layer == 0 && bulk_out) bulk_wait_read<0>();
-            bool ok = true;
-            if (!weights_ready) ok = weights_ready = mbar_wait_bounded(&bar[0], 0, kMaxPolls);
-            if (ok) {
-                tc_fence_after();
-                if (layer == 0) {
-                    mma_steps(tL, smem_u32(sAloc), 64, smem_u32(smem + S.bloc), 64, 4, NP, false);
-                } else if (layer == 1) {
-                    mma_steps(tD, a_op, KC, smem_u32(smem + S.w1c), KC, KC / 16, kH, false);
-                    mma_steps(tD, a_1h, 16, h_block, 16, 1, kH, true);
-                } else {
-                    const uint32_t w = smem_u32(smem + (layer == 2 ? S.w2 : S.w3));
-                    const int N = layer == 2 ? kH : NP;
-                    mma_steps(tD, a_op, kH, w, kKW, kH / 16, N, false);
-                    mma_steps(tD, a_1h, 16, w + (kH / 16) * 256, kKW, 1, N, true);
-                }
-                umma_commit(&bar[1 + g]);
-                ok = mbar_wait_bounded(&bar[1 + g], phase, kMaxPolls);
+    if (lead) {
+        for (int b = 0; b < 2; ++b)
+            if (first + b * stride < ntiles) {
+                prefetch_tile(A, S, first + b * stride, G + S.stage + b * S.stage_bytes, &stage_bar[b]);
+                pending |= 1u << b;
             }
-            if (!ok) sflag[g] = 1;
-        }
+    }
+    const bool bulk_out = A.n_h && A.vec;
+
+    auto give_up = [&]() { sflag[2 * g + (nbar & 1)] = 1; };
+    auto wait_mma = [&]() {
+        if (!mbar_wait_bounded(mma_bar, phase, kMaxPolls)) give_up();
         phase ^= 1;
-        named_barrier(bid, 256);
-        fault = sflag[g] != 0;
         tc_fence_after();
     };
+    auto wait_stage = [&](int b) {
+        if (mbar_wait_bounded(&stage_bar[b], (sphase >> b) & 1, kMaxPolls)) pending &= ~(1u << b);
+        else give_up();
+        sphase ^= 1u << b;
+    };
+    // Everything this group wrote is ready for the next chain (or copy); false
+    // if any of its threads gave up a wait.
+    auto ready = [&]() {
+        fence_proxy_async_smem();
+        tc_fence_before();
+        named_barrier(1 + g, kGroupThreads);
+        tc_fence_after();
+        fault = sflag[2 * g + (nbar & 1)] != 0;
+        ++nbar;
+        return !fault;
+    };
+    // A_loc of a tile: this thread writes its half of the row's blocks
+    auto put_densities = [&](int b, int tile) {
+        const float *sR = reinterpret_cast<const float *>(G + S.stage + b * S.stage_bytes + S.st_rho);
+        const bool valid = (int64_t)tile * 128 + i < A.n_leaf;
+        const float4 r0 = *reinterpret_cast<const float4 *>(sR + (i & ~7));
+        const float4 r1 = *reinterpret_cast<const float4 *>(sR + (i & ~7) + 4);
+        const uint32_t w[4] = {pack_bf16x2(r0.x, r0.y), pack_bf16x2(r0.z, r0.w), pack_bf16x2(r1.x, r1.y),
+                               pack_bf16x2(r1.z, r1.w)};
+        const int t = valid ? (i & 7) - 4 * half : -1;
+        uint32_t v[16];
+#pragma unroll
+        for (int c = 0; c < 16; ++c) v[c] = (c >> 2) == t ? w[c & 3] : 0u;
+        tmem_st16(tA + lane_off + (uint32_t)(16 * half), v);
+        tmem_st_wait();
+    };
+    auto issue_local = [&]() {
+        for (int ks = 0; ks < 4; ++ks)
+            umma_bf16_ta(tL, tA + 8 * ks, umma_smem_desc(smem_u32(smem + S.bloc) + ks * 256, 128, 64 * 16),
+                         umma_idesc_bf16(128, NP), ks > 0 ? 1u : 0u);
+    };
 
-    // GELU of a 128-column accumulator row -> the operand buffer; two 32-column
-    // loads in flight per wait
+    // GELU of a 128-column accumulator row -> the operand buffer; the next 16
+    // columns are on their way while 16 are worked on
     auto gelu_row = [&]() {
-#pragma unroll 1
-        for (int c = 64 * half; c < 64 * half + 64; c += 32) {
-            uint32_t v[32];
-            tmem_ld32(tD + lane_off + (uint32_t)c, v);
-            tmem_ld_wait();
+        const uint32_t src = tD + lane_off + (uint32_t)(64 * half);
+        unsigned char *dst = sOp + op_off(i, 64 * half, kH);
+        uint32_t v[2][16];
+        tmem_ld16(src, v[0]);
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                uint32_t o[4];
+        for (int k = 0; k < 4; ++k) {
+            uint32_t(&w)[16] = v[k & 1];
+            tmem_ld_wait(w);
+            if (k < 3) tmem_ld16(src + 16 * (k + 1), v[(k + 1) & 1]);
+            uint32_t o[8];
 #pragma unroll
-                for (int p2 = 0; p2 < 4; ++p2)
-                    o[p2] = gelu_bf16x2(pack_bf16x2(__uint_as_float(v[8 * q + 2 * p2]),
-                                                    __uint_as_float(v[8 * q + 2 * p2 + 1])));
-                *reinterpret_cast<uint4 *>(sOp + op_off(i, c + 8 * q, kH)) = make_uint4(o[0], o[1], o[2], o[3]);
-            }
+            for (int p = 0; p < 8; ++p) o[p] = gelu2_bf16x2(pack_bf16x2(__uint_as_float(w[2 * p]), __uint_as_float(w[2 * p + 1])));
+            *reinterpret_cast<uint4 *>(dst + (2 * k) * 128) = make_uint4(o[0], o[1], o[2], o[3]);
+            *reinterpret_cast<uint4 *>(dst + (2 * k + 1) * 128) = make_uint4(o[4], o[5], o[6], o[7]);
         }
     };
     // the row's 8-direction groups this thread takes: [gq0, gq1) of nd / 8
     const int ngq = nd >> 3, gq0 = half * ((ngq + 1) >> 1), gq1 = half ? ngq : (ngq + 1) >> 1;
 
+    // weights, and the first tile's local term
+    if (!mbar_wait_bounded(&bar[0], 0, kMaxPolls)) give_up();
+    if (first < ntiles) {
+        wait_stage(0);
+        put_densities(0, first);
+    }
+    if (ready() && lead && first < ntiles) {
+        issue_local();
+        umma_commit(mma_bar);
+    }
+
     int stg = 0;
-    for (int64_t tile = first; tile < A.ntiles && !fault; tile += stride, stg ^= 1) {
-        const int64_t c0 = tile * 128;
+    for (int tile = first; tile < ntiles && !fault; tile += stride, stg ^= 1) {
+        const int64_t c0 = (int64_t)tile * 128;
         const int rows = (int)std::min<int64_t>(128, A.n_leaf - c0);
         const int64_t m = c0 + i;
-        const bool valid = i < rows;
+        const bool valid = i < rows, more = tile + stride < ntiles;
         unsigned char *st = G + S.stage + stg * S.stage_bytes;
-        // the next tile's inputs go to the other stage (its last reader was the
-        // previous tile, finished at that tile's final barrier); the previous
-        // tile's N rows must have left the operand buffer
-        if (lead) {
-            if (tile + stride < A.ntiles) {
-                prefetch_tile(A, S, tile + stride, G + S.stage + (stg ^ 1) * S.stage_bytes,
-                              &bar[3 + 2 * g + (stg ^ 1)]);
-                pending[stg ^ 1] = true;
-            }
-            if (mbar_wait_bounded(&bar[3 + 2 * g + stg], sphase[stg], kMaxPolls)) pending[stg] = false;
-            else sflag[g] = 1;
-        }
-        sphase[stg] ^= 1;
-        named_barrier(bid, 256);
-        if (sflag[g]) {
-            fault = true;
-            break;
-        }
-        const float *sR = reinterpret_cast<const float *>(st + S.st_rho);
         const float *sE = reinterpret_cast<const float *>(st + S.st_ext) + (i >> 3) * nd;
-
-        // ---- local term on the tensor cores: A_loc row = the oct's 8 densities ----
-        if (half == 0) {
-            const float4 r0 = *reinterpret_cast<const float4 *>(sR + (i & ~7));
-            const float4 r1 = *reinterpret_cast<const float4 *>(sR + (i & ~7) + 4);
-            const uint4 w = valid ? make_uint4(pack_bf16x2(r0.x, r0.y), pack_bf16x2(r0.z, r0.w),
-                                               pack_bf16x2(r1.x, r1.y), pack_bf16x2(r1.z, r1.w))
-                                  : make_uint4(0, 0, 0, 0);
-            *reinterpret_cast<uint4 *>(sAloc + op_off(i, 8 * (i & 7), 64)) = w;
-        }
-        fence_proxy_async_smem();
-        tc_fence_before();
-        named_barrier(bid, 256);
-        issue_and_wait(0, 0);
-        if (fault) break;
 
         // ---- u_cell = standardised ln(local term) (8 directions per 16-byte
         //      store), then ln n and the K padding ----
-#pragma unroll 1
-        for (int q = gq0; q < gq1; ++q) {
-            const int d0 = 8 * q;
-            uint32_t v[8];
-            tmem_ld8(tL + lane_off + (uint32_t)d0, v);
-            tmem_ld_wait();
-            const float4 a0 = *reinterpret_cast<const float4 *>(sMu + d0), a1 = *reinterpret_cast<const float4 *>(sMu + d0 + 4);
-            const float4 b0 = *reinterpret_cast<const float4 *>(sSi + d0), b1 = *reinterpret_cast<const float4 *>(sSi + d0 + 4);
-            const float a[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
-            const float b[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
-            float u[8];
+        wait_mma();
+        {
+            uint32_t v[2][8];
+            if (gq0 < gq1) tmem_ld8(tL + lane_off + (uint32_t)(8 * gq0), v[0]);
 #pragma unroll
-            for (int j = 0; j < 8; ++j) u[j] = valid ? std_input(__uint_as_float(v[j]), kCFloor, a[j], b[j]) : 0.f;
-            *reinterpret_cast<uint4 *>(sOp + op_off(i, d0, KC)) =
-                make_uint4(pack_bf16x2(u[0], u[1]), pack_bf16x2(u[2], u[3]), pack_bf16x2(u[4], u[5]),
-                           pack_bf16x2(u[6], u[7]));
+            for (int k = 0; k < kMaxGq; ++k) {
+                if (gq0 + k >= gq1) break;
+                uint32_t(&w)[8] = v[k & 1];
+                const int d0 = 8 * (gq0 + k);
+                tmem_ld_wait(w);
+                if (gq0 + k + 1 < gq1) tmem_ld8(tL + lane_off + (uint32_t)(d0 + 8), v[(k + 1) & 1]);
+                const uint4 lo = *reinterpret_cast<const uint4 *>(sLo + d0);
+                const uint32_t lw[4] = {lo.x, lo.y, lo.z, lo.w};
+                uint32_t o[4];
+#pragma unroll
+                for (int p = 0; p < 4; ++p)
+                    o[p] = std_input2(make_float2(__uint_as_float(w[2 * p]), __uint_as_float(w[2 * p + 1])),
+                                      *reinterpret_cast<const float2 *>(sMu + d0 + 2 * p),
+                                      *reinterpret_cast<const float2 *>(sSi + d0 + 2 * p), lw[p]);
+                *reinterpret_cast<uint4 *>(sOp + op_off(i, d0, KC)) = make_uint4(o[0], o[1], o[2], o[3]);
+            }
         }
         for (int d0 = nd + 8 * half; d0 < KC; d0 += 16) {      // ln n at column nd, zeros after it
-            const float un = valid && d0 == nd ? std_input(sR[i], kNFloor, sMu[nd], sSi[nd]) : 0.f;
+            const float n = reinterpret_cast<const float *>(st + S.st_rho)[i];
+            const float un = d0 == nd ? std_input(n, kNFloor, sMu[nd], sSi[nd]) : 0.f;
             *reinterpret_cast<uint4 *>(sOp + op_off(i, d0, KC)) = make_uint4(pack_bf16x2(un, 0.f), 0, 0, 0);
         }
-        fence_proxy_async_smem();
-        tc_fence_before();
-        named_barrier(bid, 256);
-        issue_and_wait(1, smem_u32(st + S.st_h));
-        if (fault) break;
+        if (!ready()) break;
+        if (lead) {
+            mma_steps(tD, a_op, KC, smem_u32(smem + S.w1c), KC, KC / 16, kH, false);
+            mma_steps(tD, a_1h, 16, smem_u32(st + S.st_h), 16, 1, kH, true);
+            umma_commit(mma_bar);
+        }
 
         // ---- a1 = gelu(D1) (D1 includes h[oct] + b1) ----
+        wait_mma();
         gelu_row();
-        fence_proxy_async_smem();
-        tc_fence_before();
-        named_barrier(bid, 256);
-        issue_and_wait(2, 0);
-        if (fault) break;
+        if (!ready()) break;
+        if (lead) {
+            const uint32_t w = smem_u32(smem + S.w2);
+            mma_steps(tD, a_op, kH, w, kKW, kH / 16, kH, false);
+            mma_steps(tD, a_1h, 16, w + (kH / 16) * 256, kKW, 1, kH, true);
+            umma_commit(mma_bar);
+        }
 
-        // ---- a2 = gelu(D2) (D2 includes b2; MMA2 has finished reading a1) ----
+        // ---- a2 = gelu(D2) (D2 includes b2; MMA2 has finished reading a1); the
+        //      local term once more, beside D3 ----
+        wait_mma();
         gelu_row();
-        fence_proxy_async_smem();
-        tc_fence_before();
-        named_barrier(bid, 256);
-        issue_and_wait(3, 0);
-        if (fault) break;
+        if (!ready()) break;
+        if (lead) {
+            const uint32_t w = smem_u32(smem + S.w3);
+            mma_steps(tD, a_op, kH, w, kKW, kH / 16, NP, false);
+            mma_steps(tD, a_1h, 16, w + (kH / 16) * 256, kKW, 1, NP, true);
+            issue_local();
+            umma_commit(mma_bar);
+        }
 
         // ---- N = (local + external) 2^D3 -> the operand buffer as FP32 rows; shield ----
+        wait_mma();
         {
             float *nrow = reinterpret_cast<float *>(sOp) + (size_t)i * nd;
             float *av = A.a_v && valid ? A.a_v + m * nd : nullptr;
             float *nh = A.n_h && valid && !bulk_out ? A.n_h + m * nd : nullptr;
-            float acc = 0.f;
+            const bool swap = (i >> (nd & 8 ? 2 : nd & 16 ? 1 : 0)) & 1;
+            float2 acc = make_float2(0.f, 0.f);
+            const float2 c2 = make_float2(A.c2, A.c2);
 #pragma unroll 1
-            for (int q8 = gq0; q8 < gq1; ++q8) {
-                const int c = 8 * q8;
+            for (int k = 0; k < kMaxGq; ++k) {
+                if (gq0 + k >= gq1) break;
+                const int c = 8 * (gq0 + k);
                 uint32_t v[8], w[8];
                 tmem_ld8(tD + lane_off + (uint32_t)c, v);
                 tmem_ld8(tL + lane_off + (uint32_t)c, w);
-                tmem_ld_wait();
+                tmem_ld_wait(v);
+                tmem_ld_wait(w);
+                float2 N[4];
 #pragma unroll
-                for (int j4 = 0; j4 < 8; j4 += 4) {
-                    const float4 e4 = *reinterpret_cast<const float4 *>(sE + c + j4);
-                    const float ev[4] = {e4.x, e4.y, e4.z, e4.w};
-                    float N[4];
+                for (int p = 0; p < 4; ++p) {
+                    const float2 e = *reinterpret_cast<const float2 *>(sE + c + 2 * p);
+                    const float2 nt = __fadd2_rn(
+                        make_float2(__uint_as_float(w[2 * p]), __uint_as_float(w[2 * p + 1])), e);
+                    const float d0 = __uint_as_float(v[2 * p]), d1 = __uint_as_float(v[2 * p + 1]);
+                    N[p] = __fmul2_rn(nt, make_float2(fast_exp2(d0 >= A.dlo2 && d0 <= A.dhi2 ? d0 : 0.f),
+                                                      fast_exp2(d1 >= A.dlo2 && d1 <= A.dhi2 ? d1 : 0.f)));
+                    const float2 x = __fmul2_rn(c2, N[p]);
+                    acc = __fadd2_rn(acc, make_float2(fast_exp2(x.x), fast_exp2(x.y)));
+                }
+                // rows 32 k bytes apart start on 128 / (32 k, 128) banks of 16 bytes: every
+                // other run of them takes its two pieces in the other order
+                const float4 p0 = make_float4(N[0].x, N[0].y, N[1].x, N[1].y),
+                             p1 = make_float4(N[2].x, N[2].y, N[3].x, N[3].y);
+                *reinterpret_cast<float4 *>(nrow + c + (swap ? 4 : 0)) = swap ? p1 : p0;
+                *reinterpret_cast<float4 *>(nrow + c + (swap ? 0 : 4)) = swap ? p0 : p1;
+                if (nh || av) {
+                    const float f[8] = {p0.x, p0.y, p0.z, p0.w, p1.x, p1.y, p1.z, p1.w};
 #pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        const float dl = __uint_as_float(v[j4 + q]);
-                        const float nt = __uint_as_float(w[j4 + q]) + ev[q];
-                        N[q] = isfinite(dl) && dl >= A.dlo2 && dl <= A.dhi2 ? nt * fast_exp2(dl) : nt;
-                        acc += fast_exp2(A.c2 * N[q]);
+                    for (int q = 0; q < 8; ++q) {
+                        if (nh) nh[c + q] = f[q];
+                        if (av) av[c + q] = f[q] * A.av_per_nh;
                     }
-                    *reinterpret_cast<float4 *>(nrow + c + j4) = make_float4(N[0], N[1], N[2], N[3]);
-                    if (nh)
-#pragma unroll
-                        for (int q = 0; q < 4; ++q) nh[c + j4 + q] = N[q];
-                    if (av)
-#pragma unroll
-                        for (int q = 0; q < 4; ++q) av[c + j4 + q] = N[q] * A.av_per_nh;
                 }
             }
-            sAcc[(g * 2 + half) * 128 + i] = acc;
+            sAcc[g][half][i] = acc.x + acc.y;
         }
-        fence_proxy_async_smem();
-        tc_fence_before();
-        named_barrier(bid, 256);     // the stage is rewritten by later tiles
+        // the next tile's densities (A_loc's last reader was the chain just waited for)
+        if (more) {
+            wait_stage(stg ^ 1);
+            put_densities(stg ^ 1, tile + stride);
+        }
+        if (!ready()) break;
+        if (lead) {
+            if (bulk_out) {
+                bulk_s2g(A.n_h + c0 * nd, sOp, (uint32_t)(rows * nd * 4));
+                bulk_commit();
+            }
+            if (more) {
+                issue_local();
+                if (tile + 2 * stride < ntiles) {
+                    prefetch_tile(A, S, tile + 2 * stride, st, &stage_bar[stg]);
+                    pending |= 1u << stg;
+                }
+                // the next chain's commit also says that the rows have left the operand buffer
+                if (bulk_out) bulk_wait_read<0>();
+                umma_commit(mma_bar);
+            }
+        }
         // the row's screening factor: the two halves' sums, in a fixed order
-        if (half == 0 && A.shield && valid) A.shield[m] = (sAcc[(g * 2) * 128 + i] + sAcc[(g * 2 + 1) * 128 + i]) / (float)nd;
-        if (bulk_out && lead) {
-            bulk_s2g(A.n_h + c0 * nd, sOp, (uint32_t)(rows * nd * 4));
-            bulk_commit();
-        }
+        if (half == 0 && A.shield && valid) A.shield[m] = (sAcc[g][0][i] + sAcc[g][1][i]) / (float)nd;
     }
     if (fault && lead) {
         atomicExch(&g_ltc_fault, 1);
-        mbar_wait_bounded(&bar[1 + g], phase ^ 1, kMaxPolls);   // let an issued chain finish
+        mbar_wait_bounded(mma_bar, phase ^ 1, kMaxPolls);   // let an issued chain finish
     }
     // a prefetch still in flight must land, and the output copies must have
     // read the operand buffer, before the CTA exits
     if (lead) {
         for (int b = 0; b < 2; ++b)
-            if (pending[b]) mbar_wait_bounded(&bar[3 + 2 * g + b], sphase[b], kMaxPolls);
+            if ((pending >> b) & 1) mbar_wait_bounded(&stage_bar[b], (sphase >> b) & 1, kMaxPolls);
         bulk_wait_all<0>();
     }
     tc_fence_before();
@@ -952,8 +1011,9 @@ cd_status column_density_learned_tc(cd_tree t, cd_geom g, const cd_opts &o, floa
         A.dx_leaf = (float)(t->box_cm / (double)((int64_t)1 << t->L));
         A.av_per_nh = (float)o.av_per_nh;
         A.c2 = (float)(-o.shield_k * o.av_per_nh * 1.4426950408889634);
-        A.dlo2 = (float)((double)net->dlo * 1.4426950408889634);
-        A.dhi2 = (float)((double)net->dhi * 1.4426950408889634);
+        // finite bounds: the kernel's comparisons then refuse an infinite correction as well
+        A.dlo2 = std::max((float)((double)net->dlo * 1.4426950408889634), -FLT_MAX);
+        A.dhi2 = std::min((float)((double)net->dhi * 1.4426950408889634), FLT_MAX);
         A.rho_leaf = t->rho_leaf;
         A.kloc = g->kloc;
         A.h = ts->h;
@@ -963,7 +1023,7 @@ cd_status column_density_learned_tc(cd_tree t, cd_geom g, const cd_opts &o, floa
         A.shield = shield;
         A.vec = (uintptr_t)n_h % 16 == 0;
         CD_CUDA(cudaFuncSetAttribute(learned_cell_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_cell));
-        const int grid = (int)std::min<int64_t>((A.ntiles + 1) / 2, sms);
+        const int grid = (int)std::min<int64_t>(A.ntiles, sms);
         LaunchScope ls(CD_K_LEARNED, s);
         learned_cell_tc<<<grid, kCellThreads, smem_cell, s>>>(A);
         CD_CHECK_LAUNCH();

@@ -255,3 +255,32 @@ def test_insitu_near_shells_from_the_tables(L, dset):
         want = T.column_density(geom.dirs, level[rows], ijk[rows], mode=oracle.MODE_INSITU)
         got = nh[torch.from_numpy(rows).cuda()].double().cpu().numpy()
         assert np.max(np.abs(got - want) / want) <= 1e-5
+
+
+@pytest.mark.parametrize("dset", [("mxn", 1, 8), ("mxn", 3, 8), ("mxn", 5, 8), ("healpix", 2, 0)])
+@pytest.mark.parametrize("L", [2, 3, 5, 6])
+def test_bf16_learned_columns_over_tiles_and_widths(L, dset):
+    # tiles of 128 leaves, one to several per CTA, half a tile at the smallest, and
+    # the widths of the direction groups, against the FP32 form: the 1.5e-2 of the
+    # BF16 form against the exact network with a correction of this size
+    rho = _rho(L, 31)
+    tree = colden.build_tree_uniform(torch.from_numpy(rho).cuda(), BOX)
+    geom = colden.precompute_geometry(*dset)
+    nd = geom.n_dir
+    net = colden.Net(nd, 128, synth.mlp_init(nd, 128, 6, out_scale=0.2))
+    x = torch.empty((tree.n_leaf, 8 * nd + 1), device="cuda")
+    colden.learned_features(tree, geom, x, None)
+    net.fit_normaliser(x)
+    out = {}
+    for prec in (colden.FP32, colden.BF16):
+        nh = torch.full((tree.n_leaf, nd), -1.0, device="cuda")
+        av, sh = torch.full_like(nh, -1.0), torch.full((tree.n_leaf,), -1.0, device="cuda")
+        colden.column_density(tree, geom, n_h=nh, a_v=av, shield=sh, net=net, precision=prec)
+        colden.device_status()
+        out[prec] = nh, sh
+    (want, want_sh), (got, got_sh) = out[colden.FP32], out[colden.BF16]
+    assert float(((got - want).abs() / want).max()) < 1.5e-2
+    assert float((got_sh - want_sh).abs().max()) < 2e-3
+    assert float((av.double() - got.double() / 1.87e21).abs().max() / av.double().max()) < 2e-7
+    sh_of = torch.exp(-2.5 * got.double() / 1.87e21).mean(1)
+    assert float((got_sh.double() - sh_of).abs().max()) < 1e-5
