@@ -266,8 +266,8 @@ struct OctArgs {
     float *ext;            // [n_oct][nd]
 };
 
-constexpr int kOctThreads = 384;                              // 12 warps
-constexpr int kOctUnits = 128 * kMaxNd / 8 / kOctThreads;   // (row, 8 directions) units per thread: 2
+constexpr int kOctThreads = 128 * kMaxNd / 8;                // a (row, 8 directions) unit each: 24 warps
+constexpr int kFarRows = 20;                                 // rows above a tile of octs: 16 + 2 + 1 + 1
 
 // Far slots of a tile of 128 consecutive octs o0 .. o0+127 (o0 a multiple of
 // 128): Delta_l = 4 reads the 16 parents o0/8 + r/8, Delta_l = 5 the 2
@@ -284,41 +284,86 @@ __device__ __forceinline__ float far_slot_entry(const OctArgs &A, int64_t o0, in
     return t;
 }
 
-size_t oct_smem(const TcLayout &T)
+// 32 bytes (one sector) in one access, 32-byte aligned.
+__device__ __forceinline__ void ld_sector(const float *src, float4 &a, float4 &b)
 {
-    return 2 * align128((size_t)128 * T.KE * 2) + (size_t)8 * kHBlock * 2 +
-           (size_t)(2 * T.KE + kH + 20 * T.nd) * 4 + 2 * 8 + 16;
+    asm("ld.global.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+        : "=f"(a.x), "=f"(a.y), "=f"(a.z), "=f"(a.w), "=f"(b.x), "=f"(b.y), "=f"(b.z), "=f"(b.w)
+        : "l"(src));
 }
 
+__device__ __forceinline__ void st_sector(float *dst, float4 a, float4 b)
+{
+    asm volatile("st.global.v8.f32 [%8], {%0, %1, %2, %3, %4, %5, %6, %7};" ::"f"(a.x), "f"(a.y), "f"(a.z), "f"(a.w),
+                 "f"(b.x), "f"(b.y), "f"(b.z), "f"(b.w), "l"(dst)
+                 : "memory");
+}
+
+struct OctSmem {
+    size_t b, h, mu, si, lo, b1, far, ufar, bar, total;   // the operand [128 x KE] at 0
+};
+
+__host__ __device__ inline OctSmem oct_smem(const TcLayout &T)
+{
+    OctSmem S;
+    size_t o = align128((size_t)128 * T.KE * 2);
+    auto take = [&](size_t bytes) { const size_t r = o; o = align128(o + bytes); return r; };
+    S.b = take((size_t)128 * T.KE * 2);
+    S.h = take((size_t)8 * kHBlock * 2);
+    S.mu = take((size_t)T.KE * 4);
+    S.si = take((size_t)T.KE * 4);
+    S.lo = take((size_t)T.KE * 2);
+    S.b1 = take(kH * 4);
+    S.far = take((size_t)kFarRows * T.nd * 4);
+    S.ufar = take((size_t)kFarRows * T.nd * 2);
+    S.bar = take(64);
+    S.total = o;
+    return S;
+}
+
+// A tile is 128 octs: u_ext straight into the operand layout, one chain of
+// MMAs, the epilogue.  What bounds it: these follow one another (operand and
+// weights, 84 KB each, leave room for one tile), so a tile's epilogue runs under the
+// next one's chain and its loads under the one before's; each part is spread
+// over 24 warps, a thread building one row's piece of 8 directions, and the slots
+// that the octs of a parent share (Delta_l >= 4) are standardised once per parent
+// and copied.  The tables come in whole sectors, 32 bytes a lane: with 16 the
+// loads alone kept the L1 busy for longer than the chain.  256^3 leaves, 48
+// directions: 1.13 -> 0.74 ms (12 warps, one after the other, a row a lane before);
+// its 2.1 GB take 0.31 ms at the copy rate.
 __global__ void __launch_bounds__(kOctThreads, 1) learned_oct_tc(OctArgs A)
 {
     extern __shared__ __align__(1024) unsigned char smem[];
     const TcLayout &T = A.T;
+    const OctSmem S = oct_smem(T);
     const int nd = T.nd, KE = T.KE;
-    unsigned char *sA = smem;                                    // [128 x KE] BF16 operand
-    unsigned char *sB = sA + align128((size_t)128 * KE * 2);     // W1e image
-    __nv_bfloat16 *sHb = reinterpret_cast<__nv_bfloat16 *>(sB + align128((size_t)128 * KE * 2));  // 8 h blocks
-    float *sMu = reinterpret_cast<float *>(sHb + 8 * kHBlock);  // [KE] standardisation a
-    float *sSi = sMu + KE;                                       // [KE] standardisation b
-    float *sB1 = sSi + KE;                                       // [128]
-    float *sT = sB1 + kH;                                        // [20][nd] far slots of the tile
-    uint64_t *bar = reinterpret_cast<uint64_t *>(sT + 20 * nd);  // [0] weights, [1] MMA
+    unsigned char *sA = smem, *sB = smem + S.b, *sHb = smem + S.h;   // [128 x KE] operand, W1e image, 8 h blocks
+    float *sMu = reinterpret_cast<float *>(smem + S.mu), *sSi = reinterpret_cast<float *>(smem + S.si);
+    __nv_bfloat16 *sLo = reinterpret_cast<__nv_bfloat16 *>(smem + S.lo);
+    float *sB1 = reinterpret_cast<float *>(smem + S.b1);             // [128]
+    float *sT = reinterpret_cast<float *>(smem + S.far);             // [20][nd] far slots of the tile
+    __nv_bfloat16 *sU = reinterpret_cast<__nv_bfloat16 *>(smem + S.ufar);   // the same, standardised
+    uint64_t *bar = reinterpret_cast<uint64_t *>(smem + S.bar);      // [0] weights, [1] MMA
     uint32_t *tslot = reinterpret_cast<uint32_t *>(bar + 2);
-    int *sflag = reinterpret_cast<int *>(tslot + 1);
+    int *sflag = reinterpret_cast<int *>(tslot + 1);                 // [2] by iteration parity: a wait was given up
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     if (tid == 0) {
         mbar_init(&bar[0], 1);
         mbar_init(&bar[1], 1);
         fence_mbar_init();
-        *sflag = 0;
+        sflag[0] = sflag[1] = 0;
     }
-    for (int i = tid; i < KE; i += kOctThreads) {
-        sMu[i] = reinterpret_cast<const float *>(A.tc + T.mue)[i];
-        sSi[i] = reinterpret_cast<const float *>(A.tc + T.sie)[i];
+    for (int k = tid; k < KE; k += kOctThreads) {
+        const float a = reinterpret_cast<const float *>(A.tc + T.mue)[k], b = reinterpret_cast<const float *>(A.tc + T.sie)[k];
+        sMu[k] = a;
+        sSi[k] = b;
+        sLo[k] = __float2bfloat16_rn(fmaxf(fmaf(a, fast_log2(kCFloor), b), -kUMax));
     }
     for (int i = tid; i < kH; i += kOctThreads) sB1[i] = reinterpret_cast<const float *>(A.tc + T.b1)[i];
-    if (warp == 0) tmem_alloc(tslot, 128);
+    for (int e = tid; e < 128 * (KE - 7 * nd) / 8; e += kOctThreads)   // K padding
+        *reinterpret_cast<uint4 *>(sA + op_off(e & 127, 7 * nd + 8 * (e >> 7), KE)) = make_uint4(0, 0, 0, 0);
+    if (warp == 0) tmem_alloc(tslot, 256);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -328,167 +373,173 @@ __global__ void __launch_bounds__(kOctThreads, 1) learned_oct_tc(OctArgs A)
         mbar_expect_tx(&bar[0], bytes);
         bulk_g2s(sB, A.tc + T.w1e, bytes, &bar[0]);
     }
-    bool weights_ready = false;
-    uint32_t phase = 0;
-    const int units = 128 * (nd / 8);
+    // this thread's unit: a row of the tile, 8 consecutive directions.  A warp
+    // takes 8 rows of 4 such pieces: runs of 128 bytes in the tables, and eight
+    // rows side by side in the operand (no bank conflicts)
+    const int piece = tid >> 3, r = 8 * (piece / (nd >> 3)) + (tid & 7), d0 = 8 * (piece % (nd >> 3));
+    const bool unit = r < 128;
+    // its entries of the far slots: row of sT, direction
+    constexpr int kFs = (kFarRows * kMaxNd + kOctThreads - 1) / kOctThreads;
+    int frow[kFs], fd[kFs];
+#pragma unroll
+    for (int q = 0; q < kFs; ++q) {
+        const int e = tid + q * kOctThreads;
+        frow[q] = e / nd;
+        fd[q] = e - frow[q] * nd;
+    }
 
-    // Software pipeline over tiles: the loads of tile k+1 (near slots into
-    // registers, far slots into registers) are issued right after tile k's
-    // operand is built, so they are in flight during tile k's MMA and epilogue.
-    float c[kOctUnits][3][8];
-    float fs[(20 * kMaxNd + kOctThreads - 1) / kOctThreads];
-    auto issue_loads = [&](int64_t tile) {
-        const int64_t o0 = tile * 128;
-        const int rows = (int)std::min<int64_t>(128, A.n_oct - o0);
-        // near slots (Delta_l = 1..3) of this thread's units: lanes take
-        // consecutive octs, each 8 consecutive directions (two 16-byte loads
-        // per table)
+    float4 c[3][2];
+    float fs[kFs];
+    auto issue_loads = [&](int64_t tile) {   // rows past the end repeat the last one
+        const int64_t o0 = tile * 128, o = std::min<int64_t>(o0 + r, A.n_oct - 1);
 #pragma unroll
-        for (int j = 0; j < kOctUnits; ++j) {
-            const int u = tid + j * kOctThreads;
-            const int r = u & 127, d0 = (u >> 7) * 8;
-            const bool ok = u < units && r < rows;
-#pragma unroll
-            for (int t = 0; t < 3; ++t) {
-                if (ok && t + 1 <= A.L - 1) {
-                    const float4 *src = reinterpret_cast<const float4 *>(A.Et[t + 1] + (o0 + r) * nd + d0);
-                    const float4 a = src[0], b = src[1];
-                    c[j][t][0] = a.x; c[j][t][1] = a.y; c[j][t][2] = a.z; c[j][t][3] = a.w;
-                    c[j][t][4] = b.x; c[j][t][5] = b.y; c[j][t][6] = b.z; c[j][t][7] = b.w;
-                } else {
-#pragma unroll
-                    for (int q = 0; q < 8; ++q) c[j][t][q] = 0.f;
-                }
+        for (int t = 0; t < 3; ++t) {
+            c[t][0] = c[t][1] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (unit && t + 1 <= A.L - 1) {
+                ld_sector(A.Et[t + 1] + o * nd + d0, c[t][0], c[t][1]);
             }
         }
-        // far slots shared by the tile
 #pragma unroll
-        for (int q = 0; q < (20 * kMaxNd + kOctThreads - 1) / kOctThreads; ++q) {
-            const int e = tid + q * kOctThreads;
-            fs[q] = e < 20 * nd ? far_slot_entry(A, o0, e / nd, e % nd, nd) : 0.f;
-        }
+        for (int q = 0; q < kFs; ++q) fs[q] = frow[q] < kFarRows ? far_slot_entry(A, o0, frow[q], fd[q], nd) : 0.f;
     };
-    if (blockIdx.x < A.ntiles) issue_loads(blockIdx.x);
+    const int64_t first = blockIdx.x, stride = gridDim.x;
+    const int n_tile = (int)((A.ntiles - first + stride - 1) / stride);   // at least 1
+    issue_loads(first);
+    bool ok = mbar_wait_bounded(&bar[0], 0, kMaxPolls), fault = false;
+    auto rows_of = [&](int64_t o0) { return (int)std::min<int64_t>(128, A.n_oct - o0); };
 
-    for (int64_t tile = blockIdx.x; tile < A.ntiles; tile += gridDim.x) {
-        const int64_t o0 = tile * 128;
-        const int rows = (int)std::min<int64_t>(128, A.n_oct - o0);
-#pragma unroll
-        for (int q = 0; q < (20 * kMaxNd + kOctThreads - 1) / kOctThreads; ++q) {
-            const int e = tid + q * kOctThreads;
-            if (e < 20 * nd) sT[e] = fs[q];
-        }
-        // the previous tile's h blocks must have been read out of sHb
-        if (tid == 0) bulk_wait_read<0>();
-        __syncthreads();
-        // 3. u_ext -> operand rows (16-byte stores, lanes on consecutive rows),
-        //    external column -> HBM
-#pragma unroll
-        for (int j = 0; j < kOctUnits; ++j) {
-            const int u = tid + j * kOctThreads;
-            if (u >= units) continue;
-            const int r = u & 127, d0 = (u >> 7) * 8;
-            const bool ok = r < rows;
-            float tot[8];
-#pragma unroll
-            for (int q = 0; q < 8; ++q) tot[q] = 0.f;
-#pragma unroll
-            for (int s = 0; s < 7; ++s) {
-                float cv[8], a[8], b[8], v[8];
-                if (s < 3) {
-#pragma unroll
-                    for (int q = 0; q < 8; ++q) cv[q] = c[j][s][q];
-                } else {
-                    const int row = s == 3 ? (r >> 3) : s == 4 ? 16 + (r >> 6) : s == 5 ? 18 : 19;
-                    const float4 x0 = *reinterpret_cast<const float4 *>(sT + row * nd + d0);
-                    const float4 x1 = *reinterpret_cast<const float4 *>(sT + row * nd + d0 + 4);
-                    cv[0] = x0.x; cv[1] = x0.y; cv[2] = x0.z; cv[3] = x0.w;
-                    cv[4] = x1.x; cv[5] = x1.y; cv[6] = x1.z; cv[7] = x1.w;
-                }
-                {
-                    const int k = s * nd + d0;
-                    const float4 a0 = *reinterpret_cast<const float4 *>(sMu + k), a1 = *reinterpret_cast<const float4 *>(sMu + k + 4);
-                    const float4 b0 = *reinterpret_cast<const float4 *>(sSi + k), b1 = *reinterpret_cast<const float4 *>(sSi + k + 4);
-                    a[0] = a0.x; a[1] = a0.y; a[2] = a0.z; a[3] = a0.w; a[4] = a1.x; a[5] = a1.y; a[6] = a1.z; a[7] = a1.w;
-                    b[0] = b0.x; b[1] = b0.y; b[2] = b0.z; b[3] = b0.w; b[4] = b1.x; b[5] = b1.y; b[6] = b1.z; b[7] = b1.w;
-                }
-#pragma unroll
-                for (int q = 0; q < 8; ++q) {
-                    tot[q] += cv[q];
-                    v[q] = ok ? std_input(cv[q], kCFloor, a[q], b[q]) : 0.f;
-                }
-                *reinterpret_cast<uint4 *>(sA + op_off(r, s * nd + d0, KE)) =
-                    make_uint4(pack_bf16x2(v[0], v[1]), pack_bf16x2(v[2], v[3]), pack_bf16x2(v[4], v[5]),
-                               pack_bf16x2(v[6], v[7]));
-            }
-            if (ok) {
-                float4 *dst = reinterpret_cast<float4 *>(A.ext + (o0 + r) * nd + d0);
-                dst[0] = make_float4(tot[0], tot[1], tot[2], tot[3]);
-                dst[1] = make_float4(tot[4], tot[5], tot[6], tot[7]);
-            }
-        }
-        for (int e = tid; e < 128 * (KE - 7 * nd); e += kOctThreads)   // K padding
-            *reinterpret_cast<__nv_bfloat16 *>(sA + op_off(e & 127, 7 * nd + (e >> 7), KE)) = __float2bfloat16_rn(0.f);
-        fence_proxy_async_smem();
-        tc_fence_before();
-        __syncthreads();
-        if (tile + gridDim.x < A.ntiles) issue_loads(tile + gridDim.x);   // in flight during MMA + epilogue
-        if (tid == 0) {
-            bool ok = true;
-            if (!weights_ready) ok = weights_ready = mbar_wait_bounded(&bar[0], 0, kMaxPolls);
-            if (ok) {
-                tc_fence_after();
-                mma_steps(tbase, smem_u32(sA), KE, smem_u32(sB), KE, KE / 16, kH, false);
-                umma_commit(&bar[1]);
-                ok = mbar_wait_bounded(&bar[1], phase, kMaxPolls);
-            }
-            if (!ok) *sflag = 1;
-        }
-        phase ^= 1;
-        __syncthreads();
-        if (*sflag) break;
+    int it = 0;
+    for (; it <= n_tile; ++it) {
+        const int64_t tile = first + it * stride, o0 = tile * 128;
+        const bool more = it < n_tile;
+        if (it > 0) ok = mbar_wait_bounded(&bar[1], (it - 1) & 1, kMaxPolls);   // the operand is free, D is complete
+        if (!ok) sflag[it & 1] = 1;
         tc_fence_after();
-        // 4. h = D + b1 -> the B-operand blocks of the per-leaf kernel: block
-        //    r / 16, element (n, r % 16); rows past the end are zero (a 0 x NaN
-        //    in the product would poison a real row).  Warps w, w + 4, w + 8
-        //    share TMEM lanes 32 (w % 4) .., taking columns 0-63, 64-95, 96-127.
-        {
-            const int quarter = warp & 3, part = warp >> 2;
-            const int r = quarter * 32 + lane;
-            unsigned char *blk = reinterpret_cast<unsigned char *>(sHb + (r >> 4) * kHBlock);
-            const int cbeg = part == 0 ? 0 : part == 1 ? 64 : 96, cend = part == 0 ? 64 : part == 1 ? 96 : 128;
-#pragma unroll 1
-            for (int c0 = cbeg; c0 < cend; c0 += 32) {
-                uint32_t v[32];
-                tmem_ld32(tbase + ((uint32_t)(quarter * 32) << 16) + (uint32_t)c0, v);
-                tmem_ld_wait();
+        float2 tot[4];
 #pragma unroll
-                for (int q = 0; q < 32; ++q) {
-                    const int n = c0 + q;
-                    const float hv = r < rows ? __uint_as_float(v[q]) + sB1[n] : 0.f;
-                    *reinterpret_cast<__nv_bfloat16 *>(blk + op_off(n, r & 15, 16)) = __float2bfloat16_rn(hv);
+        for (int p = 0; p < 4; ++p) tot[p] = make_float2(0.f, 0.f);
+        auto add = [&](float4 a, float4 b) {
+            tot[0] = __fadd2_rn(tot[0], make_float2(a.x, a.y));
+            tot[1] = __fadd2_rn(tot[1], make_float2(a.z, a.w));
+            tot[2] = __fadd2_rn(tot[2], make_float2(b.x, b.y));
+            tot[3] = __fadd2_rn(tot[3], make_float2(b.z, b.w));
+        };
+        if (more) {
+#pragma unroll
+            for (int q = 0; q < kFs; ++q) {
+                if (frow[q] < kFarRows) {
+                    const int e = tid + q * kOctThreads;
+                    const int k = (frow[q] < 16 ? 3 : frow[q] < 18 ? 4 : frow[q] - 13) * nd + fd[q];
+                    sT[e] = fs[q];
+                    sU[e] = __float2bfloat16_rn(std_input(fs[q], kCFloor, sMu[k], sSi[k]));
                 }
             }
+            // near slots -> operand rows
+            if (unit) {
+#pragma unroll
+                for (int s = 0; s < 3; ++s) {
+                    const float2 x[4] = {make_float2(c[s][0].x, c[s][0].y), make_float2(c[s][0].z, c[s][0].w),
+                                         make_float2(c[s][1].x, c[s][1].y), make_float2(c[s][1].z, c[s][1].w)};
+                    const int k = s * nd + d0;
+                    const uint4 lo = *reinterpret_cast<const uint4 *>(sLo + k);
+                    const uint32_t l[4] = {lo.x, lo.y, lo.z, lo.w};
+                    uint32_t v[4];
+#pragma unroll
+                    for (int p = 0; p < 4; ++p)
+                        v[p] = std_input2(x[p], *reinterpret_cast<const float2 *>(sMu + k + 2 * p),
+                                          *reinterpret_cast<const float2 *>(sSi + k + 2 * p), l[p]);
+                    *reinterpret_cast<uint4 *>(sA + op_off(r, k, KE)) = make_uint4(v[0], v[1], v[2], v[3]);
+                    add(c[s][0], c[s][1]);
+                }
+            }
+            if (it + 1 < n_tile) issue_loads(tile + stride);   // in flight until the next iteration
         }
         fence_proxy_async_smem();
         tc_fence_before();
         __syncthreads();
+        if (sflag[it & 1]) {
+            fault = true;
+            break;
+        }
+        if (tid == 0 && it > 1) {       // the h blocks of the last iteration's epilogue
+            const int64_t p0 = o0 - 2 * 128 * stride;
+            bulk_s2g(A.h + (p0 >> 4) * kHBlock, sHb, (uint32_t)((rows_of(p0) + 15) / 16 * kHBlock * 2));
+            bulk_commit();
+        }
+        // far slots: copies; the external column -> HBM
+        if (more && unit) {
+#pragma unroll
+            for (int s = 3; s < 7; ++s) {
+                const int e = (s == 3 ? (r >> 3) : s == 4 ? 16 + (r >> 6) : s == 5 ? 18 : 19) * nd + d0;
+                *reinterpret_cast<uint4 *>(sA + op_off(r, s * nd + d0, KE)) = *reinterpret_cast<const uint4 *>(sU + e);
+                add(*reinterpret_cast<const float4 *>(sT + e), *reinterpret_cast<const float4 *>(sT + e + 4));
+            }
+            if (o0 + r < A.n_oct) {
+                st_sector(A.ext + (o0 + r) * nd + d0, make_float4(tot[0].x, tot[0].y, tot[1].x, tot[1].y),
+                          make_float4(tot[2].x, tot[2].y, tot[3].x, tot[3].y));
+            }
+        }
+        if (tid == 0) bulk_wait_read<0>();   // sHb is free
+        fence_proxy_async_smem();
+        tc_fence_before();
+        __syncthreads();
+        tc_fence_after();
+        if (more && tid == 0) {
+            mma_steps(tbase + 128 * (it & 1), smem_u32(sA), KE, smem_u32(sB), KE, KE / 16, kH, false);
+            umma_commit(&bar[1]);
+        }
+        __syncwarp();
+        // Epilogue of the tile before: h = D + b1 -> the B-operand blocks of the
+        // per-leaf kernel, block r / 16, element (n, r % 16); rows past the end are
+        // zero (a 0 x NaN in the product would poison a real row).  Warps w,
+        // w + 4, .. share TMEM lanes 32 (w % 4) .. and take 8 columns in turn.  Two
+        // rows of one column make a word: even lanes store the even columns of a
+        // pair of rows, odd lanes the odd ones.
+        if (it > 0) {
+            const int quarter = warp & 3, row = quarter * 32 + lane;
+            const bool odd = lane & 1, live = row < rows_of(o0 - 128 * stride);
+            unsigned char *blk = sHb + (row >> 4) * kHBlock * 2;
+            const uint32_t src = tbase + 128 * ((it - 1) & 1) + ((uint32_t)(quarter * 32) << 16);
+#pragma unroll 1
+            for (int c0 = 8 * (warp >> 2); c0 < kH; c0 += 8 * (kOctThreads / 128)) {
+                uint32_t v[8];
+                tmem_ld8(src + (uint32_t)c0, v);
+                tmem_ld_wait(v);
+#pragma unroll
+                for (int p = 0; p < 4; ++p) {
+                    const float2 b = *reinterpret_cast<const float2 *>(sB1 + c0 + 2 * p);
+                    const float x = live ? __uint_as_float(v[2 * p]) + b.x : 0.f,
+                                y = live ? __uint_as_float(v[2 * p + 1]) + b.y : 0.f;
+                    const float got = __shfl_xor_sync(0xffffffffu, odd ? x : y, 1);
+                    *reinterpret_cast<uint32_t *>(blk + op_off(c0 + 2 * p + (odd ? 1 : 0), row & 14, 16)) =
+                        odd ? pack_bf16x2(got, y) : pack_bf16x2(x, got);
+                }
+            }
+        }
+    }
+    if (!fault) {
+        fence_proxy_async_smem();
+        tc_fence_before();
+        __syncthreads();
         if (tid == 0) {
-            const int nblk = (rows + 15) / 16;
-            bulk_s2g(A.h + (o0 >> 4) * kHBlock, sHb, (uint32_t)(nblk * kHBlock * 2));
+            const int64_t p0 = (first + (n_tile - 1) * stride) * 128;
+            bulk_s2g(A.h + (p0 >> 4) * kHBlock, sHb, (uint32_t)((rows_of(p0) + 15) / 16 * kHBlock * 2));
             bulk_commit();
         }
     }
-    if (*sflag && tid == 0) {
-        atomicExch(&g_ltc_fault, 1);
-        mbar_wait_bounded(&bar[1], phase ^ 1, kMaxPolls);   // let an issued chain finish
+    if (tid == 0) {
+        if (fault) {
+            atomicExch(&g_ltc_fault, 1);
+            mbar_wait_bounded(&bar[0], 0, kMaxPolls);
+            if (it > 0) mbar_wait_bounded(&bar[1], (it - 1) & 1, kMaxPolls);   // let an issued chain finish
+        }
+        bulk_wait_all<0>();
     }
-    if (tid == 0) bulk_wait_all<0>();
     tc_fence_before();
     __syncthreads();
     if (warp == 0) {
         tc_fence_after();
-        tmem_dealloc(tbase, 128);
+        tmem_dealloc(tbase, 256);
     }
 }
 
@@ -959,7 +1010,7 @@ cd_status column_density_learned_tc(cd_tree t, cd_geom g, const cd_opts &o, floa
     }
     const int sms = num_sms(), smax = max_smem_optin();
     const TcLayout lay = make_layout(nd);
-    const size_t smem_oct = oct_smem(lay), smem_cell = cell_smem(lay).total;
+    const size_t smem_oct = oct_smem(lay).total, smem_cell = cell_smem(lay).total;
     if ((int)smem_oct > smax || (int)smem_cell > smax) {
         set_error("the learned kernels need %zu / %zu bytes of shared memory, the device offers %d", smem_oct,
                   smem_cell, smax);
