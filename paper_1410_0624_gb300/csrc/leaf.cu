@@ -21,6 +21,7 @@
 // of them to a generic one-thread-per-leaf kernel.
 #include <algorithm>
 #include <mutex>
+#include <type_traits>
 
 #include "common.cuh"
 #include "ptx.cuh"
@@ -44,16 +45,23 @@ struct LeafTmaArgs {
     float inv_nd;
 };
 
-// W = lanes pre-reduced by shuffles before the shared-memory add of the
-// screening sum (a leaf's 4-direction slots are W-aligned runs of lanes).
-// W = lanes pre-reduced by shuffles before a leaf's screening partial goes to
-// shared memory (a leaf's 4-direction slots are W-aligned runs of lanes).  The
-// partials of batch i are summed in a fixed order while batch i+1 is computed
-// and their store trails the N_H store by one batch, so results are bitwise
-// reproducible with two barriers per batch.
+// A leaf's screening partials, one per slot, in shared memory: from three on padded
+// (with zeros) to an odd number of 16-byte words, so that a lane per leaf reads
+// them 16 bytes at a time without bank conflicts.
+__host__ __device__ constexpr int part_pitch(int nd) { return nd <= 8 ? nd / 4 : 4 * (((nd / 4 + 3) / 4) | 1); }
+
+// Thread group g takes octs 4 g .. 4 g + 3 of a batch: siblings, so their
+// parent's prefix is read once.  The screening partials of batch i are summed in a
+// fixed order while batch i+1 is computed and their store trails the N_H store
+// by one batch, so results are bitwise reproducible with two barriers per batch.
 // ND > 0 fixes the direction count at compile time (every offset folds to an
 // immediate); ND = 0 reads it from the arguments.
-template <int ND, int W>
+// What bounds it: issue slots (the product's 32 FMA2 cycles of some 60 a unit), two
+// barriers a batch and the N_H stores.  256^3 FP32 with N_H: 48 directions 0.804 ->
+// 0.686 ms (4.9 TB/s; the stores alone take 0.55), 40 directions 1.068 -> 0.706, 12
+// 0.222 -> 0.188, with a load of the prefix for every oct, a check of every output
+// in the loop and conflicts in the screening sums before.
+template <int ND>
 __global__ void __launch_bounds__(384, 2) leaf_tma(LeafTmaArgs P)
 {
     extern __shared__ __align__(128) unsigned char smem[];
@@ -62,15 +70,15 @@ __global__ void __launch_bounds__(384, 2) leaf_tma(LeafTmaArgs P)
     const int G = ND ? kG : P.G;
     const int B = ND ? 4 * kG : P.B;
     const int prows = ND ? (4 * kG) / 8 + 2 : P.prows;
-    const int q4 = nd >> 2, slots = 2 * nd, pw = slots / W, lw = q4 / W;
+    const int q4 = nd >> 2, slots = 2 * nd, lp = part_pitch(nd);
     const bool want_nh = P.a.n_h != nullptr, want_sh = P.a.shield != nullptr;
     uint64_t *bar = reinterpret_cast<uint64_t *>(smem);
     float *Eb = reinterpret_cast<float *>(smem + 128);      // [kLoadStages][B nd]
     float *Rb = Eb + kLoadStages * B * nd;                  // [kLoadStages][B 8]
     float *Pb = Rb + kLoadStages * B * 8;                   // [kLoadStages][(B/8 + 2) nd] parent rows
     float *Sb = Pb + kLoadStages * prows * nd;              // [3][B 8]
-    float *part = Sb + 3 * B * 8;                           // [2][B][slots / W]
-    float *Ob = part + 2 * B * pw;                          // [2][B 8 nd]
+    float *part = Sb + 3 * B * 8;                           // [2][B 8][lp]
+    float *Ob = part + 2 * B * 8 * lp;                      // [2][B 8 nd]
 
     const int tid = threadIdx.x;
     const int g = tid / slots, r = tid - g * slots;
@@ -84,11 +92,10 @@ __global__ void __launch_bounds__(384, 2) leaf_tma(LeafTmaArgs P)
             KP[j][i] = make_float2(P.a.dx_leaf * P.a.kloc[(t * 8 + 2 * j) * nd + d0 + i],
                                    P.a.dx_leaf * P.a.kloc[(t * 8 + 2 * j + 1) * nd + d0 + i]);
 
-    // this thread's offsets in the stages (oct g of the batch) and the strides
-    // to its next octs g + G, g + 2G, g + 3G (B = 4G)
+    // this thread's offsets in the stages (oct 4 g of the batch, the next three follow)
     const bool has_E = P.a.E != nullptr, has_Sp = P.a.Sp != nullptr;
-    const int eoff = g * nd + d0, roff = g * 8, ooff = (g * 8 + t) * nd + d0, poff = g * pw + r / W;
-    const int sE = G * nd, sR = G * 8, sO = G * 8 * nd, sP = G * pw;
+    const int b0 = 4 * g, eoff = b0 * nd + d0, roff = b0 * 8, ooff = (b0 * 8 + t) * nd + d0,
+              poff = (b0 * 8 + t) * lp + (d0 >> 2);
 
     const int64_t n_oct = P.a.n_oct;
     const int64_t first = blockIdx.x, stride = gridDim.x;
@@ -119,15 +126,23 @@ __global__ void __launch_bounds__(384, 2) leaf_tma(LeafTmaArgs P)
     };
     // screening factor of batch `it` from its partials, in a fixed order
     auto shield_sum = [&](int it) {
-        const float *pp = part + (it & 1) * B * pw;
+        const float *pp = part + (it & 1) * B * 8 * lp;
         float *S = Sb + (it % 3) * B * 8;
-        for (int j = tid; j < batch_nb(it) * 8; j += blockDim.x) {
-            const float *p = pp + (j >> 3) * pw + (j & 7) * lw;
-            float acc = 0.f;
-            for (int q = 0; q < lw; ++q) acc += p[q];
-            S[j] = acc * P.inv_nd;
+        for (int j = tid; j < B * 8; j += blockDim.x) {
+            if (nd <= 8) {
+                S[j] = (nd == 4 ? pp[j] : pp[2 * j] + pp[2 * j + 1]) * P.inv_nd;
+                continue;
+            }
+            float2 acc = make_float2(0.f, 0.f);
+            for (int q = 0; q < lp; q += 4) {
+                const float4 p = *reinterpret_cast<const float4 *>(pp + j * lp + q);
+                acc = __fadd2_rn(acc, __fadd2_rn(make_float2(p.x, p.y), make_float2(p.z, p.w)));
+            }
+            S[j] = (acc.x + acc.y) * P.inv_nd;
         }
     };
+    for (int j = tid; j < 2 * B * 8; j += blockDim.x)
+        for (int q = q4; q < lp; ++q) part[j * lp + q] = 0.f;
 
     if (tid == 0) {
         for (int s = 0; s < kLoadStages; ++s) mbar_init(&bar[s], 1);
@@ -155,32 +170,37 @@ __global__ void __launch_bounds__(384, 2) leaf_tma(LeafTmaArgs P)
 
         const int64_t o0 = batch_o0(it);
         const int nb = batch_nb(it);
-        // 32-bit shared-memory bases of this thread's slot in every stage
         const float *E = Eb + ls * B * nd + eoff;
-        const float *Spr = Pb + ls * prows * nd + d0;
         const float *R = Rb + ls * B * 8 + roff;
         float *O = Ob + os * B * 8 * nd + ooff;
-        float *pp = part + (it & 1) * B * pw + poff;
-        const int par0 = (int)(o0 & 7);           // parent row of oct b: (par0 + b) >> 3
+        float *pp = part + (it & 1) * B * 8 * lp + poff;
         float *AV = P.a.a_v ? P.a.a_v + o0 * 8 * nd + ooff : nullptr;
+        float2 s01 = make_float2(0.f, 0.f), s23 = s01;
+        if (has_Sp) {   // octs o0 + 4 g .. have one parent (o0 is a multiple of 4)
+            const float4 p4 = *reinterpret_cast<const float4 *>(
+                Pb + ls * prows * nd + (((int)(o0 & 7) + b0) >> 3) * nd + d0);
+            s01 = make_float2(p4.x, p4.y);
+            s23 = make_float2(p4.z, p4.w);
+        }
+        // all: a whole batch with E, Sp and the screening factor, without A_V (the
+        // checks of the other forms cost a seventh); rows: N_H is wanted
+        const auto octs = [&](auto all, auto rows) {
+            constexpr bool kAll = decltype(all)::value;
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            const int b = g + k * G;
-            const bool live = nb == B || b < nb;
-            float2 n01 = make_float2(0.f, 0.f), n23 = make_float2(0.f, 0.f);
-            if (live) {
-                if (has_E) {
-                    const float4 e4 = *reinterpret_cast<const float4 *>(E + k * sE);
+            for (int k = 0; k < 4; ++k) {
+                if (!kAll && b0 + k >= nb) break;
+                float2 n01 = make_float2(0.f, 0.f), n23 = n01;
+                if (kAll || has_E) {
+                    const float4 e4 = *reinterpret_cast<const float4 *>(E + k * nd);
                     n01 = make_float2(e4.x, e4.y);
                     n23 = make_float2(e4.z, e4.w);
                 }
-                if (has_Sp) {
-                    const float4 p4 = *reinterpret_cast<const float4 *>(Spr + ((par0 + b) >> 3) * nd);
-                    n01 = __fadd2_rn(n01, make_float2(p4.x, p4.y));
-                    n23 = __fadd2_rn(n23, make_float2(p4.z, p4.w));
+                if (kAll || has_Sp) {
+                    n01 = __fadd2_rn(n01, s01);
+                    n23 = __fadd2_rn(n23, s23);
                 }
-                const float4 r0 = *reinterpret_cast<const float4 *>(R + k * sR);
-                const float4 r1 = *reinterpret_cast<const float4 *>(R + k * sR + 4);
+                const float4 r0 = *reinterpret_cast<const float4 *>(R + k * 8);
+                const float4 r1 = *reinterpret_cast<const float4 *>(R + k * 8 + 4);
                 // packed FP32x2 FMAs over sibling pairs (s, s+1): acc[i] holds the
                 // even- and odd-sibling partial sums of direction d0 + i
                 const float2 rp[4] = {make_float2(r0.x, r0.y), make_float2(r0.z, r0.w), make_float2(r1.x, r1.y),
@@ -196,23 +216,27 @@ __global__ void __launch_bounds__(384, 2) leaf_tma(LeafTmaArgs P)
                 n01.y += acc[1].x + acc[1].y;
                 n23.x += acc[2].x + acc[2].y;
                 n23.y += acc[3].x + acc[3].y;
-                if (want_nh) *reinterpret_cast<float4 *>(O + k * sO) = make_float4(n01.x, n01.y, n23.x, n23.y);
-                if (AV) {
+                if (rows)
+                    *reinterpret_cast<float4 *>(O + k * 8 * nd) = make_float4(n01.x, n01.y, n23.x, n23.y);
+                if (!kAll && AV) {
                     const float2 a2 = make_float2(P.a.av_per_nh, P.a.av_per_nh);
                     const float2 x = __fmul2_rn(n01, a2), y = __fmul2_rn(n23, a2);
-                    *reinterpret_cast<float4 *>(AV + k * sO) = make_float4(x.x, x.y, y.x, y.y);
+                    *reinterpret_cast<float4 *>(AV + k * 8 * nd) = make_float4(x.x, x.y, y.x, y.y);
+                }
+                if (kAll || want_sh) {
+                    // exp(-k A_V) = 2^(c2 N_H), c2 = -k av log2(e) precomputed on the host
+                    const float2 c2 = make_float2(P.c_exp2, P.c_exp2);
+                    const float2 a = __fmul2_rn(c2, n01), b = __fmul2_rn(c2, n23);
+                    pp[k * 8 * lp] = (exp2f(a.x) + exp2f(a.y)) + (exp2f(b.x) + exp2f(b.y));
                 }
             }
-            if (want_sh) {
-                // exp(-k A_V) = 2^(c2 N_H), c2 = -k av log2(e) precomputed on the host
-                const float2 c2 = make_float2(P.c_exp2, P.c_exp2);
-                const float2 a = __fmul2_rn(c2, n01), bb = __fmul2_rn(c2, n23);
-                float e = (exp2f(a.x) + exp2f(a.y)) + (exp2f(bb.x) + exp2f(bb.y));
-#pragma unroll
-                for (int w = 1; w < W; w <<= 1) e += __shfl_xor_sync(0xffffffffu, e, w);
-                pp[k * sP] = e;
-            }
-        }
+        };
+        // (a third copy of the loop pays with runtime offsets alone: 40 directions
+        // of 256^3 0.706 against 0.759 ms, 48 at compile time 0.709 against 0.686)
+        if (nb != B || !has_E || !has_Sp || !want_sh || AV) octs(std::false_type{}, want_nh);
+        else if (ND) octs(std::true_type{}, want_nh);
+        else if (want_nh) octs(std::true_type{}, std::true_type{});
+        else octs(std::true_type{}, std::false_type{});
         fence_proxy_async_smem();
         __syncthreads();
         if (tid == 0) {
@@ -400,11 +424,16 @@ cd_status launch_leaf(const LeafLaunch &a, cudaStream_t s)
     const bool tma = (nd % 4 == 0) && 2 * nd <= 384 && aligned16(a.n_h) && aligned16(a.a_v) &&
                      aligned16(a.shield) && aligned16(a.E) && aligned16(a.Sp) && aligned16(a.rho_leaf);
     if (tma) {
-        const int W = 1;
-        auto kern = nd == 48 ? leaf_tma<48, 1> : nd == 12 ? leaf_tma<12, 1> : leaf_tma<0, 1>;
+        auto kern = nd == 48 ? leaf_tma<48> : nd == 12 ? leaf_tma<12> : leaf_tma<0>;
         LeafTmaArgs P;
         P.a = a;
         P.G = std::max(1, 384 / (2 * nd));
+        // small trees: smaller batches, so that every SM gets one (16^3, 48 directions,
+        // the whole evaluation as a graph 16.4 -> 14.4 us, 12 directions the same)
+        while (P.G > 1 && P.G * nd >= 96 && a.n_oct < (int64_t)4 * P.G * sm_count()) {
+            P.G /= 2;
+            kern = leaf_tma<0>;
+        }
         P.B = 4 * P.G;
         P.prows = P.B / 8 + 2;
         P.nbatch = (a.n_oct + P.B - 1) / P.B;
@@ -412,7 +441,7 @@ cd_status launch_leaf(const LeafLaunch &a, cudaStream_t s)
         P.inv_nd = inv_nd;
         const int threads = P.G * 2 * nd;
         const size_t smem = 128 + sizeof(float) * ((size_t)kLoadStages * (P.B * (nd + 8) + (size_t)P.prows * nd) + 3 * P.B * 8 +
-                                                   (size_t)2 * P.B * (2 * nd / W) +
+                                                   (size_t)2 * P.B * 8 * part_pitch(nd) +
                                                    (a.n_h ? (size_t)2 * P.B * 8 * nd : 0));
         CD_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
         int per_sm = 0;

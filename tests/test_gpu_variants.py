@@ -284,3 +284,32 @@ def test_bf16_learned_columns_over_tiles_and_widths(L, dset):
     assert float((av.double() - got.double() / 1.87e21).abs().max() / av.double().max()) < 2e-7
     sh_of = torch.exp(-2.5 * got.double() / 1.87e21).mean(1)
     assert float((got_sh.double() - sh_of).abs().max()) < 1e-5
+
+
+@pytest.mark.parametrize("dset", [("mxn", 1, 4), ("mxn", 2, 4), ("mxn", 3, 4), ("mxn", 4, 4), ("mxn", 5, 4), ("mxn", 4, 8),
+                                  ("healpix", 2, 0), ("mxn", 7, 12), ("mxn", 12, 16)])
+@pytest.mark.parametrize("L", [1, 2, 3, 5])
+def test_fp32_leaves_in_fours(L, dset):
+    # whole and partial batches of octs, padded screening sums, with and without the
+    # prefix of the parents: every combination of outputs against the oracle (FP32
+    # sums to 1e-5, as the path's other tests) and against each other
+    rho = _rho(L, 41)
+    n = 8 ** L
+    tree = colden.build_tree_uniform(torch.from_numpy(rho).cuda(), BOX)
+    geom = colden.precompute_geometry(*dset)
+    nd = geom.n_dir
+    new = lambda *s: torch.full(s, -1.0, device="cuda")  # noqa: E731
+    nh, sh, nh2, sh2, av2, only, alone = new(n, nd), new(n), new(n, nd), new(n), new(n, nd), new(n), new(n, nd)
+    colden.column_density(tree, geom, n_h=nh, shield=sh)
+    colden.column_density(tree, geom, n_h=nh2, a_v=av2, shield=sh2)
+    colden.column_density(tree, geom, shield=only)
+    colden.column_density(tree, geom, n_h=alone)
+    colden.device_status()
+    assert torch.equal(nh, nh2) and torch.equal(nh, alone) and torch.equal(sh, sh2) and torch.equal(sh, only)
+    rows = np.arange(n) if n <= 4096 else np.unique(np.random.default_rng(L).integers(0, n, 1500))
+    want = oracle.Tree.uniform(rho, BOX).column_density(geom.dirs, np.full(len(rows), L), oracle.morton_ijk(L)[rows])
+    at = torch.from_numpy(rows).cuda()
+    got = nh[at].double().cpu().numpy()
+    assert np.max(np.abs(got - want) / want) <= 1e-5
+    assert np.max(np.abs(av2[at].double().cpu().numpy() - oracle.a_v(got)) / oracle.a_v(got)) < 1e-6
+    assert np.max(np.abs(sh[at].double().cpu().numpy() - oracle.shield(want))) <= 1e-5
