@@ -478,7 +478,11 @@ cd_status build_row_lists(cd_geom g, cudaStream_t s)
 
 cd_status launch_ext_fp32(const ExtLaunch &a, cd_geom g, cudaStream_t s)
 {
-    if (ext_fp32_serves_list(a.k, a.tmask, g)) return launch_rows(a, g, s);
+    // 16^3 receivers are eight rows of each of 64 classes, too few for the row form
+    // (evaluations of 32^3 replayed as graphs, row against block form: 12
+    // directions 22.5 and 18.5 us, 84 directions 37.0 and 28.8, 40
+    // cone-averaged ones 48.3 and 35.4; at 64^3 48 directions take 43 and 64)
+    if ((a.list || a.k > 4) && ext_fp32_serves_list(a.k, a.tmask, g)) return launch_rows(a, g, s);
     if (a.list) {
         set_error("the FP32 block form serves whole levels only");
         return CD_EUNSUPPORTED;
