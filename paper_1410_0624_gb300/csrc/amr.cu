@@ -905,7 +905,10 @@ cd_status column_density_amr(cd_tree t, cd_geom g, const cd_opts &opts, float *n
     // far-shell prefixes of the refined cells
     for (int k = 3; k <= L - 2 && !insitu; ++k) {
         if (!t->n_ref[k]) continue;
-        if ((tc || ext_fp32_serves_list(k, 4, g)) && k >= 4 && t->tc_ref[k].ntiles) {
+        // a fully refined level (below the base level) keeps every cell in Morton
+        // order, so it takes the whole-level forms of a uniform tree
+        const TcList *list = t->n_ref[k] == ((int64_t)1 << (3 * k)) ? nullptr : &t->tc_ref[k];
+        if ((tc || !list || ext_fp32_serves_list(k, 4, g, list)) && k >= 4 && t->tc_ref[k].ntiles) {
             ExtLaunch e = {};
             e.k = k;
             e.nd = nd;
@@ -914,9 +917,7 @@ cd_status column_density_amr(cd_tree t, cd_geom g, const cd_opts &opts, float *n
             e.dx[3] = dx(k - 2);
             e.prefix_in = (k - 1 >= 3) ? t->ws.S[k - 1] : nullptr;
             e.out = t->ws.S[k];
-            // a fully refined level (below the base level) keeps every cell in Morton
-            // order, so it takes the whole-level tiles of a uniform tree
-            e.list = t->n_ref[k] == ((int64_t)1 << (3 * k)) ? nullptr : &t->tc_ref[k];
+            e.list = list;
             const cd_status st = tc ? launch_ext_tc(e, t->rho_brick, g, s) : launch_ext_fp32(e, g, s);
             if (st != CD_OK) return st;
             CD_CUDA(cudaEventRecord(t->ev_S[k], s));
@@ -956,7 +957,7 @@ cd_status column_density_amr(cd_tree t, cd_geom g, const cd_opts &opts, float *n
             have_E[k] = true;
             continue;
         }
-        if ((tc || ext_fp32_serves_list(k, 7, g)) && k >= 4 && t->tc_oct[k].ntiles) {
+        if ((tc || ext_fp32_serves_list(k, 7, g, &t->tc_oct[k])) && k >= 4 && t->tc_oct[k].ntiles) {
             ExtLaunch e = {};
             e.k = k;
             e.nd = nd;

@@ -127,7 +127,8 @@ __global__ void __launch_bounds__(kExtThreads) shell_sum_fp32(ExtArgs P)
 // instructions an output row, entries read by every warp), the entries from L1
 // instead of the ring 0.68 (their latency).
 constexpr int kRowThreads = 512, kRowPitch = 36, kRowCells = CD_STENCIL, kRingQuads = 4;
-constexpr int kRowMinEntries = 48;   // directions x longest row
+constexpr int kRowMinEntries = 48;       // directions x longest row
+constexpr int kRowMinReceivers = 1024;   // of a list
 
 struct RowArgs {
     int k, nd;
@@ -441,13 +442,21 @@ cd_status launch_rows(const ExtLaunch &a, cd_geom g, cudaStream_t s)
 
 }  // namespace
 
-bool ext_fp32_serves_list(int k, int tmask, cd_geom g)
+bool ext_fp32_serves_list(int k, int tmask, cd_geom g, const TcList *list)
 {
     // with hardly anything to sum (the six axis rays have three entries at most)
     // staging a parent's stencils costs more than the block form's gathers
     // (64^3: 24.6 against 23.1 us; 12 HEALPix directions 24.4 against 28.7)
     const int li = row_list(tmask);
-    return k >= 4 && li >= 0 && g->rows[li].quad != nullptr && g->n_dir * g->maxe >= kRowMinEntries;
+    if (k < 4 || li < 0 || g->rows[li].quad == nullptr || g->n_dir * g->maxe < kRowMinEntries) return false;
+    // A CTA reads its class's entries for 32 cells: too few receivers per class
+    // leave it little to share them with.  The whole level of 16^3 has eight parents in
+    // each of 64 classes (evaluations of 32^3 replayed as graphs, row against block
+    // form: 12 directions 22.5 and 18.5 us, 84 directions 37.0 and 28.8, 40
+    // cone-averaged ones 48.3 and 35.4; at 64^3 48 directions take 43 and 64).  Lists
+    // have a slower alternative: 84 directions of a mesh of 16^3 with 288 octs one
+    // level up 65.7 and 55.4 us, of 32^3 with 2 230 66.1 and 78.0.
+    return list ? list->n_recv >= kRowMinReceivers : k > 4;
 }
 
 cd_status build_row_lists(cd_geom g, cudaStream_t s)
@@ -478,11 +487,7 @@ cd_status build_row_lists(cd_geom g, cudaStream_t s)
 
 cd_status launch_ext_fp32(const ExtLaunch &a, cd_geom g, cudaStream_t s)
 {
-    // 16^3 receivers are eight rows of each of 64 classes, too few for the row form
-    // (evaluations of 32^3 replayed as graphs, row against block form: 12
-    // directions 22.5 and 18.5 us, 84 directions 37.0 and 28.8, 40
-    // cone-averaged ones 48.3 and 35.4; at 64^3 48 directions take 43 and 64)
-    if ((a.list || a.k > 4) && ext_fp32_serves_list(a.k, a.tmask, g)) return launch_rows(a, g, s);
+    if (ext_fp32_serves_list(a.k, a.tmask, g, a.list)) return launch_rows(a, g, s);
     if (a.list) {
         set_error("the FP32 block form serves whole levels only");
         return CD_EUNSUPPORTED;

@@ -403,9 +403,10 @@ struct ExtLaunch {
     int tiles_per_cta;        // tensor-core form: 0 = persistent CTAs (two per SM); n = one CTA per n tiles
 };
 cd_status launch_ext_fp32(const ExtLaunch &a, cd_geom g, cudaStream_t s);
-// whether launch_ext_fp32 takes the row form for receivers of level k with these
-// tables (lists have no other form there: the caller goes to its own kernel)
-bool ext_fp32_serves_list(int k, int tmask, cd_geom g);
+// whether launch_ext_fp32 takes the row form for these receivers of level k (a
+// list, or NULL for the whole level) with these tables; lists have no other form
+// there: the caller goes to its own kernel
+bool ext_fp32_serves_list(int k, int tmask, cd_geom g, const TcList *list);
 // the chunk lists of the tables (after build_geometry_tables)
 cd_status build_row_lists(cd_geom g, cudaStream_t s);
 
