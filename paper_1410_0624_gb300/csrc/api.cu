@@ -131,12 +131,12 @@ static cd_status ensure_side_streams(cd_tree t)
     return CD_OK;
 }
 
-SideFork::SideFork(cd_tree t, cudaStream_t s) : t_(t), s_(s)
+SideFork::SideFork(cd_tree t, cudaStream_t s, bool alone) : t_(t), s_(s)
 {
     // the events exist in both modes: the callers record and wait on them
     // unconditionally (on s alone they order nothing new)
     st_ = ensure_side_streams(t);
-    serial_ = stats_timing();
+    serial_ = alone || stats_timing();
     if (st_ != CD_OK || serial_) {
         joined_ = true;   // nothing was forked
         return;
@@ -554,7 +554,18 @@ static cd_status evaluate(cd_tree tree, cd_geom geom, const cd_opts *opts_in, fl
     // 0 in launches of kOctTilesPerCta tiles per CTA, while the far-shell prefix
     // chain (S_k needs S_{k-1}) runs on side stream 1, the high-priority one, so
     // its CTAs take SMs as the oct level's retire; the leaves wait for both.
-    SideFork fork(tree, s);
+    // Up to 16^3 there is no chain, and for 32^3 it is one launch of 512 cells: the
+    // host is the slower side there, and ordering the side streams costs it more
+    // than they gain, unless the call is being captured or the rows are long
+    // (eager calls with and without: 16^3, 48 directions 24.8 and 23.1 us; 32^3,
+    // 12 directions 29.5 and 28.1, 48 directions 31.1 and 32.9)
+    bool alone = false;
+    if (L < 5 || (L == 5 && nd * geom->maxe <= 160)) {
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        CD_CUDA(cudaStreamIsCapturing(s, &cap));
+        alone = cap == cudaStreamCaptureStatusNone;
+    }
+    SideFork fork(tree, s, alone);
     if ((st = fork.status()) != CD_OK) return st;
     cudaStream_t s_oct = fork.side(0), s_chain = fork.side(1);
     for (int k = 3; k <= L - 2; ++k) {

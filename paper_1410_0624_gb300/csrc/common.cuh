@@ -338,7 +338,8 @@ void stats_add(const int64_t *count, const double *flops, int sign = 1);
 // order, so that each launch's events time that launch alone.
 class SideFork {
   public:
-    SideFork(cd_tree t, cudaStream_t s);
+    // alone: nothing to gain from the side streams, everything stays on s
+    SideFork(cd_tree t, cudaStream_t s, bool alone = false);
     ~SideFork();
     SideFork(const SideFork &) = delete;
     SideFork &operator=(const SideFork &) = delete;

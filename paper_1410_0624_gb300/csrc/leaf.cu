@@ -443,9 +443,9 @@ cd_status launch_leaf(const LeafLaunch &a, cudaStream_t s)
         const size_t smem = 128 + sizeof(float) * ((size_t)kLoadStages * (P.B * (nd + 8) + (size_t)P.prows * nd) + 3 * P.B * 8 +
                                                    (size_t)2 * P.B * 8 * part_pitch(nd) +
                                                    (a.n_h ? (size_t)2 * P.B * 8 * nd : 0));
-        CD_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        int per_sm = 0;
-        CD_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem));
+        if (smem > 48 * 1024) CD_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        int per_sm = 1;
+        if (P.nbatch > sm_count()) CD_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem));
         if (per_sm < 1) per_sm = 1;
         const int64_t grid = std::min<int64_t>(P.nbatch, (int64_t)per_sm * sm_count());
         LaunchScope ls(CD_K_LEAF, s);
