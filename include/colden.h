@@ -70,9 +70,10 @@ enum {
 enum {
     CD_MODE_PREC = 0,      /* precalculation module, two-level approximation: the shell at level l is seen from
                               the centre of the target's ancestor at level min(l+2, l0-1) */
-    CD_MODE_INSITU = 1,    /* every shell seen from the oct centre: an exact walk over each shell's cells per
-                              (oct, direction) on the CUDA cores, FP32 whatever cd_opts.precision says; no far-shell
-                              sharing, so it costs more (§4.3, Table 1) */
+    CD_MODE_INSITU = 1,    /* every shell seen from the oct centre, on the CUDA cores, FP32 whatever
+                              cd_opts.precision says: the three nearest shells from the tables (seen from there
+                              anyway), the coarser ones by an exact walk over their cells per (oct, direction);
+                              no far-shell sharing, so it costs more (§4.3, Table 1) */
     CD_MODE_CONE = 2       /* as CD_MODE_PREC, but every geometric factor (shell tables, Kloc, BF16 operands) is
                               the mean over the 32 sub-rays of the direction's cone (below) instead of the value
                               of one ray; the evaluation costs the same, only wider rows of the FP32 tables */
@@ -163,7 +164,7 @@ cd_status cd_tree_update(cd_tree tree, const float *rho, int rho_on_device, void
  *   scheme         CD_DIRS_*; p0, p1 as documented there
  *   dirs           CD_DIRS_CUSTOM only: n_custom x 3 doubles (host)
  *   mode           CD_MODE_PREC, CD_MODE_INSITU (the tables are built either way; in-situ
- *                  evaluations use only the local ones) or CD_MODE_CONE (tables averaged
+ *                  evaluations use the local ones and those of the three nearest shells) or CD_MODE_CONE (tables averaged
  *                  over each direction's cone)
  * 1 <= number of directions <= 768.  Components below 1e-14 in magnitude are
  * set to zero and each vector renormalised.  The tables are built on
@@ -442,13 +443,13 @@ void cd_debug_leaf_span(int rows);
  * indices of their gathers and stores before each access; one that falls
  * outside what it addresses is skipped and recorded (first failure wins) in
  * a device error word, with no trap.  Sites:
- *   11 FP32 shell kernel: stencil offset from the tables within the staged
- *      density region;  12: output row;  13: far-shell prefix row
+ *   11 FP32 shell kernels: stencil offset from the tables within the staged
+ *      densities;  12: output row;  13: far-shell prefix row
  *   21 tensor-core shell kernel: brick index of an A-operand gather
  *   31 tensor-core leaf kernel: a tile's octs (E, densities) and parents (S)
  *   32 tensor-core leaf kernel: output row (N_H, A_V, screening factor)
- *   41 FP32 leaf kernel: a batch's octs and parents
- *   51 AMR list shell kernel: stencil offset within the stencil region
+ *   41 FP32 leaf kernels: a batch's octs and parents
+ *   51 FP32 list shells: stencil offset within the stencil region or dense level
  *    1 cd_debug_check_probe
  * cd_checked_status synchronises the device and returns, in *site and
  * *index, the first failure since the last call (0 and 0 when none), then

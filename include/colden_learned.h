@@ -159,8 +159,9 @@ cd_status cd_net_info(cd_net net, int *n_dir, int *hidden, int64_t *num_params);
 void cd_net_free(cd_net net);
 
 /* The learned form of cd_column_density: set cd_opts.net to a cd_net whose
- * n_dir equals the geometry's.  CD_FP32 runs features, the FP32 network and
- * the correction in chunks of leaves; CD_BF16 runs them in one fused kernel
+ * n_dir equals the geometry's.  CD_FP32 runs features, the FP32 network (the
+ * external slots' part of layer 1 once per oct) and the correction in chunks
+ * of leaves; CD_BF16 runs them in one fused kernel
  * on the tcgen05 tensor cores (BF16 weights and activations, FP32
  * accumulation) where the sizes allow (see colden.h, cd_column_density). */
 

@@ -1,7 +1,7 @@
 // FP32 CUDA-core forms of the shell contraction (Eq. N_discret, one level of
-// receiving cells per launch): the row form below serves receiving levels >= 4
-// and lists, the block form the few cells of coarser levels and runs of tables
-// the row form has no list for.  For every cell c at level k and direction d:
+// receiving cells per launch): the row form below serves whole levels above 16^3
+// and lists of enough receivers, the block form the few cells of coarser levels
+// and what the row form has no lists for.  For every cell c at level k and direction d:
 //   out[c][d] = prefix_in[parent(c)][d]
 //             + sum_{t in tmask} dx_{k-t+1} sum_s rho_{k-t+1}(stencil_t(c), s) K_t[cfg_t(c)][d][s]
 // with the 6^3 stencil of table t anchored at the ancestor A_{k-t} of c and
@@ -462,7 +462,8 @@ bool ext_fp32_serves_list(int k, int tmask, cd_geom g, const TcList *list)
 cd_status build_row_lists(cd_geom g, cudaStream_t s)
 {
     // rows of a list are as wide as the largest counts allow; direction sets
-    // whose lists would take more than 256 MB stay with the tables alone
+    // whose lists would take more than 256 MB, or find no room, stay with the
+    // tables alone
     constexpr size_t kMaxBytes = (size_t)256 << 20;
     for (int i = 0; i < 4; ++i) {
         cd_geom_s::RowList &L = g->rows[i];
@@ -473,9 +474,11 @@ cd_status build_row_lists(cd_geom g, cudaStream_t s)
         if (quads * sizeof(RowQuad) > kMaxBytes) continue;
         if (cudaMalloc(&L.quad, quads * sizeof(RowQuad)) != cudaSuccess ||
             cudaMalloc(&L.start, sizeof(int) * ncfg * (nq + 1)) != cudaSuccess) {
-            cudaGetLastError();
-            set_error("cannot allocate the shell row lists (%zu bytes)", quads * sizeof(RowQuad));
-            return CD_ENOMEM;
+            cudaGetLastError();           // no room: the other forms serve these tables
+            if (L.quad) cd::lib_free(L.quad);
+            L.quad = nullptr;
+            L.start = nullptr;
+            continue;
         }
         LaunchScope ls(CD_K_OTHER, s);
         row_lists<<<(unsigned)((ncfg + 3) / 4), 128, 0, s>>>(i, g->n_dir, ncfg, g->tab[1], g->tab[2], g->tab[3], g->maxe,
