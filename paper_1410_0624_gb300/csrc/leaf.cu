@@ -53,14 +53,16 @@ __host__ __device__ constexpr int part_pitch(int nd) { return nd <= 8 ? nd / 4 :
 // Thread group g takes octs 4 g .. 4 g + 3 of a batch: siblings, so their
 // parent's prefix is read once.  The screening partials of batch i are summed in a
 // fixed order while batch i+1 is computed and their store trails the N_H store
-// by one batch, so results are bitwise reproducible with two barriers per batch.
+// by one batch, so results are bitwise reproducible with one barrier per batch (it also
+// says whether any thread gave up its wait for the batch's inputs).
 // ND > 0 fixes the direction count at compile time (every offset folds to an
 // immediate); ND = 0 reads it from the arguments.
-// What bounds it: issue slots (the product's 32 FMA2 cycles of some 60 a unit), two
-// barriers a batch and the N_H stores.  256^3 FP32 with N_H: 48 directions 0.804 ->
-// 0.686 ms (4.9 TB/s; the stores alone take 0.55), 40 directions 1.068 -> 0.706, 12
-// 0.222 -> 0.188, with a load of the prefix for every oct, a check of every output
-// in the loop and conflicts in the screening sums before.
+// What bounds it: issue slots (the product's 32 FMA2 cycles of some 60 a unit), the
+// barrier of a batch and the N_H stores.  256^3 FP32 with N_H: 48 directions 0.804 ->
+// 0.653 ms (5.2 TB/s; the stores alone take 0.55), 40 directions 1.068 -> 0.668, 84
+// 2.342 -> 1.373, 12 0.222 -> 0.180, with a load of the prefix for every oct, a check
+// of every output in the loop, conflicts in the screening sums and a second barrier
+// (one thread polled for the inputs: 0.696, 0.704, 1.553 and 0.192) before.
 template <int ND>
 __global__ void __launch_bounds__(384, 2) leaf_tma(LeafTmaArgs P)
 {
@@ -155,17 +157,9 @@ __global__ void __launch_bounds__(384, 2) leaf_tma(LeafTmaArgs P)
     bool fault = false;
     for (; it < n_iter; ++it) {
         const int ls = it % kLoadStages, os = it & 1;
-        if (tid == 0) {
-            if (it + kLoadStages - 1 < n_iter) issue(it + kLoadStages - 1);
-            bulk_wait_read<1>();   // stores issued two iterations ago have read O[os] and their S
-        }
-        // one thread polls; the others sleep in the hardware barrier
-        bool ok = true;
-        if (tid == 0) ok = mbar_wait_bounded(&bar[ls], (it / kLoadStages) & 1, kMaxPolls);
-        if (__syncthreads_or(!ok)) {
-            fault = true;
-            break;
-        }
+        // the stage of batch it - 1 is free: every thread has passed its barrier
+        if (tid == 0 && it + kLoadStages - 1 < n_iter) issue(it + kLoadStages - 1);
+        const bool ok = mbar_wait_bounded(&bar[ls], (it / kLoadStages) & 1, kMaxPolls);
         if (want_sh && it > 0) shield_sum(it - 1);
 
         const int64_t o0 = batch_o0(it);
@@ -232,15 +226,20 @@ __global__ void __launch_bounds__(384, 2) leaf_tma(LeafTmaArgs P)
             }
         };
         // (a third copy of the loop pays with runtime offsets alone: 40 directions
-        // of 256^3 0.706 against 0.759 ms, 48 at compile time 0.709 against 0.686)
+        // of 256^3 0.706 against 0.759 ms, 48 at compile time 0.709 against 0.686, both
+        // with a second barrier)
         if (nb != B || !has_E || !has_Sp || !want_sh || AV) octs(std::false_type{}, want_nh);
         else if (ND) octs(std::true_type{}, want_nh);
         else if (want_nh) octs(std::true_type{}, std::true_type{});
         else octs(std::true_type{}, std::false_type{});
+        if (tid == 0) bulk_wait_read<0>();   // the last batch's stores have read O[os ^ 1] and their S
         fence_proxy_async_smem();
-        __syncthreads();
+        if (__syncthreads_or(!ok)) {
+            fault = true;
+            break;
+        }
         if (tid == 0) {
-            if (want_nh) bulk_s2g(P.a.n_h + o0 * 8 * nd, O, (uint32_t)nb * 32 * nd);
+            if (want_nh) bulk_s2g(P.a.n_h + o0 * 8 * nd, Ob + os * B * 8 * nd, (uint32_t)nb * 32 * nd);
             if (want_sh && it > 0)
                 bulk_s2g(P.a.shield + batch_o0(it - 1) * 8, Sb + ((it - 1) % 3) * B * 8, (uint32_t)batch_nb(it - 1) * 32);
             bulk_commit();
@@ -263,7 +262,7 @@ __global__ void __launch_bounds__(384, 2) leaf_tma(LeafTmaArgs P)
         if (fault) {
             atomicExch(&g_leaf_fault, 1);
             // let the loads already issued land before shared memory is released
-            for (int j = it; j < it + kLoadStages - 1 && j < n_iter; ++j)
+            for (int j = it; j < it + kLoadStages && j < n_iter; ++j)
                 mbar_wait_bounded(&bar[j % kLoadStages], (j / kLoadStages) & 1, kMaxPolls);
         }
         bulk_wait_all<0>();
