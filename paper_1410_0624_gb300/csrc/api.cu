@@ -562,8 +562,8 @@ static cd_status evaluate(cd_tree tree, cd_geom geom, const cd_opts *opts_in, fl
     bool alone = false;
     if (L < 5 || (L == 5 && nd * geom->maxe <= 160)) {
         cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-        CD_CUDA(cudaStreamIsCapturing(s, &cap));
-        alone = cap == cudaStreamCaptureStatusNone;
+        if (cudaStreamIsCapturing(s, &cap) == cudaSuccess) alone = cap == cudaStreamCaptureStatusNone;
+        else cudaGetLastError();   // a stream that cannot be asked: the fork says what is wrong with it
     }
     SideFork fork(tree, s, alone);
     if ((st = fork.status()) != CD_OK) return st;
