@@ -109,12 +109,19 @@ __device__ __forceinline__ int frag(int t, int i)
 // waited for between two barriers; 8 192 rows (64 x 64 tiles): 32 against
 // 45 us.  Moving the standardisation into the copies of layer 1 made them wait
 // for their loads again (67 us at 8 192 rows); a fourth stage changed nothing.
-template <int BM, int BN, int TM, int TN, int FA, int FB, int EPI>
+// KS = 2 gives a tile two sets of threads, each with half of every slab's k; the
+// second set's sums are added at the end.  The 32 x 32 tiles of small batches take
+// it: one set is two warps, too few to hide a slab's reads (gradient and Adam
+// steps of 256 rows, 48 directions, 192 units: 132 -> 115 us; 2 000 rows 194 -> 183).  In
+// 64 x 64 tiles it loses (8 192 rows, 128 units: 283 against 296 us).
+template <int BM, int BN, int TM, int TN, int FA, int FB, int EPI, int KS = 1>
 __device__ __forceinline__ void gemm_tile(const Gemm &g, int bm, int bn, int z, TileSmem<BM, BN> &sm)
 {
-    constexpr int THREADS = (BM / TM) * (BN / TN);
+    constexpr int SET = (BM / TM) * (BN / TN), THREADS = KS * SET;
     static_assert(TM % 4 == 0 && TN % 4 == 0, "fragments of four");
-    const int tid = threadIdx.x, tx = tid % (BN / TN), ty = tid / (BN / TN);
+    static_assert(KS == 1 || (KS == 2 && sizeof(TileSmem<BM, BN>) >= BM * BN * sizeof(float)), "room for a set's sums");
+    const int tid = threadIdx.x, set = KS == 1 ? 0 : tid / SET, at = KS == 1 ? tid : tid % SET;
+    const int tx = at % (BN / TN), ty = at / (BN / TN);
     const int m0 = bm * BM, n0 = bn * BN;
     const int kb = z * g.kps, ke = min(g.K, kb + g.kps);
     float2 acc[TM / 2][TN];                // pairs of rows
@@ -140,7 +147,8 @@ __device__ __forceinline__ void gemm_tile(const Gemm &g, int bm, int bn, int z, 
         __syncthreads();   // slab k0 has landed for every thread, and the slab before it is done with
         issue(k0 + (kGemmStages - 1) * BK, cur == 0 ? kGemmStages - 1 : cur - 1);
 #pragma unroll 4
-        for (int kk = 0; kk < BK; ++kk) {
+        for (int q = 0; q < BK / KS; ++q) {
+            const int kk = set * (BK / KS) + q;
             float4 b[TN / 4];
 #pragma unroll
             for (int j = 0; j < TN; j += 4)
@@ -165,6 +173,21 @@ __device__ __forceinline__ void gemm_tile(const Gemm &g, int bm, int bn, int z, 
         cur = cur + 1 == kGemmStages ? 0 : cur + 1;
     }
 
+    if (KS == 2) {
+        float2 *sums = reinterpret_cast<float2 *>(&sm);
+        __syncthreads();                   // the slabs are done with
+#pragma unroll
+        for (int i = 0; i < TM / 2; ++i)
+#pragma unroll
+            for (int j = 0; j < TN; ++j)
+                if (set) sums[(i * TN + j) * SET + at] = acc[i][j];
+        __syncthreads();
+#pragma unroll
+        for (int i = 0; i < TM / 2; ++i)
+#pragma unroll
+            for (int j = 0; j < TN; ++j)
+                if (!set) acc[i][j] = __fadd2_rn(acc[i][j], sums[(i * TN + j) * SET + at]);
+    }
     if (want_rsum && tid < BM && m0 + tid < g.M) g.rowsum[(int64_t)z * g.split_stride + m0 + tid] = rsum;
     float *C = g.C + (int64_t)z * g.split_stride;
     const bool vec = g.ldc % 4 == 0 && ((uintptr_t)C & 15) == 0 &&
@@ -173,7 +196,7 @@ __device__ __forceinline__ void gemm_tile(const Gemm &g, int bm, int bn, int z, 
 #pragma unroll
     for (int i = 0; i < TM; ++i) {
         const int m = m0 + frag<BM, TM>(ty, i);
-        if (m >= g.M) continue;
+        if (m >= g.M || set) continue;
         const int64_t src = EPI == EPI_RESIDUAL && g.rows ? g.rows[m] : (int64_t)m;
 #pragma unroll
         for (int j = 0; j < TN; j += 4) {
@@ -231,24 +254,25 @@ __device__ __forceinline__ void gemm_tile(const Gemm &g, int bm, int bn, int z, 
     }
 }
 
-template <int BM, int BN, int TM, int TN, int FA, int FB, int EPI>
-__global__ void __launch_bounds__((BM / TM) * (BN / TN), BM == 128 ? 2 : 4) sgemm(const __grid_constant__ Gemm g)
+template <int BM, int BN, int TM, int TN, int FA, int FB, int EPI, int KS>
+__global__ void __launch_bounds__(KS * (BM / TM) * (BN / TN), BM == 128 ? 2 : 4)
+    sgemm(const __grid_constant__ Gemm g)
 {
     extern __shared__ __align__(16) unsigned char smem[];
     TileSmem<BM, BN> &sm = *reinterpret_cast<TileSmem<BM, BN> *>(smem);
     const int ntn = (g.N + BN - 1) / BN;
-    gemm_tile<BM, BN, TM, TN, FA, FB, EPI>(g, (int)(blockIdx.x / ntn), (int)(blockIdx.x % ntn), 0, sm);
+    gemm_tile<BM, BN, TM, TN, FA, FB, EPI, KS>(g, (int)(blockIdx.x / ntn), (int)(blockIdx.x % ntn), 0, sm);
 }
 
-template <int BM, int BN, int TM, int TN, int FA, int FB, int EPI>
+template <int BM, int BN, int TM, int TN, int FA, int FB, int EPI, int KS = 1>
 cd_status launch_gemm(const Gemm &g, cudaStream_t s)
 {
     const int64_t tiles = (int64_t)((g.M + BM - 1) / BM) * ((g.N + BN - 1) / BN);
     constexpr int smem = sizeof(TileSmem<BM, BN>);
     if (smem > 48 * 1024)
-        CD_CUDA(cudaFuncSetAttribute(sgemm<BM, BN, TM, TN, FA, FB, EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+        CD_CUDA(cudaFuncSetAttribute(sgemm<BM, BN, TM, TN, FA, FB, EPI, KS>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
     LaunchScope ls(CD_K_NET, s);
-    sgemm<BM, BN, TM, TN, FA, FB, EPI><<<(unsigned)tiles, (BM / TM) * (BN / TN), smem, s>>>(g);
+    sgemm<BM, BN, TM, TN, FA, FB, EPI, KS><<<(unsigned)tiles, KS * (BM / TM) * (BN / TN), smem, s>>>(g);
     CD_CHECK_LAUNCH();
     return CD_OK;
 }
@@ -277,7 +301,7 @@ cd_status run_gemm(Gemm g, cudaStream_t s)
     if (g.M <= 0 || g.N <= 0) return CD_OK;
     g.kps = 1 << 30;
     const TileShape t = tile_shape(g.M, g.N);
-    if (t.bm == 32) return launch_gemm<32, 32, 4, 4, FA, FB, EPI>(g, s);
+    if (t.bm == 32) return launch_gemm<32, 32, 4, 4, FA, FB, EPI, 2>(g, s);
     if (t.bm == 64) return launch_gemm<64, 64, 8, 4, FA, FB, EPI>(g, s);
     if (t.bn == 48) return launch_gemm<128, 48, 8, 4, FA, FB, EPI>(g, s);
     if (t.bn == 64) return launch_gemm<128, 64, 8, 4, FA, FB, EPI>(g, s);
