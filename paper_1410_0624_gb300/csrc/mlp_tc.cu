@@ -1008,6 +1008,12 @@ cd_status column_density_learned_tc(cd_tree t, cd_geom g, const cd_opts &o, floa
         set_error("the BF16 learned form needs at least two tree levels");
         return CD_EUNSUPPORTED;
     }
+    // the kernels index the tables, the scratch and the outputs, all sized by the
+    // geometry, with the network's direction count
+    if (net->lay.nd != nd) {
+        set_error("the network has %d directions, the geometry %d", net->lay.nd, nd);
+        return CD_EINVAL;
+    }
     const int sms = num_sms(), smax = max_smem_optin();
     const TcLayout lay = make_layout(nd);
     const size_t smem_oct = oct_smem(lay).total, smem_cell = cell_smem(lay).total;

@@ -495,6 +495,23 @@ def test_learned_rejects_mismatched_directions_and_amr():
     assert e.value.code == colden.CD_EUNSUPPORTED
 
 
+@pytest.mark.parametrize("precision", [colden.FP32, colden.BF16])
+@pytest.mark.parametrize("n_net,n_geom", [(48, 8), (48, 24), (8, 48), (24, 40)])
+def test_learned_refuses_a_network_of_other_directions_in_both_precisions(n_net, n_geom, precision):
+    # sizes that either form takes when the two agree: refused before anything is launched
+    _, tree, _, _ = _setup(4, 94)
+    geom = colden.precompute_geometry("mxn", n_geom // 8, 8)
+    net, _ = _net(n_net, 128)
+    n_h = torch.full((tree.n_leaf * n_geom,), -1.0, device="cuda")
+    torch.cuda.synchronize()
+    colden.stats_reset()
+    with pytest.raises(colden.ColdenError) as e:
+        colden.column_density(tree, geom, n_h=n_h, net=net, precision=precision)
+    assert e.value.code == colden.CD_EINVAL and "directions" in str(e.value)
+    assert sum(colden.stats_get(k)[0] for k in range(len(colden.KERNEL_KINDS))) == 0
+    assert bool((n_h == -1.0).all())
+
+
 # ---------------------------------------------------------------------------
 # What the trained network gains over the plain tree method
 # ---------------------------------------------------------------------------
