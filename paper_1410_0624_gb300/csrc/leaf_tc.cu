@@ -682,7 +682,10 @@ __global__ void __launch_bounds__(128 * LeafOctShape<ND>::kGroups, 1) leaf_oct_t
     extern __shared__ __align__(1024) unsigned char smem[];
     __shared__ uint64_t bar[3 * S::kGroups];      // [g] products, [G + 2 g + stage] input stages
     __shared__ uint32_t tslot;
-    __shared__ int sflag[S::kGroups];
+    // [0] an input wait, [1] a product wait was given up.  Two flags: a slow warp may still
+    // read a tile's last product flag when thread 0 gives up the next tile's input wait,
+    // and either flag is read before a barrier that comes before its next write
+    __shared__ int sflag[S::kGroups][2];
     const int tid = threadIdx.x, warp = tid >> 5, g = warp >> 2, quarter = warp & 3, i = tid & 127;
     const int G = blockDim.x >> 7;
     unsigned char *sA = smem + S::kB + (size_t)g * S::kGroup;
@@ -709,7 +712,7 @@ __global__ void __launch_bounds__(128 * LeafOctShape<ND>::kGroups, 1) leaf_oct_t
     if (tid == 0) {
         for (int b = 0; b < 3 * S::kGroups; ++b) mbar_init(&bar[b], 1);
         fence_mbar_init();
-        for (int q = 0; q < S::kGroups; ++q) sflag[q] = 0;
+        for (int q = 0; q < S::kGroups; ++q) sflag[q][0] = sflag[q][1] = 0;
     }
     for (int n = tid; n < S::N; n += blockDim.x) {
         const float *k = P.a.kloc + (n / ND) * 8 * ND + n % ND;
@@ -745,11 +748,11 @@ __global__ void __launch_bounds__(128 * LeafOctShape<ND>::kGroups, 1) leaf_oct_t
                 pending[s] = false;
                 sphase[s] ^= 1;
             } else {
-                sflag[g] = 1;
+                sflag[g][0] = 1;
             }
         }
         named_barrier(1 + g, 128);
-        if (sflag[g]) {
+        if (sflag[g][0]) {
             fault = true;
             break;
         }
@@ -801,11 +804,11 @@ __global__ void __launch_bounds__(128 * LeafOctShape<ND>::kGroups, 1) leaf_oct_t
                     umma_bf16(tD, umma_smem_desc(smem_u32(sA), 128, 256), umma_smem_desc(smem_u32(smem) + c * 32, 128, 256),
                               umma_idesc_bf16(128, S::kN), 0u);
                     umma_commit(&bar[g]);
-                    if (!mbar_wait_bounded(&bar[g], phase, P.pipe_polls)) sflag[g] = 1;
+                    if (!mbar_wait_bounded(&bar[g], phase, P.pipe_polls)) sflag[g][1] = 1;
                 }
                 phase ^= 1;
                 named_barrier(1 + g, 128);
-                if (sflag[g]) {
+                if (sflag[g][1]) {
                     fault = true;
                     break;
                 }

@@ -56,3 +56,45 @@ def test_bounded_wait_runs_out_and_the_context_recovers():
     colden.device_status()
     rows = np.random.default_rng(3).choice(tree.n_leaf, size=300, replace=False)
     _oracle_check(tree, rho, n_h, sh, nd, rows)
+
+
+def _give_up(call, limits):
+    """`call` under poll limits that let its waits run out at the first tile, at
+    a later one or not at all: it returns, and reports what happened."""
+    codes = []
+    colden.device_status()                      # no flag left over from earlier work
+    try:
+        for polls in limits:
+            colden.debug_wait_polls(polls)
+            call()
+            try:
+                colden.device_status()
+                codes.append(0)
+            except colden.ColdenError as e:
+                assert e.code == colden.CD_ETIMEOUT and "bounded wait" in str(e)
+                codes.append(e.code)
+    finally:
+        colden.debug_wait_polls(-1)
+    return codes
+
+
+@pytest.mark.parametrize("dset,rows", [(("mxn", 1, 4), True), (("healpix", 1), True), (("mxn", 4, 8), True),
+                                       (("mxn", 5, 8), False), (("mxn", 8, 8), False)])
+def test_waits_of_the_oct_form_run_out_at_any_tile(dset, rows):
+    # leaves by octs: many tiles a group, one product each or two (beyond 32
+    # directions); the evaluation after it is the one before it
+    rho = synth.lognormal_iid(256, 10.0, 1.0, seed=62)
+    tree = colden.build_tree_uniform(torch.from_numpy(rho).cuda(), BOX)
+    geom = colden.precompute_geometry(*dset)
+    n_h = torch.full((tree.n_leaf, geom.n_dir), -1.0, device="cuda") if rows else None
+    sh = torch.full((tree.n_leaf,), -1.0, device="cuda")
+    call = lambda: colden.column_density(tree, geom, n_h=n_h, shield=sh, precision=colden.BF16)  # noqa: E731
+    call()
+    colden.device_status()
+    want = sh.clone(), n_h.clone() if rows else None
+    codes = _give_up(call, [0, 1, 2, 3, 5, 8, 0, 13, 1, 2])
+    assert codes[0] == codes[6] == colden.CD_ETIMEOUT
+    sh.fill_(-1.0)
+    call()
+    colden.device_status()
+    assert torch.equal(sh, want[0]) and (not rows or torch.equal(n_h, want[1]))
