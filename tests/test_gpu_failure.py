@@ -98,3 +98,43 @@ def test_waits_of_the_oct_form_run_out_at_any_tile(dset, rows):
     call()
     colden.device_status()
     assert torch.equal(sh, want[0]) and (not rows or torch.equal(n_h, want[1]))
+
+
+@pytest.mark.parametrize("kind,ndir", [("uniform", 36), ("uniform", 48), ("list", 12), ("list", 48), ("list", 64),
+                                       ("unprefixed", 48), ("batch", 48)])
+def test_waits_of_the_tiles_of_128_leaves_run_out_at_any_tile(kind, ndir):
+    # uniform trees with rows beyond 32 directions, adaptive lists (with the parents'
+    # prefix and, directly under the base level, without) and the persistent batch
+    geom = colden.precompute_geometry("mxn", ndir // 4, 4)
+    if kind == "uniform":
+        trees = [colden.build_tree_uniform(torch.from_numpy(synth.lognormal_iid(64, 10.0, 1.0, seed=63)).cuda(), BOX)]
+    else:
+        n, base = (32, 4) if kind == "unprefixed" else (128, 5)
+        fine = synth.lognormal_iid(n, 10.0, 1.0, seed=64)
+        fine[: n // 2, : n // 2] *= 20.0
+        lv = synth.amr_leaves(fine, base, [40.0] if n == 32 else [40.0, 200.0])
+        trees = [colden.build_tree_amr(lv["base"], lv["lmax"], BOX, lv["level"], lv["ijk"], lv["rho"])
+                 for _ in range(2 if kind == "batch" else 1)]
+    outs = [torch.full((t.n_leaf, ndir), -1.0, device="cuda") for t in trees]
+    if kind == "batch":
+        colden.debug_batch_form(1)
+        b = colden.Batch(trees, [geom] * 2, n_h=outs, precision=colden.BF16)
+        assert b.info()["persistent"]
+        call = b.run
+        colden.stats_reset(timing=True)         # its launches one by one, not the captured graph
+    else:
+        call = lambda: colden.column_density(trees[0], geom, n_h=outs[0], precision=colden.BF16)  # noqa: E731
+    try:
+        call()
+        colden.device_status()
+        want = [o.clone() for o in outs]
+        codes = _give_up(call, [0, 1, 2, 3, 5, 8, 0])
+        assert codes[0] == codes[-1] == colden.CD_ETIMEOUT
+        for o in outs:
+            o.fill_(-1.0)
+        call()
+        colden.device_status()
+        assert all(torch.equal(o, w) for o, w in zip(outs, want))
+    finally:
+        colden.debug_batch_form(-1)
+        colden.stats_reset(timing=False)
