@@ -1001,9 +1001,7 @@ cd_status column_density_amr(cd_tree t, cd_geom g, const cd_opts &opts, float *n
     // leaves: the 16-lanes-per-oct kernel when 16-byte rows are possible
     const bool vec = nd % 4 == 0 && (uintptr_t)n_h % 16 == 0 && (uintptr_t)a_v % 16 == 0;
     const size_t smem = sizeof(float) * (vec ? 64 * nd + 8 * 2 * nd : 64 * nd + 64 * nd);
-    if (smem > 48 * 1024)
-        CD_CUDA(cudaFuncSetAttribute(vec ? leaf_list : leaf_list_scalar, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)smem));
+    CD_ALLOW_SMEM(vec ? leaf_list : leaf_list_scalar, smem, kSmemOptin);
     for (int k = 0; k <= L - 1; ++k) {
         const int64_t no = t->oct_begin[k + 1] - t->oct_begin[k];
         if (!no) continue;

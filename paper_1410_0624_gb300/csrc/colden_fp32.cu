@@ -433,7 +433,7 @@ cd_status launch_rows(const ExtLaunch &a, cd_geom g, cudaStream_t s)
     if (grid == 0) return CD_OK;
     const size_t smem = row_smem(A.nt);
     const auto kern = a.list ? shell_rows_fp32<true> : shell_rows_fp32<false>;
-    CD_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)row_smem(3)));
+    CD_ALLOW_SMEM(kern, smem, row_smem(3));
     LaunchScope ls(CD_K_SHELL, s);
     kern<<<(unsigned)grid, kRowThreads, smem, s>>>(A);
     CD_CHECK_LAUNCH();

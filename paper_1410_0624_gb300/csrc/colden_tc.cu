@@ -715,7 +715,7 @@ cd_status launch_ext_tc(const ExtLaunch &a, const __nv_bfloat16 *const *brick, c
         if (P.ntiles == 0) return CD_OK;
     }
     const size_t smem = tc_smem_bytes((size_t)P.Nt * kChunkBricks * 16, false);
-    CD_CUDA(cudaFuncSetAttribute(shell_sum_tc<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    CD_ALLOW_SMEM(shell_sum_tc<false>, smem, tc_smem_bytes((size_t)kTmemCols * kChunkBricks * 16, false));
     // persistent CTAs hold every SM until the last tile; n tiles per CTA let the
     // CTAs of other streams' launches in as these retire
     const int64_t grid = a.tiles_per_cta > 0 ? (P.ntiles + a.tiles_per_cta - 1) / a.tiles_per_cta
@@ -819,7 +819,7 @@ cd_status launch_tc_batch(const void *jobs, const int2 *tile_ref, int64_t total,
     Bt.claim = claim;
     Bt.bstage_max = bstage_max;
     const size_t smem = tc_smem_bytes(bstage_max, true);
-    CD_CUDA(cudaFuncSetAttribute(shell_sum_tc<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    CD_ALLOW_SMEM(shell_sum_tc<true>, smem, tc_smem_bytes((size_t)kTmemCols * kChunkBricks * 16, true));
     // two CTAs per SM need the largest shared-memory carveout
     CD_CUDA(cudaFuncSetAttribute(shell_sum_tc<true>, cudaFuncAttributePreferredSharedMemoryCarveout,
                                  (int)cudaSharedmemCarveoutMaxShared));

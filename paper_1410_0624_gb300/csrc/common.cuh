@@ -84,6 +84,19 @@ constexpr int kRegionTotal = 12 * 12 * 12 + 8 * 8 * 8 + 6 * 6 * 6;
         }                                                                              \
     } while (0)
 
+// Shared memory above 48 KB (some of it static) has to be allowed per kernel, and
+// a launch that asks for more than was allowed last fails.  The attribute is shared by all
+// host threads, so every launch of a kernel allows the same amount, the most
+// that any of its sizes takes: one that allowed its own would fail a larger launch of
+// another thread.
+#define CD_ALLOW_SMEM(kern, smem, most)                                                \
+    do {                                                                               \
+        if ((size_t)(smem) > 40 * 1024)                                                \
+            CD_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, \
+                                         (int)((size_t)(smem) > (size_t)(most) ? (smem) : (most)))); \
+    } while (0)
+constexpr size_t kSmemOptin = 227 * 1024;   // of a block on sm_103a
+
 #define CD_CHECK_LAUNCH()                                                              \
     do {                                                                               \
         cudaError_t e_ = cudaGetLastError();                                           \

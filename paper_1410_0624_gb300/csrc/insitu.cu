@@ -56,6 +56,9 @@ __device__ __forceinline__ float box_exit(const float p[3], const float u[3], co
 
 constexpr int kOctsPerCta = 32;   // a lane each
 
+// directions and reciprocals, the octs' sums
+constexpr size_t insitu_smem(int nc) { return sizeof(float) * (6 * (size_t)nc + kOctsPerCta * (size_t)(nc | 1)); }
+
 __global__ void __launch_bounds__(256) insitu_external(const __grid_constant__ InsituArgs A)
 {
     extern __shared__ float s_dir[];     // [nc][6]: direction and reciprocals (0 where a component is 0)
@@ -204,8 +207,8 @@ cd_status launch_insitu(cd_tree t, cd_geom g, int k, int64_t n, const uint64_t *
     const dim3 grid((unsigned)std::max<int64_t>(blocks, 1), (unsigned)((g->n_dir + A.chunk - 1) / A.chunk));
     const int nc = std::min(A.chunk, g->n_dir);
     LaunchScope ls(CD_K_SHELL, s);
-    const size_t smem = sizeof(float) * (6 * (size_t)nc + kOctsPerCta * (size_t)(nc | 1));
-    CD_CUDA(cudaFuncSetAttribute(insitu_external, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    const size_t smem = insitu_smem(nc);
+    CD_ALLOW_SMEM(insitu_external, smem, insitu_smem(CD_MAXDIR));
     insitu_external<<<grid, 32 * std::min(8, nc), smem, s>>>(A);
     CD_CHECK_LAUNCH();
     return CD_OK;

@@ -50,6 +50,27 @@ struct LeafTmaArgs {
 // them 16 bytes at a time without bank conflicts.
 __host__ __device__ constexpr int part_pitch(int nd) { return nd <= 8 ? nd / 4 : 4 * (((nd / 4 + 3) / 4) | 1); }
 
+// shared memory of G groups: the input stages, the screening sums and partials, the
+// rows of two batches if they are wanted
+constexpr size_t leaf_tma_smem(int nd, int G, bool rows)
+{
+    const size_t B = 4 * (size_t)G, prows = B / 8 + 2;
+    return 128 + sizeof(float) * (kLoadStages * (B * (nd + 8) + prows * nd) + 3 * B * 8 + 2 * B * 8 * part_pitch(nd) +
+                                  (rows ? 2 * B * 8 * nd : 0));
+}
+
+constexpr int leaf_tma_groups(int nd) { return 384 / (2 * nd) > 1 ? 384 / (2 * nd) : 1; }
+
+constexpr size_t leaf_tma_smem_most()
+{
+    size_t most = 0;
+    for (int nd = 4; 2 * nd <= 384; nd += 4) {
+        const size_t v = leaf_tma_smem(nd, leaf_tma_groups(nd), true);
+        most = v > most ? v : most;
+    }
+    return most;
+}
+
 // Thread group g takes octs 4 g .. 4 g + 3 of a batch: siblings, so their
 // parent's prefix is read once.  The screening partials of batch i are summed in a
 // fixed order while batch i+1 is computed and their store trails the N_H store
@@ -67,7 +88,7 @@ template <int ND>
 __global__ void __launch_bounds__(384, 2) leaf_tma(LeafTmaArgs P)
 {
     extern __shared__ __align__(128) unsigned char smem[];
-    constexpr int kG = ND ? (384 / (2 * ND) > 1 ? 384 / (2 * ND) : 1) : 0;
+    constexpr int kG = ND ? leaf_tma_groups(ND ? ND : 1) : 0;
     const int nd = ND ? ND : P.a.nd;
     const int G = ND ? kG : P.G;
     const int B = ND ? 4 * kG : P.B;
@@ -313,6 +334,7 @@ __global__ void __launch_bounds__(256) leaf_generic(LeafLaunch P, float c_exp, f
 // a store) and takes 1.83, at 81 directions 14.6 and 4.7, of 64^3 at 9
 // directions 32 and 25 us.
 constexpr int kOctWarps = 8;   // one per child
+constexpr size_t kOctSmemMost = 200 * 1024;
 
 __host__ __device__ constexpr int oct_pitch(int nd) { return nd | 1; }
 
@@ -426,7 +448,7 @@ cd_status launch_leaf(const LeafLaunch &a, cudaStream_t s)
         auto kern = nd == 48 ? leaf_tma<48> : nd == 12 ? leaf_tma<12> : leaf_tma<0>;
         LeafTmaArgs P;
         P.a = a;
-        P.G = std::max(1, 384 / (2 * nd));
+        P.G = leaf_tma_groups(nd);
         // small trees: smaller batches, so that every SM gets one (16^3, 48 directions,
         // the whole evaluation as a graph 16.4 -> 14.4 us, 12 directions the same)
         while (P.G > 1 && P.G * nd >= 96 && a.n_oct < (int64_t)4 * P.G * sm_count()) {
@@ -439,10 +461,9 @@ cd_status launch_leaf(const LeafLaunch &a, cudaStream_t s)
         P.c_exp2 = (float)(-(double)a.shield_k * (double)a.av_per_nh * 1.4426950408889634);
         P.inv_nd = inv_nd;
         const int threads = P.G * 2 * nd;
-        const size_t smem = 128 + sizeof(float) * ((size_t)kLoadStages * (P.B * (nd + 8) + (size_t)P.prows * nd) + 3 * P.B * 8 +
-                                                   (size_t)2 * P.B * 8 * part_pitch(nd) +
-                                                   (a.n_h ? (size_t)2 * P.B * 8 * nd : 0));
-        if (smem > 48 * 1024) CD_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        const size_t smem = leaf_tma_smem(nd, P.G, a.n_h != nullptr);
+        constexpr size_t most = leaf_tma_smem_most();
+        CD_ALLOW_SMEM(kern, smem, most);
         int per_sm = 1;
         if (P.nbatch > sm_count()) CD_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem));
         if (per_sm < 1) per_sm = 1;
@@ -456,10 +477,10 @@ cd_status launch_leaf(const LeafLaunch &a, cudaStream_t s)
     // hardly any directions leave a warp too little to do per tile: up to 4 at any
     // size (256^3 at 3 directions 0.39 against 0.26 ms), up to 8 on trees below 32^3
     // (16^3 at 6: 12.3 against 10.4 us)
-    if (nd >= (a.n_oct >= 4096 ? 5 : 9) && leaf_oct_smem(nd, rows) <= 200 * 1024 && aligned16(a.rho_leaf)) {
+    if (nd >= (a.n_oct >= 4096 ? 5 : 9) && leaf_oct_smem(nd, rows) <= kOctSmemMost && aligned16(a.rho_leaf)) {
         const auto kern = rows ? leaf_oct_fp32<true> : leaf_oct_fp32<false>;
         const size_t smem = leaf_oct_smem(nd, rows);
-        CD_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        CD_ALLOW_SMEM(kern, smem, kOctSmemMost);
         int per_sm = 0;
         CD_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 32 * kOctWarps, smem));
         const int64_t grid = std::min<int64_t>((a.n_oct + 31) / 32, (int64_t)sm_count() * std::max(1, per_sm));
@@ -469,9 +490,7 @@ cd_status launch_leaf(const LeafLaunch &a, cudaStream_t s)
         return CD_OK;
     }
     const size_t smem = sizeof(float) * 64 * nd;
-    if (smem > 48 * 1024) {
-        CD_CUDA(cudaFuncSetAttribute(leaf_generic, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    }
+    CD_ALLOW_SMEM(leaf_generic, smem, sizeof(float) * 64 * CD_MAXDIR);
     int64_t blocks = (a.n_oct * 8 + 255) / 256;
     blocks = std::min<int64_t>(blocks, (int64_t)sm_count() * 8);
     LaunchScope ls(CD_K_LEAF, s);

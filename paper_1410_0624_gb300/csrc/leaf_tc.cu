@@ -76,9 +76,9 @@ struct LeafTcSmem {
     size_t bloc, bar, grp, grp_stride, aloc, out, stage, stage_bytes, st_e, st_p, st_r, st_l, total;
 };
 
-__host__ __device__ inline LeafTcSmem leaf_tc_smem(int nd, int NP, int G, bool list)
+__host__ __device__ constexpr LeafTcSmem leaf_tc_smem(int nd, int NP, int G, bool list)
 {
-    LeafTcSmem S;
+    LeafTcSmem S = {};
     size_t o = 0;
     auto take = [&](size_t bytes) { const size_t r = o; o = align128(o + bytes); return r; };
     S.bloc = take((size_t)NP * kK * 2);
@@ -95,6 +95,24 @@ __host__ __device__ inline LeafTcSmem leaf_tc_smem(int nd, int NP, int G, bool l
     S.grp_stride = S.stage + 2 * S.stage_bytes;
     S.total = S.grp + (size_t)G * S.grp_stride;
     return S;
+}
+
+// groups that fit smax bytes, at most four
+constexpr int leaf_tc_groups(int nd, bool list, size_t smax)
+{
+    int G = 4;
+    while (G > 1 && leaf_tc_smem(nd, round16(nd), G, list).total > smax) --G;
+    return G;
+}
+
+constexpr size_t leaf_tc_smem_most(bool list)
+{
+    size_t most = 0;
+    for (int nd = 4; nd <= 64; nd += 4) {
+        const size_t v = leaf_tc_smem(nd, round16(nd), leaf_tc_groups(nd, list, kSmemOptin), list).total;
+        most = v > most ? v : most;
+    }
+    return most;
 }
 
 __device__ __forceinline__ float fast_exp2(float x)
@@ -887,7 +905,7 @@ cd_status launch_leaf_oct(const LeafOctArgs &P, cudaStream_t s)
     if constexpr (S::kParts == 1)
         if (rows) kern = leaf_oct_tc<ND, true>;
     const size_t smem = S::smem(G, rows);
-    CD_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::smem(S::kGroups, rows)));
+    CD_ALLOW_SMEM(kern, smem, S::smem(S::kGroups, rows));
     const int64_t grid = std::min<int64_t>((P.ntiles + G - 1) / G, sms());
     LaunchScope ls(CD_K_LEAF, s, 2.0 * (double)P.ntiles * 128.0 * 16 * S::N);
     kern<<<(unsigned)grid, 128 * G, smem, s>>>(P);
@@ -957,12 +975,12 @@ cd_status launch_leaf_tc(const LeafLaunch &a, cudaStream_t s)
     int dev = 0, smax = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&smax, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-    P.G = 4;
-    while (P.G > 1 && (int)leaf_tc_smem(nd, P.NP, P.G, list).total > smax) --P.G;
+    P.G = leaf_tc_groups(nd, list, smax);
     const size_t smem = leaf_tc_smem(nd, P.NP, P.G, list).total;
     if ((int)smem > smax) return CD_EUNSUPPORTED;
     const auto kern = list ? leaf_tc<1> : leaf_tc<0>;
-    CD_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    constexpr size_t most[2] = {leaf_tc_smem_most(false), leaf_tc_smem_most(true)};
+    CD_ALLOW_SMEM(kern, smem, most[list]);
     const int64_t grid = std::min<int64_t>((P.ntiles + P.G - 1) / P.G, sms());
     LaunchScope ls(CD_K_LEAF, s, 2.0 * (double)P.ntiles * 128.0 * kK * P.NP);
     kern<<<(unsigned)grid, 128 * P.G, smem, s>>>(P, LeafBatch{});
@@ -1016,8 +1034,7 @@ cd_status launch_leaf_tc_batch(const void *jobs, const int2 *tile_ref, int64_t t
     int dev = 0, smax = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&smax, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-    P.G = 4;
-    while (P.G > 1 && (int)leaf_tc_smem(nd, P.NP, P.G, true).total > smax) --P.G;
+    P.G = leaf_tc_groups(nd, true, smax);
     const size_t smem = leaf_tc_smem(nd, P.NP, P.G, true).total;   // the kernel's layout (mode 2) has the list rows
     if ((int)smem > smax) {
         set_error("the batched leaf kernel needs %zu bytes of shared memory", smem);
@@ -1027,7 +1044,8 @@ cd_status launch_leaf_tc_batch(const void *jobs, const int2 *tile_ref, int64_t t
     Bt.jobs = static_cast<const LeafTcArgs *>(jobs);
     Bt.tile_ref = tile_ref;
     Bt.total = total;
-    CD_CUDA(cudaFuncSetAttribute(leaf_tc<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    constexpr size_t most = leaf_tc_smem_most(true);
+    CD_ALLOW_SMEM(leaf_tc<2>, smem, most);
     const int64_t grid = std::min<int64_t>((total + P.G - 1) / P.G, sms());
     LaunchScope ls(CD_K_LEAF, s, flops);
     leaf_tc<2><<<(unsigned)grid, 128 * P.G, smem, s>>>(P, Bt);

@@ -173,7 +173,8 @@ struct __align__(16) MarchStep {
     float t;                  // exit distance (len is the difference of two)
 };
 
-size_t march_smem(int L) { return ((size_t)3 << L) * (sizeof(MarchStep) + sizeof(uint16_t)); }
+constexpr int kMarchMaxLevel = 10;         // of a uniform tree
+constexpr size_t march_smem(int L) { return ((size_t)3 << L) * (sizeof(MarchStep) + sizeof(uint16_t)); }
 
 // Exact column from the leaf centre to the box edge: Amanatides-Woo DDA over
 // the leaf grid in cell units.
@@ -496,6 +497,8 @@ cd_status launch_march(cd_tree t, cd_geom g, int64_t n, const int64_t *leaves, f
     A.rho_leaf = t->rho_leaf;
     A.dirs = g->dirs_dev;
     A.out = n_ray;
+    const size_t smem = march_smem(A.L);
+    CD_ALLOW_SMEM(raymarch, smem, march_smem(kMarchMaxLevel));
     // rows listed in any order are marched in spatial order.  The order lives in
     // stream-ordered scratch; without it (a capture, no memory, more rows than
     // 32-bit places) the rows are taken as they come
@@ -531,8 +534,6 @@ cd_status launch_march(cd_tree t, cd_geom g, int64_t n, const int64_t *leaves, f
     A.rows_per_thread = (int)std::max<int64_t>(1, std::min<int64_t>(4, n * A.nd / (kThreads * 152 * 8)));
     const int64_t chunk = (int64_t)kThreads * A.rows_per_thread;
     A.items = (n + chunk - 1) / chunk * A.nd;
-    const size_t smem = march_smem(A.L);
-    cudaFuncSetAttribute(raymarch, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     {
         LaunchScope ls(CD_K_RAYMARCH, s);
         raymarch<<<(unsigned)std::min<int64_t>(A.items, 1 << 20), kThreads, smem, s>>>(A);

@@ -269,10 +269,10 @@ cd_status launch_gemm(const Gemm &g, cudaStream_t s)
 {
     const int64_t tiles = (int64_t)((g.M + BM - 1) / BM) * ((g.N + BN - 1) / BN);
     constexpr int smem = sizeof(TileSmem<BM, BN>);
-    if (smem > 48 * 1024)
-        CD_CUDA(cudaFuncSetAttribute(sgemm<BM, BN, TM, TN, FA, FB, EPI, KS>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    const auto kern = sgemm<BM, BN, TM, TN, FA, FB, EPI, KS>;
+    CD_ALLOW_SMEM(kern, smem, smem);
     LaunchScope ls(CD_K_NET, s);
-    sgemm<BM, BN, TM, TN, FA, FB, EPI, KS><<<(unsigned)tiles, KS * (BM / TM) * (BN / TN), smem, s>>>(g);
+    kern<<<(unsigned)tiles, KS * (BM / TM) * (BN / TN), smem, s>>>(g);
     CD_CHECK_LAUNCH();
     return CD_OK;
 }

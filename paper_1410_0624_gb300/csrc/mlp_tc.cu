@@ -1053,7 +1053,7 @@ cd_status column_density_learned_tc(cd_tree t, cd_geom g, const cd_opts &o, floa
         for (int k = 0; k <= CD_MAXL; ++k) A.C[k] = t->lv.C[k];
         A.h = ts->h;
         A.ext = ts->ext;
-        CD_CUDA(cudaFuncSetAttribute(learned_oct_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_oct));
+        CD_ALLOW_SMEM(learned_oct_tc, smem_oct, oct_smem(make_layout(kMaxNd)).total);
         const int grid = (int)std::min<int64_t>(A.ntiles, sms);
         LaunchScope ls(CD_K_NET, s);
         learned_oct_tc<<<grid, kOctThreads, smem_oct, s>>>(A);
@@ -1079,7 +1079,7 @@ cd_status column_density_learned_tc(cd_tree t, cd_geom g, const cd_opts &o, floa
         A.a_v = a_v;
         A.shield = shield;
         A.vec = (uintptr_t)n_h % 16 == 0;
-        CD_CUDA(cudaFuncSetAttribute(learned_cell_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_cell));
+        CD_ALLOW_SMEM(learned_cell_tc, smem_cell, cell_smem(make_layout(kMaxNd)).total);
         const int grid = (int)std::min<int64_t>(A.ntiles, sms);
         LaunchScope ls(CD_K_LEARNED, s);
         learned_cell_tc<<<grid, kCellThreads, smem_cell, s>>>(A);
