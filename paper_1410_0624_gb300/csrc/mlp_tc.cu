@@ -114,6 +114,8 @@ struct PackArgs {
     unsigned char *buf;
 };
 
+// An input with a negative scale is packed as its negative, together with its
+// weights: the same products, and the kernels may count on a >= 0 (std_input2).
 // W2 and W3 carry the half of GELU.  W3 and b3 are scaled by log2(e) so that the last chain gives delta log2(e)
 // and N = N_tree 2^(that).
 __global__ void pack_tc(PackArgs A)
@@ -129,14 +131,16 @@ __global__ void pack_tc(PackArgs A)
         int64_t i = e;
         if (i < n1c) {
             const int n = (int)(i / T.KC), k = (int)(i % T.KC);
-            const float v = k < nd ? W1[(int64_t)n * N.n_in + k] : (k == nd ? W1[(int64_t)n * N.n_in + kSlots * nd] : 0.f);
+            const int src = k < nd ? k : kSlots * nd;
+            const float w = k <= nd ? W1[(int64_t)n * N.n_in + src] : 0.f, v = A.sinv[src] < 0.f ? -w : w;
             reinterpret_cast<__nv_bfloat16 *>(A.buf + T.w1c + op_off(n, k, T.KC))[0] = __float2bfloat16_rn(v);
             continue;
         }
         i -= n1c;
         if (i < n1e) {
             const int n = (int)(i / T.KE), k = (int)(i % T.KE);
-            const float v = k < 7 * nd ? W1[(int64_t)n * N.n_in + nd + k] : 0.f;
+            const float w = k < 7 * nd ? W1[(int64_t)n * N.n_in + nd + k] : 0.f,
+                        v = k < 7 * nd && A.sinv[nd + k] < 0.f ? -w : w;
             reinterpret_cast<__nv_bfloat16 *>(A.buf + T.w1e + op_off(n, k, T.KE))[0] = __float2bfloat16_rn(v);
             continue;
         }
@@ -157,12 +161,12 @@ __global__ void pack_tc(PackArgs A)
         i -= n3;
         if (i < kH) { reinterpret_cast<float *>(A.buf + T.b1)[i] = A.p[N.b1 + i]; continue; }
         i -= kH;
-        // standardisation as u = a lg2(x) + b: a = ln(2) sinv, b = -mu sinv
+        // standardisation as u = a lg2(x) + b: a = ln(2) |sinv|, b = -mu |sinv|
         if (i < 2 * T.KC) {
             const int k = (int)(i % T.KC);
             const int src = k < nd ? k : (k == nd ? kSlots * nd : -1);
             const bool is_a = i < T.KC;
-            const float v = src < 0 ? 0.f : (is_a ? kLn2 * A.sinv[src] : -A.mu[src] * A.sinv[src]);
+            const float v = src < 0 ? 0.f : (is_a ? kLn2 * fabsf(A.sinv[src]) : -A.mu[src] * fabsf(A.sinv[src]));
             reinterpret_cast<float *>(A.buf + (is_a ? T.muc : T.sic))[k] = v;
             continue;
         }
@@ -170,7 +174,7 @@ __global__ void pack_tc(PackArgs A)
         {
             const int k = (int)(i % T.KE);
             const bool is_a = i < T.KE;
-            const float v = k < 7 * nd ? (is_a ? kLn2 * A.sinv[nd + k] : -A.mu[nd + k] * A.sinv[nd + k]) : 0.f;
+            const float v = k < 7 * nd ? (is_a ? kLn2 * fabsf(A.sinv[nd + k]) : -A.mu[nd + k] * fabsf(A.sinv[nd + k])) : 0.f;
             reinterpret_cast<float *>(A.buf + (is_a ? T.mue : T.sie))[k] = v;
         }
     }
@@ -217,8 +221,8 @@ __device__ __forceinline__ float std_input(float x, float floor_, float a, float
 
 // Two standardised, clipped inputs in BF16.  Rounding keeps order, so clipping
 // after it gives the same values; lo = max(a lg2(floor) + b, -clip) does for the
-// floor and the lower clip (a >= 0; an ignored input has a = b = 0, and its
-// 0 x inf falls back to lo = 0).
+// floor and the lower clip (a >= 0: pack_tc sees to it; an ignored input has
+// a = b = 0, and its 0 x inf falls back to lo = 0).
 __device__ __forceinline__ uint32_t std_input2(float2 x, float2 a, float2 b, uint32_t lo)
 {
     const float2 u = __ffma2_rn(a, make_float2(fast_log2(x.x), fast_log2(x.y)), b);

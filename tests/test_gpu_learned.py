@@ -512,6 +512,34 @@ def test_learned_refuses_a_network_of_other_directions_in_both_precisions(n_net,
     assert bool((n_h == -1.0).all())
 
 
+@pytest.mark.parametrize("precision", [colden.FP32, colden.BF16])
+@pytest.mark.parametrize("L,dset", [(4, ("healpix", 2, 0)), (5, ("mxn", 3, 8)), (8, ("mxn", 1, 8))])
+def test_learned_columns_with_negative_scales(L, dset, precision):
+    # u = clip((x - mu) sinv): an input's scale and its weights negated together are
+    # the same network, product by product, so the columns are the same bits; every
+    # kind of input among them (own oct, near and far slots, density, empty slots)
+    rho = torch.from_numpy(synth.lognormal_iid(1 << L, 10.0, 1.5, seed=3)).cuda()
+    tree, geom = colden.build_tree_uniform(rho, 10 * PC), colden.precompute_geometry(*dset)
+    nd, H = geom.n_dir, 128
+    n_in = 8 * nd + 1
+    net = colden.Net(nd, H, synth.mlp_init(nd, H, 8, out_scale=0.3))
+    x = torch.empty((4096, n_in), device="cuda")
+    colden.learned_features(tree, geom, x, leaves=torch.randint(tree.n_leaf, (4096,), device="cuda"))
+    net.fit_normaliser(x)
+    st = net.state()
+    out = []
+    for sign in (1.0, -1.0):
+        flip = np.where(np.arange(n_in) % 2 == 0, sign, 1.0).astype(np.float32)
+        p = st["params"].copy()
+        p[: H * n_in] = (p[: H * n_in].reshape(H, n_in) * flip).reshape(-1)
+        net.load_state(dict(st, params=p, sinv=st["sinv"] * flip))
+        n_h = torch.full((tree.n_leaf, nd), -1.0, device="cuda")
+        colden.column_density(tree, geom, n_h=n_h, net=net, precision=precision)
+        colden.device_status()
+        out.append(n_h)
+    assert torch.equal(out[0], out[1])
+
+
 # ---------------------------------------------------------------------------
 # What the trained network gains over the plain tree method
 # ---------------------------------------------------------------------------
