@@ -540,6 +540,28 @@ def test_learned_columns_with_negative_scales(L, dset, precision):
     assert torch.equal(out[0], out[1])
 
 
+@pytest.mark.parametrize("nd,H,B", [(48, 128, 300_001), (48, 512, 300_001), (12, 1024, 300_001), (1, 1024, 1_000_003)])
+def test_gradient_of_a_long_batch(nd, H, B):
+    # B times the same row: every sum over the batch adds equal terms, whose roundings
+    # do not cancel, and the gradient is that of the one row.  Chains of n1 rows, n2 of
+    # them, err by (n1 + n2) / 2 x 2^-24 at most; with n1 + n2 <= 2 B^(2/3) beside the 1e-4
+    # of the largest component that a gradient's terms are held to
+    p = synth.mlp_init(nd, H, 4)
+    n_in = 8 * nd + 1
+    net = colden.Net(nd, H, p)
+    rng = np.random.default_rng(5)
+    x, y = rng.standard_normal((1, n_in)).astype(np.float32), rng.uniform(0.5, 1.0, (1, nd)).astype(np.float32)
+    want, g = ol.loss_grad(ol.unpack(p.astype(np.float64), nd, H), np.zeros(n_in), np.ones(n_in), x.astype(np.float64),
+                           y.astype(np.float64))
+    g = ol.pack(g)
+    loss, grad = torch.zeros(1, device="cuda"), torch.empty(net.n_params, device="cuda")
+    rows = torch.zeros(B, dtype=torch.int64, device="cuda")
+    net.loss_grad(torch.from_numpy(x).cuda(), torch.from_numpy(y).cuda(), loss, grad, rows=rows)
+    tol = 1e-4 + B ** (2 / 3) * 2.0 ** -24
+    assert np.max(np.abs(grad.cpu().numpy() - g)) < tol * np.max(np.abs(g))
+    assert loss.item() == pytest.approx(want, rel=1e-5)
+
+
 # ---------------------------------------------------------------------------
 # What the trained network gains over the plain tree method
 # ---------------------------------------------------------------------------
