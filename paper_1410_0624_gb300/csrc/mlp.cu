@@ -637,7 +637,20 @@ static cd_status loss_grad(cd_net net, int64_t B, const float *x, const float *y
     // delta = W3 a2 + b3; d loss / d delta = 2 (delta - y) / (B nd) and the squared residuals
     const TileShape t = tile_shape(B, L.nd);
     const int n_sq = (int)tiles_of(B, L.nd, t.bm, t.bn);
-    if ((st = grow(&a.red, &a.red_cap, (size_t)n_sq)) != CD_OK) return st;
+    // dW1 = dz1^T u, dW2 = dz2^T a1, dW3 = G3^T a2, each with its bias gradient,
+    // split over the batch so that four CTAs reach every SM
+    constexpr int BM = 64, BN = 64;
+    const int64_t tiles = tiles_of(L.H, L.n_in, BM, BN) + tiles_of(L.H, L.H, BM, BN) + tiles_of(L.nd, L.H, BM, BN);
+    const int64_t slabs = (B + BK - 1) / BK,
+                  z_most = std::max<int64_t>(1, std::min<int64_t>(4 * 152 / tiles, kPartFloats / L.total));
+    int64_t z = std::min(slabs, z_most);
+    const int64_t per = (slabs + z - 1) / z;
+    z = (slabs + per - 1) / per;
+    // Scratch for any batch up to this one, with or without a gradient: neither the
+    // splits nor the tiles of a smaller batch need be fewer, and a call whose buffers
+    // exist can be captured
+    if ((st = grow(&a.red, &a.red_cap, (size_t)tiles_of(B, L.nd, 32, 32))) != CD_OK) return st;
+    if ((st = grow(&a.part, &a.part_cap, (size_t)(z_most * L.total))) != CD_OK) return st;
     g.N = L.nd; g.K = L.H; g.A = a.A2; g.lda = L.H; g.B = P + L.W3; g.ldb = L.H;
     g.C = a.D; g.ldc = L.nd; g.bias = P + L.b3; g.Y = y; g.sq = a.red;
     g.scale = (float)(2.0 / ((double)B * L.nd));
@@ -661,15 +674,6 @@ static cd_status loss_grad(cd_net net, int64_t B, const float *x, const float *y
     g.M = (int)B; g.N = L.H; g.K = L.H; g.A = a.G; g.lda = L.H; g.B = P + L.W2; g.ldb = L.H;
     g.C = a.Z1; g.ldc = L.H; g.Zin = a.Z1;
     if ((st = run_gemm<OP_N, OP_T, EPI_GELU_BWD>(g, s)) != CD_OK) return st;
-    // dW1 = dz1^T u, dW2 = dz2^T a1, dW3 = G3^T a2, each with its bias gradient,
-    // split over the batch so that four CTAs reach every SM
-    constexpr int BM = 64, BN = 64;
-    const int64_t tiles = tiles_of(L.H, L.n_in, BM, BN) + tiles_of(L.H, L.H, BM, BN) + tiles_of(L.nd, L.H, BM, BN);
-    const int64_t slabs = (B + BK - 1) / BK;
-    int64_t z = std::max<int64_t>(1, std::min<int64_t>({slabs, 4 * 152 / tiles, kPartFloats / L.total}));
-    const int64_t per = (slabs + z - 1) / z;
-    z = (slabs + per - 1) / per;
-    if ((st = grow(&a.part, &a.part_cap, (size_t)(z * L.total))) != CD_OK) return st;
     Grads G = {};
     const auto job = [&](int j, int M, int N, const float *A, const float *Bp, int64_t w, int64_t b) {
         Gemm &q = G.g[j];

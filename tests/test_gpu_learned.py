@@ -562,6 +562,32 @@ def test_gradient_of_a_long_batch(nd, H, B):
     assert loss.item() == pytest.approx(want, rel=1e-5)
 
 
+@pytest.mark.parametrize("nd,H,first,B,n", [(48, 128, "loss", 4096, 4096), (48, 128, "gradient", 8192, 480),
+                                            (48, 128, "step", 39_000, 9_700), (12, 40, "loss", 3000, 17)])
+def test_gradient_is_captured_after_an_eager_call_of_any_kind(nd, H, first, B, n):
+    # the first call at B rows, of the loss alone, the gradient or a step, allocates what
+    # a gradient of up to B rows takes: it can then be captured at any such size
+    net, _ = _net(nd, H)
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(7)
+    x = torch.randn(B, 8 * nd + 1, device="cuda", generator=gen)
+    y = torch.randn(B, nd, device="cuda", generator=gen)
+    loss, grad, want = (torch.zeros(k, device="cuda") for k in (1, net.n_params, net.n_params))
+    if first == "step":
+        net.train_step(x, y, loss=loss)
+    else:
+        net.loss_grad(x, y, loss, grad if first == "gradient" else None)
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=torch.cuda.Stream()):
+        net.loss_grad(x, y, loss, grad, batch=n, stream=torch.cuda.current_stream())
+    grad.fill_(-1.0)
+    g.replay()
+    torch.cuda.synchronize()
+    net.loss_grad(x, y, loss, want, batch=n)
+    assert torch.equal(grad, want)
+
+
 # ---------------------------------------------------------------------------
 # What the trained network gains over the plain tree method
 # ---------------------------------------------------------------------------
