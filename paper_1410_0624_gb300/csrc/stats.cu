@@ -72,8 +72,24 @@ int64_t free_generation() { return g_free_gen.load(); }
 static std::mutex g_scratch_mu;
 static cudaMemPool_t g_scratch[64];
 
+// While another thread (or this one, on another stream) captures in the global
+// mode, stream-ordered allocation counts as unsafe and ends that capture.  It is
+// not: the scratch is allocated and freed in the order of a stream that does not
+// capture (the caller's part), so this thread relaxes its mode meanwhile.
+class RelaxedCapture {
+  public:
+    RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode_); }
+    ~RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode_); }
+    RelaxedCapture(const RelaxedCapture &) = delete;
+    RelaxedCapture &operator=(const RelaxedCapture &) = delete;
+
+  private:
+    cudaStreamCaptureMode mode_ = cudaStreamCaptureModeRelaxed;
+};
+
 cudaError_t scratch_alloc(void **p, size_t bytes, cudaStream_t s)
 {
+    const RelaxedCapture relaxed;
     *p = nullptr;
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
@@ -104,7 +120,11 @@ cudaError_t scratch_alloc(void **p, size_t bytes, cudaStream_t s)
     return e;
 }
 
-void scratch_free(void *p, cudaStream_t s) { cudaFreeAsync(p, s); }
+void scratch_free(void *p, cudaStream_t s)
+{
+    const RelaxedCapture relaxed;
+    cudaFreeAsync(p, s);
+}
 
 void scratch_trim()
 {

@@ -102,3 +102,54 @@ def test_two_threads_launch_the_same_kernels_at_different_sizes(name):
     colden.device_status()
     for (out, _), w in zip(jobs, want):
         assert float(w.min()) > 0 and torch.equal(out, w)
+
+
+@pytest.mark.parametrize("name", ["raymarch_sorted", "raymarch", "small_tree", "tree"])
+def test_eager_calls_leave_another_threads_capture_alone(name):
+    # a thread captures in the global mode; calls of another one, on a stream of its own,
+    # work and do not end that capture
+    L = 4 if name == "small_tree" else 6
+    t, g = _tree(L, 5), colden.precompute_geometry("healpix", 2)
+    s = torch.cuda.Stream()
+    if name.startswith("raymarch"):
+        n = 100_000 if name == "raymarch_sorted" else 500
+        leaves = torch.from_numpy(np.random.default_rng(1).integers(0, t.n_leaf, n)).cuda()
+        out = torch.full((n, g.n_dir), -1.0, device="cuda")
+        call = lambda: colden.raymarch(t, g, out, leaves=leaves, stream=s)  # noqa: E731
+        colden.raymarch(t, g, torch.empty((8, g.n_dir), device="cuda"))     # the module is loaded
+    else:
+        out = torch.full((t.n_leaf, g.n_dir), -1.0, device="cuda")
+        call = lambda: colden.column_density(t, g, n_h=out, stream=s)  # noqa: E731
+        call()                                   # the tree's workspace exists
+    x, y = torch.ones(4, device="cuda"), torch.zeros(4, device="cuda")
+    torch.cuda.synchronize()
+    out.fill_(-1.0)
+    torch.cuda.synchronize()
+    capturing, called, errors = threading.Event(), threading.Event(), []
+
+    def capture():
+        graph = torch.cuda.CUDAGraph()
+        try:
+            with torch.cuda.graph(graph, stream=torch.cuda.Stream(), capture_error_mode="global"):
+                y.copy_(x)
+                capturing.set()
+                called.wait(60)
+                y.add_(x)
+            graph.replay()
+            torch.cuda.synchronize()
+        except Exception as e:  # noqa: BLE001
+            errors.append(e)
+        finally:
+            capturing.set()
+
+    th = threading.Thread(target=capture)
+    th.start()
+    capturing.wait(60)
+    try:
+        call()
+    finally:
+        called.set()
+        th.join()
+    torch.cuda.synchronize()
+    assert not errors, errors
+    assert float(out.min()) > 0 and bool((y == 2).all())
