@@ -743,7 +743,12 @@ __global__ void __launch_bounds__(128 * LeafOctShape<ND>::kGroups, 1) leaf_oct_t
     }
     *reinterpret_cast<uint4 *>(sA + op_off(i, 8, 16)) = make_uint4(0, 0, 0, 0);
     fence_proxy_async_smem();
-    if (warp == 0) tmem_alloc(&tslot, S::kCols * S::kGroups);
+    // the columns of the groups that there are (a power of two): on a small tree one or two,
+    // and CTAs of other calls can have the rest of the SM's (eight evaluations of 32^3
+    // at 32 directions on streams of their own, screening factor: 107 us with all
+    // groups' columns, 81 so; 64^3: 149 and 122)
+    const uint32_t cols = S::kCols * (G > 2 ? 4 : G);
+    if (warp == 0) tmem_alloc(&tslot, cols);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -879,7 +884,7 @@ __global__ void __launch_bounds__(128 * LeafOctShape<ND>::kGroups, 1) leaf_oct_t
     __syncthreads();
     if (warp == 0) {
         tc_fence_after();
-        tmem_dealloc(tslot, S::kCols * S::kGroups);
+        tmem_dealloc(tslot, cols);
     }
 }
 
