@@ -50,6 +50,35 @@ def test_raymarch_in_spatial_order_is_row_by_row_the_same(L, n, dset):
     assert np.max(np.abs(got - want) / want) < 2e-5   # the ray-marcher's tolerance
 
 
+@pytest.mark.parametrize("L,n,dset,kind", [(1, 2_100_001, ("axes", 0, 0), "random"), (2, 1_050_003, ("axes", 0, 0), "one"),
+                                           (3, 530_001, ("axes", 0, 0), "random"), (3, 530_001, ("axes", 0, 0), "one"),
+                                           (4, 270_001, ("axes", 0, 0), "random"), (4, 270_001, ("axes", 0, 0), "one"),
+                                           (4, 140_017, ("healpix", 1, 0), "few"), (4, 270_001, ("axes", 0, 0), "sorted"),
+                                           (5, 70_001, ("healpix", 1, 0), "runs"), (7, 40_003, ("mxn", 3, 4), "few")])
+def test_raymarch_of_repeated_leaves(L, n, dset, kind):
+    # long lists of the smallest trees that are marched as listed and of the smallest
+    # that are sorted (a bucket a leaf), with one leaf, a few, runs and sorted ones: rows
+    # of one leaf are the same bits, and those of the leaf marched in a short list
+    tree = colden.build_tree_uniform(torch.from_numpy(_rho(L, 7)).cuda(), BOX)
+    geom = colden.precompute_geometry(*dset)
+    rng = np.random.default_rng(n)
+    m = {"random": lambda: rng.integers(-1, tree.n_leaf + 1, n), "one": lambda: np.full(n, tree.n_leaf // 3),
+         "few": lambda: rng.choice([0, 1, tree.n_leaf // 2, tree.n_leaf - 1, -1], n),
+         "sorted": lambda: np.sort(rng.integers(0, tree.n_leaf, n)),
+         "runs": lambda: np.repeat(rng.integers(0, tree.n_leaf, n // 50 + 1), 50)[:n]}[kind]()
+    out = torch.full((n, geom.n_dir), -1.0, device="cuda")
+    colden.raymarch(tree, geom, out, leaves=torch.from_numpy(m).cuda())
+    leaf, back = np.unique(m, return_inverse=True)
+    one = torch.full((len(leaf), geom.n_dir), -1.0, device="cuda")
+    for i in range(0, len(leaf), 1000):
+        piece = torch.empty((len(leaf[i:i + 1000]), geom.n_dir), device="cuda")
+        colden.raymarch(tree, geom, piece, leaves=torch.from_numpy(leaf[i:i + 1000].copy()).cuda())
+        one[i:i + 1000] = piece
+    assert torch.equal(out, one[torch.from_numpy(back).cuda()])
+    bad = torch.from_numpy((leaf < 0) | (leaf >= tree.n_leaf)).cuda()
+    assert bool((one[bad] == 0).all()) and bool((one[~bad] > 0).all())
+
+
 @pytest.mark.parametrize("nd,H,B", [(5, 16, 33), (3, 97, 130), (12, 64, 4931), (48, 128, 9729), (7, 50, 38913),
                                     (13, 61, 38912), (12, 100, 39001)])
 def test_network_at_the_edges_of_its_gemm_tiles(nd, H, B):
