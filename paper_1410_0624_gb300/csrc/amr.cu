@@ -916,6 +916,7 @@ cd_status column_density_amr(cd_tree t, cd_geom g, const cd_opts &opts, float *n
             e.rho[3] = t->rho_lvl[k - 2];
             e.dx[3] = dx(k - 2);
             e.prefix_in = (k - 1 >= 3) ? t->ws.S[k - 1] : nullptr;
+            e.n_prefix = t->n_ref[k - 1];
             e.out = t->ws.S[k];
             e.list = list;
             const cd_status st = tc ? launch_ext_tc(e, t->rho_brick, g, s) : launch_ext_fp32(e, g, s);

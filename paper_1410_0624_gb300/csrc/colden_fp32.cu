@@ -421,7 +421,7 @@ cd_status launch_rows(const ExtLaunch &a, cd_geom g, cudaStream_t s)
         A.row_out = a.list->out;
         A.prefix_row = a.list->recv_parent;
         A.n_out = a.list->n_recv;
-        A.n_prefix = (int64_t)1 << (3 * (a.k - 1));
+        A.n_prefix = a.n_prefix;
         grid = a.list->ntiles / 2 * 4;
     } else {
         A.nG = (int64_t)1 << (3 * (a.k - 3));

@@ -412,6 +412,7 @@ struct ExtLaunch {
     const float *rho[4];      // dense level arrays of the shell level of each table
     float dx[4];              // dx of that shell level, cm
     const float *prefix_in;   // S_{k-1} (Morton) or NULL
+    int64_t n_prefix;         // with a list: the rows of prefix_in (bounds checks; a whole level has 8^(k-1))
     float *out;               // Morton [8^k][nd], or [n_recv][nd] with a list
     const TcList *list;       // receivers of an AMR level (NULL: every cell of level k)
     int tiles_per_cta;        // tensor-core form: 0 = persistent CTAs (two per SM); n = one CTA per n tiles

@@ -103,3 +103,42 @@ def test_checked_build_records_out_of_bounds_and_is_clean_and_identical_on_every
     for f in files:
         a, b = np.load(tmp_path / "plain" / f), np.load(tmp_path / "checked" / f)
         assert np.array_equal(a, b), f
+
+
+RUN_LISTS = r'''
+import json, os, sys
+import numpy as np, torch
+sys.path.insert(0, sys.argv[1])
+from paper_1410_0624_gb300 import colden, synth
+checked = os.environ.get("COLDEN_CHECKED") == "1"
+colden.load()
+fine = synth.lognormal_iid(128, 10.0, 0.5, seed=4)
+fine[:64, :64] *= 10.0
+lv = synth.amr_leaves(fine, 4, [60.0, 80.0, 100.0])
+t = colden.build_tree_amr(lv["base"], lv["lmax"], 10 * synth.PC_CM, lv["level"], lv["ijk"], lv["rho"])
+g = colden.precompute_geometry("mxn", 5, 3)
+nh = torch.empty(t.n_leaf * g.n_dir, device="cuda")
+colden.column_density(t, g, n_h=nh)
+torch.cuda.synchronize()
+np.save(sys.argv[2], nh.cpu().numpy())
+split = [int((lv["level"] > l).sum()) for l in (4, 5)]
+print(json.dumps({"status": colden.checked_status() if checked else (0, 0), "deeper": split}))
+'''
+
+
+def test_prefix_rows_of_lists_on_a_level_refined_in_part(tmp_path):
+    # lists of the row form whose parents' prefix has fewer rows than their level has
+    # cells, the extent the check is made against: clean, and bit-identical
+    _build.build(checked=True)
+    out = {}
+    for name in ("plain", "checked"):
+        env = dict(os.environ, COLDEN_CHECKED="1") if name == "checked" else dict(os.environ)
+        if name == "plain":
+            env.pop("COLDEN_CHECKED", None)
+        r = subprocess.run([sys.executable, "-c", RUN_LISTS, ROOT, str(tmp_path / (name + ".npy"))], env=env,
+                           capture_output=True, text=True, timeout=600)
+        assert r.returncode == 0, r.stderr[-3000:]
+        info = json.loads(r.stdout.strip().splitlines()[-1])
+        assert tuple(info["status"]) == (0, 0) and min(info["deeper"]) > 0
+        out[name] = np.load(tmp_path / (name + ".npy"))
+    assert np.all(out["plain"] > 0) and np.array_equal(out["plain"], out["checked"])
