@@ -554,21 +554,17 @@ static cd_status evaluate(cd_tree tree, cd_geom geom, const cd_opts *opts_in, fl
     // 0 in launches of kOctTilesPerCta tiles per CTA, while the far-shell prefix
     // chain (S_k needs S_{k-1}) runs on side stream 1, the high-priority one, so
     // its CTAs take SMs as the oct level's retire; the leaves wait for both.
-    // Up to 16^3 there is no chain, and for 32^3 it is one launch of 512 cells: the
-    // host is the slower side there, and ordering the side streams costs it more
-    // than they gain, unless the call is being captured or the rows are long
-    // (eager calls with and without: 16^3, 48 directions 24.8 and 23.1 us; 32^3,
-    // 12 directions 29.5 and 28.1, 48 directions 31.1 and 32.9)
-    bool alone = false;
-    if (L < 5 || (L == 5 && nd * geom->maxe <= 160)) {
-        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-        if (cudaStreamIsCapturing(s, &cap) == cudaSuccess) alone = cap == cudaStreamCaptureStatusNone;
-        else cudaGetLastError();   // a stream that cannot be asked: the fork says what is wrong with it
-    }
-    SideFork fork(tree, s, alone);
+    // Up to 32^3 everything stays on s.  Up to 16^3 there is no chain; for 32^3 it is one
+    // launch of 512 cells, in FP32 part of the octs' launch below, and the side streams
+    // cost the host more than they gain: calls one after another, 16^3, 12 directions
+    // 14.1 us, 16.9 with side streams; 32^3, 12 directions 16.4 (17.2; 19.6 in order in two
+    // launches), 48 directions 22.6 (22.7; 24.7), 84 directions 28.8 (28.7; 29.9).  In
+    // BF16 they would also leave the octs' 128 tiles to 16 CTAs: 12 directions 22.6
+    // (55.7), 48 directions 27.5 (71.4), captured 18.5 (53.5) and 24.6 (67.7).
+    SideFork fork(tree, s, L <= 5);
     if ((st = fork.status()) != CD_OK) return st;
     cudaStream_t s_oct = fork.side(0), s_chain = fork.side(1);
-    for (int k = 3; k <= L - 2; ++k) {
+    const auto far = [&](int k) {
         ExtLaunch a = {};
         a.k = k;
         a.nd = nd;
@@ -577,6 +573,11 @@ static cd_status evaluate(cd_tree tree, cd_geom geom, const cd_opts *opts_in, fl
         a.dx[3] = dx_of(tree, k - 2);
         a.prefix_in = (k > 3) ? tree->ws.S[k - 1] : nullptr;
         a.out = tree->ws.S[k];
+        return a;
+    };
+    const bool pair = L == 5 && !bf16;   // 32^3: the chain's one level and the octs in one launch
+    for (int k = 3; k <= L - 2 && !pair; ++k) {
+        const ExtLaunch a = far(k);
         st = use_tc(k) ? launch_ext_tc(a, tree->rho_brick, geom, s_chain) : launch_ext_fp32(a, geom, s_chain);
         if (st != CD_OK) return st;
     }
@@ -593,7 +594,9 @@ static cd_status evaluate(cd_tree tree, cd_geom geom, const cd_opts *opts_in, fl
         a.prefix_in = nullptr;   // the leaf kernel adds S_{L-2}[parent]
         a.out = tree->ws.E;
         a.tiles_per_cta = fork.serial() ? 0 : kOctTilesPerCta;
-        st = use_tc(k) ? launch_ext_tc(a, tree->rho_brick, geom, s_oct) : launch_ext_fp32(a, geom, s_oct);
+        st = use_tc(k) ? launch_ext_tc(a, tree->rho_brick, geom, s_oct)
+             : pair    ? launch_ext_fp32_pair(a, far(3), geom, s_oct)
+                       : launch_ext_fp32(a, geom, s_oct);
         if (st != CD_OK) return st;
     }
     if ((st = fork.join()) != CD_OK) return st;

@@ -418,6 +418,8 @@ struct ExtLaunch {
     int tiles_per_cta;        // tensor-core form: 0 = persistent CTAs (two per SM); n = one CTA per n tiles
 };
 cd_status launch_ext_fp32(const ExtLaunch &a, cd_geom g, cudaStream_t s);
+// two launches that do not depend on one another, as one where the block form serves both
+cd_status launch_ext_fp32_pair(const ExtLaunch &a, const ExtLaunch &b, cd_geom g, cudaStream_t s);
 // whether launch_ext_fp32 takes the row form for these receivers of level k (a
 // list, or NULL for the whole level) with these tables; lists have no other form
 // there: the caller goes to its own kernel

@@ -131,6 +131,31 @@ def test_fp32_shell_rows_match_oracle(L, dset, mode):
     assert np.max(np.abs(got - want) / want) <= 1e-5
 
 
+@pytest.mark.parametrize("dset,mode", [(("custom", 0, 0, [[0.3, -0.5, 0.8]]), 0), (("axes", 0, 0), 0), (("healpix", 1, 0), 0),
+                                       (("mxn", 7, 3), 0), (("healpix", 2, 0), 0), (("mxn", 5, 8), 2), (("mxn", 16, 17), 0)])
+@pytest.mark.parametrize("L", [3, 4, 5, 6])
+def test_fp32_small_trees_match_their_launches_one_by_one(L, dset, mode):
+    # 32^3 sums the octs' shells and the far ones in one launch; the form with fixed
+    # scratch launches every level by itself: the same kernels, bit for bit, also captured
+    tree = colden.build_tree_uniform(torch.from_numpy(_rho(L, 50 + L)).cuda(), BOX)
+    geom = colden.precompute_geometry(*dset, mode=mode)
+    new = lambda: (torch.full((tree.n_leaf, geom.n_dir), -1.0, device="cuda"),  # noqa: E731
+                   torch.full((tree.n_leaf,), -1.0, device="cuda"))
+    a, b, c = new(), new(), new()
+    colden.column_density(tree, geom, n_h=a[0], shield=a[1])
+    try:
+        colden.column_density_noalloc(tree, geom, n_h=b[0], shield=b[1])
+    except colden.ColdenError:
+        assert L == 6 and geom.n_dir > 40        # the fixed scratch is too small
+        b = a
+    colden.EvalGraph(tree, geom, n_h=c[0], shield=c[1]).launch()
+    torch.cuda.synchronize()
+    colden.device_status()
+    assert float(a[0].min()) > 0
+    for x, y, z in zip(a, b, c):
+        assert torch.equal(x, y) and torch.equal(x, z)
+
+
 @pytest.mark.parametrize("dset", [("mxn", 5, 3), ("axes", 0, 0), ("healpix", 2, 0)])
 def test_fp32_shell_rows_on_lists_match_uniform(dset):
     # a mesh refined in one corner: its finest leaves far inside the refined part
