@@ -18,6 +18,8 @@
 // {shared-memory offset, weight} pairs, so a warp's loads of one entry are
 // contiguous, and each (cfg) row is walked to the largest non-zero count of
 // its directions (padding entries have weight 0).
+#include <algorithm>
+
 #include "common.cuh"
 #include "umma.cuh"
 
@@ -132,6 +134,7 @@ __global__ void __launch_bounds__(kExtThreads) shell_sum_fp32(const __grid_const
 constexpr int kRowThreads = 512, kRowPitch = 36, kRowCells = CD_STENCIL, kRingQuads = 4;
 constexpr int kRowMinEntries = 48;       // directions x longest row
 constexpr int kRowMinReceivers = 1024;   // of a list
+constexpr int kRowShort = 24;            // entries of single rays (18), not of cones (39)
 
 struct RowArgs {
     int k, nd;
@@ -471,21 +474,36 @@ cd_status launch_block(const ExtLaunch *job, int n, cd_geom g, cudaStream_t s)
 
 }  // namespace
 
-bool ext_fp32_serves_list(int k, int tmask, cd_geom g, const TcList *list)
+// the row form has the lists of these tables and something to sum
+static bool rows_serve(int k, int tmask, cd_geom g)
 {
     // with hardly anything to sum (the six axis rays have three entries at most)
     // staging a parent's stencils costs more than the block form's gathers
     // (64^3: 24.6 against 23.1 us; 12 HEALPix directions 24.4 against 28.7)
     const int li = row_list(tmask);
-    if (k < 4 || li < 0 || g->rows[li].quad == nullptr || g->n_dir * g->maxe < kRowMinEntries) return false;
+    return k >= 4 && li >= 0 && g->rows[li].quad != nullptr && g->n_dir * g->maxe >= kRowMinEntries;
+}
+
+bool ext_fp32_serves_list(int k, int tmask, cd_geom g, const TcList *list, bool walk)
+{
+    if (!rows_serve(k, tmask, g)) return false;
     // A CTA reads its class's entries for 32 cells: too few receivers per class
     // leave it little to share them with.  The whole level of 16^3 has eight parents in
     // each of 64 classes (evaluations of 32^3 replayed as graphs, row against block
     // form: 12 directions 22.5 and 18.5 us, 84 directions 37.0 and 28.8, 40
-    // cone-averaged ones 48.3 and 35.4; at 64^3 48 directions take 43 and 64).  Lists
-    // have a slower alternative: 84 directions of a mesh of 16^3 with 288 octs one
-    // level up 65.7 and 55.4 us, of 32^3 with 2 230 66.1 and 78.0.
-    return list ? list->n_recv >= kRowMinReceivers : k > 4;
+    // cone-averaged ones 48.3 and 35.4; at 64^3 48 directions take 43 and 64).
+    if (!list) return k > 4;
+    // Lists have slower alternatives.  On 16^3, where a whole class has eight parents,
+    // the list kernel's gathers hit few lines: with the short rows of single rays it
+    // keeps lists of up to about 131 072 / directions receivers.  Graphs of meshes of 16^3
+    // with refined cells, row against list form: 1 050 cells 20 directions 24.6 and
+    // 22.7 us, 32 26.8 and 24.6, 84 41.2 and 39.0, but 12 directions 24.6 and 24.7, 192 57
+    // and 65, 12 cone-averaged ones 68 and 88; 1 600 cells 32 directions 28.7 and 26.7,
+    // 84 41.1 and 41.1; 2 600 cells 48 directions 32.8 and 34.9.  On 32^3 1 050 cells
+    // take 48 directions 34.9 and 45.1 us.  In-situ columns would walk instead.
+    const bool coarse = k == 4 && !walk && g->maxe <= kRowShort && g->n_dir > 16;
+    const int64_t least = coarse ? std::min(2400, 131072 / g->n_dir) : 0;
+    return list->n_recv >= std::max<int64_t>(kRowMinReceivers, least);
 }
 
 cd_status build_row_lists(cd_geom g, cudaStream_t s)
@@ -519,7 +537,7 @@ cd_status build_row_lists(cd_geom g, cudaStream_t s)
 
 cd_status launch_ext_fp32(const ExtLaunch &a, cd_geom g, cudaStream_t s)
 {
-    if (ext_fp32_serves_list(a.k, a.tmask, g, a.list)) return launch_rows(a, g, s);
+    if (a.list ? rows_serve(a.k, a.tmask, g) : ext_fp32_serves_list(a.k, a.tmask, g, nullptr)) return launch_rows(a, g, s);
     if (a.list) {
         set_error("the FP32 block form serves whole levels only");
         return CD_EUNSUPPORTED;

@@ -420,10 +420,10 @@ struct ExtLaunch {
 cd_status launch_ext_fp32(const ExtLaunch &a, cd_geom g, cudaStream_t s);
 // two launches that do not depend on one another, as one where the block form serves both
 cd_status launch_ext_fp32_pair(const ExtLaunch &a, const ExtLaunch &b, cd_geom g, cudaStream_t s);
-// whether launch_ext_fp32 takes the row form for these receivers of level k (a
-// list, or NULL for the whole level) with these tables; lists have no other form
-// there: the caller goes to its own kernel
-bool ext_fp32_serves_list(int k, int tmask, cd_geom g, const TcList *list);
+// whether the row form is the one for these receivers of level k (a list, or NULL
+// for the whole level) with these tables; lists have no other form in
+// launch_ext_fp32: the caller goes to its own kernel (walk: the in-situ walks)
+bool ext_fp32_serves_list(int k, int tmask, cd_geom g, const TcList *list, bool walk = false);
 // the chunk lists of the tables (after build_geometry_tables)
 cd_status build_row_lists(cd_geom g, cudaStream_t s);
 

@@ -175,7 +175,7 @@ cd_status launch_insitu(cd_tree t, cd_geom g, int k, int64_t n, const uint64_t *
     if (n == 0) return CD_OK;
     InsituArgs A = {};
     A.top = k;
-    if (ext_fp32_serves_list(k, 7, g, keys ? list : nullptr) && (!keys || (list && list->ntiles))) {
+    if (ext_fp32_serves_list(k, 7, g, keys ? list : nullptr, true) && (!keys || (list && list->ntiles))) {
         ExtLaunch e = {};
         e.k = k;
         e.nd = g->n_dir;

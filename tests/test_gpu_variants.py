@@ -175,6 +175,29 @@ def test_fp32_shell_rows_on_lists_match_uniform(dset):
     assert np.max(np.abs(got - want) / want) <= 1e-5
 
 
+@pytest.mark.parametrize("count", [900, 1100, 1500, 1700, 2500])
+@pytest.mark.parametrize("dset,mode", [(("mxn", 4, 4), 0), (("mxn", 5, 4), 0), (("mxn", 7, 12), 0), (("mxn", 3, 4), 2),
+                                       (("mxn", 5, 4), 1)])
+def test_fp32_lists_of_16_cubed_on_both_sides_of_the_row_forms_lines(count, dset, mode):
+    # lists of 16^3 below and above the receivers from which the row form takes them, by
+    # directions and kind of ray, against the oracle's adaptive tree
+    fine = synth.lognormal_grf(32, 10.0, 1.5, seed=3)
+    mean = fine.reshape(16, 2, 16, 2, 16, 2).mean((1, 3, 5))
+    lv = synth.amr_leaves(fine, 4, [float(np.sort(mean.reshape(-1))[-count - 1])])
+    tree = colden.build_tree_amr(4, 5, BOX, lv["level"], lv["ijk"], lv["rho"])
+    geom = colden.precompute_geometry(*dset, mode=mode)
+    nh = torch.full((tree.n_leaf, geom.n_dir), -1.0, device="cuda")
+    colden.column_density(tree, geom, n_h=nh)
+    level, ijk = tree.leaves()
+    rng = np.random.default_rng(count)
+    rows = np.concatenate([rng.choice(np.flatnonzero(level == l), 100) for l in (4, 5)])
+    T = oracle.Tree.amr(4, 5, BOX, lv["level"], lv["ijk"], lv["rho"])
+    want = (T.column_density_cone(geom.dirs, level[rows], ijk[rows]) if mode == 2 else
+            T.column_density(geom.dirs, level[rows], ijk[rows], mode=oracle.MODE_INSITU if mode else oracle.MODE_PREC))
+    got = nh[torch.from_numpy(rows).cuda()].double().cpu().numpy()
+    assert np.max(np.abs(got - want) / want) <= 1e-5
+
+
 @pytest.mark.parametrize("dset", [("mxn", 1, 4), ("mxn", 2, 4), ("healpix", 1, 0), ("mxn", 4, 4), ("mxn", 5, 4),
                                   ("mxn", 4, 6), ("mxn", 4, 7), ("mxn", 8, 4), ("mxn", 9, 4), ("mxn", 5, 8),
                                   ("mxn", 11, 4), ("healpix", 2, 0), ("mxn", 13, 4), ("mxn", 7, 8), ("mxn", 15, 4),
