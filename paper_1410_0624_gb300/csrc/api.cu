@@ -558,9 +558,10 @@ static cd_status evaluate(cd_tree tree, cd_geom geom, const cd_opts *opts_in, fl
     // launch of 512 cells, in FP32 part of the octs' launch below, and the side streams
     // cost the host more than they gain: calls one after another, 16^3, 12 directions
     // 14.1 us, 16.9 with side streams; 32^3, 12 directions 16.4 (17.2; 19.6 in order in two
-    // launches), 48 directions 22.6 (22.7; 24.7), 84 directions 28.8 (28.7; 29.9).  In
-    // BF16 they would also leave the octs' 128 tiles to 16 CTAs: 12 directions 22.6
-    // (55.7), 48 directions 27.5 (71.4), captured 18.5 (53.5) and 24.6 (67.7).
+    // launches), 48 directions 20.5 (22.7; 24.7), 84 directions 24.7 (28.7; 29.9), 192
+    // directions 37.0 (41.0).  In BF16 they would also leave the octs' 128 tiles to 16
+    // CTAs: 12 directions 22.6 (55.7), 48 directions 27.5 (71.4), captured 18.5 (53.5)
+    // and 24.6 (67.7).
     SideFork fork(tree, s, L <= 5);
     if ((st = fork.status()) != CD_OK) return st;
     cudaStream_t s_oct = fork.side(0), s_chain = fork.side(1);
@@ -595,7 +596,7 @@ static cd_status evaluate(cd_tree tree, cd_geom geom, const cd_opts *opts_in, fl
         a.out = tree->ws.E;
         a.tiles_per_cta = fork.serial() ? 0 : kOctTilesPerCta;
         st = use_tc(k) ? launch_ext_tc(a, tree->rho_brick, geom, s_oct)
-             : pair    ? launch_ext_fp32_pair(a, far(3), geom, s_oct)
+             : pair    ? launch_ext_fp32_pair(far(3), a, geom, s_oct)
                        : launch_ext_fp32(a, geom, s_oct);
         if (st != CD_OK) return st;
     }
