@@ -561,8 +561,15 @@ static cd_status evaluate(cd_tree tree, cd_geom geom, const cd_opts *opts_in, fl
     // launches), 48 directions 20.5 (22.7; 24.7), 84 directions 24.7 (28.7; 29.9), 192
     // directions 37.0 (41.0).  In BF16 they would also leave the octs' 128 tiles to 16
     // CTAs: 12 directions 22.6 (55.7), 48 directions 27.5 (71.4), captured 18.5 (53.5)
-    // and 24.6 (67.7).
-    SideFork fork(tree, s, L <= 5);
+    // and 24.6 (67.7).  Other captures keep the fork, which costs a replay nothing (8^3,
+    // 6 directions 10.2 us, 10.9 without).
+    bool alone = false;
+    if (L <= 5) {
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) cudaGetLastError();   // the fork says what is wrong with s
+        else alone = cap == cudaStreamCaptureStatusNone || (L == 5 && bf16);
+    }
+    SideFork fork(tree, s, alone);
     if ((st = fork.status()) != CD_OK) return st;
     cudaStream_t s_oct = fork.side(0), s_chain = fork.side(1);
     const auto far = [&](int k) {
