@@ -150,7 +150,7 @@ __global__ void __launch_bounds__(kExtThreads) shell_pair_fp32(const __grid_cons
 constexpr int kRowThreads = 512, kRowPitch = 36, kRowCells = CD_STENCIL, kRingQuads = 4;
 constexpr int kRowMinEntries = 48;       // directions x longest row
 constexpr int kRowMinReceivers = 1024;   // of a list
-constexpr int kRowShort = 24;            // entries of single rays (18), not of cones (39)
+constexpr int kRowShort = 24;            // longest row of a table: single rays have about ten entries, cones over thirty
 
 struct RowArgs {
     int k, nd;
@@ -528,7 +528,7 @@ cd_status build_row_lists(cd_geom g, cudaStream_t s)
         if (cudaMalloc(&L.quad, quads * sizeof(RowQuad)) != cudaSuccess ||
             cudaMalloc(&L.start, sizeof(int) * ncfg * (nq + 1)) != cudaSuccess) {
             cudaGetLastError();           // no room: the other forms serve these tables
-            if (L.quad) cd::lib_free(L.quad);
+            if (L.quad) cudaFree(L.quad);   // no evaluation has seen it: captured graphs stay valid
             L.quad = nullptr;
             L.start = nullptr;
             continue;

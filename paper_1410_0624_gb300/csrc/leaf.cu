@@ -477,9 +477,10 @@ cd_status launch_leaf(const LeafLaunch &a, cudaStream_t s)
     // hardly any directions leave a warp too little to do per tile: up to 4 at any
     // size (256^3 at 3 directions 0.39 against 0.26 ms), 5 where N_H or A_V is written (128^3
     // 41 against 35 us; both 60 against 61, the screening factor alone 23 against 25; 6
-    // directions with N_H 43 against 47).  Below 32^3 a tile is a CTA's only one: rows of up to 8 directions
-    // (16^3 at 6: 12.3 against 10.4 us) and the screening factor alone of up to 31 (8^3 at
-    // 10: 6.6 against 6.2 us, 15: 7.6 against 6.9, 16^3 at 27: 8.8 against 8.2)
+    // directions with N_H 43 against 47).  Below 32^3 a tile is a CTA's only one: rows
+    // of up to 8 directions (16^3 at 6: 12.3 against 10.4 us) and the screening factor
+    // alone of up to 31 (8^3 at 10: 6.6 against 6.2 us, 15: 7.6 against 6.9, 16^3 at 27:
+    // 8.8 against 8.2)
     const bool tiny = a.n_oct < 4096;
     const bool one = (a.n_h != nullptr) != (a.a_v != nullptr);
     const int least = tiny ? (rows ? 9 : 32) : one ? 6 : 5;
